@@ -108,6 +108,16 @@ struct grx_graph {
     float *pr_s;                     // cross-tile partial sums
     int32_t *pr_fix;                 // per-tile row needing a fix-up
     int64_t pr_fix_len;
+    // PageRank rows sorted by degree (allocated by the first call that pays for
+    // them): relabelled columns in int4 units, header, and per sorted row the
+    // vertex, degree and first int4; chunk -> row, chunk sums, chunks done
+    void *prs_cols, *prs_hdr;
+    int32_t *prs_vert, *prs_chunk_row;
+    uint32_t *prs_deg, *prs_unit;
+    float *prs_part;
+    unsigned int *prs_done;
+    int prs_chunk_shift;
+    int64_t pr_csr_iters;            // iterations run in CSR order so far
     // PageRank column blocks (segments of rows per block of 2^prb_shift columns)
     int pr_shift_req;                // requested block width (0 = automatic, < 0 = never)
     int prb_K, prb_shift;            // built blocks (prb_K < 2: none)
@@ -199,6 +209,10 @@ grx_status grx_bcm_launch(grx_graph *g, const int32_t *srcs, int n, double *bc_o
                           cudaStream_t s);
 grx_status grx_pr_launch(grx_graph *g, float damping, int iters, float *rank,
                          cudaStream_t s);
+// PageRank over degree-sorted rows (pr_rows.cu).
+grx_status grx_prs_build(grx_graph *g, cudaStream_t s, int *ready);
+void grx_prs_init(grx_graph *g, float r0, float *c0, float *c1, cudaStream_t s);
+void grx_prs_iterate(grx_graph *g, const float *c_in, float *c_out, float *rank, float base, float d, cudaStream_t s);
 
 // ---------------------------------------------------------------------------
 // Device helpers

@@ -8,6 +8,10 @@
 // isolated vertex holds the same rank; D_i = n_isolated * r_i[isolated] and
 // base_i follow from a scalar recurrence the host evaluates in double.
 //
+// Graphs that are ranked for more than a few iterations get their rows sorted by
+// degree first (pr_rows.cu); what follows here is the CSR-order form for the
+// others, and for when there is no memory for the sorted copy.
+//
 // One launch per iteration over equal tiles of the edge array (the active
 // list of non-isolated vertices has the CSR offsets as its edge prefix, so a
 // tile holds at most TILE+1 rows; the first row and row count of every tile
@@ -26,6 +30,13 @@ namespace {
 constexpr int PR_BLOCK = 256;
 constexpr int PR_ITEMS = 9;                  // odd: conflict-free strided smem reads
 constexpr int PR_TILE = PR_BLOCK * PR_ITEMS;
+
+// Iterations a graph must be worth before its rows are sorted (pr_rows.cu);
+// those it ran in CSR order count.  On GB300 the sort takes 1.1 ms at R-MAT 22
+// and 18 ms at R-MAT 26, and every iteration after it is 0.39 and 10.9 ms
+// shorter: it is paid for by the fourth.  Below 16M edges it takes 0.2 ms,
+// mostly launches and allocation, against 0.02-0.04 ms an iteration.
+inline int64_t prs_min_iters(int64_t ne) { return ne >= (16ll << 20) ? 4 : 12; }
 
 struct PrSmem {
     union alignas(16) {
@@ -492,8 +503,8 @@ grx_status prb_build(grx_graph *g, int shift, cudaStream_t s) {
 grx_status grx_pr_launch(grx_graph *g, float damping, int iters, float *rank, cudaStream_t s) {
     const int64_t ntiles = (g->ne + PR_TILE - 1) / PR_TILE;
     if (!g->pr_c[0]) {
-        g->pr_c[0] = (float *)grx_alloc(g, (size_t)g->nv * 4, s);
-        g->pr_c[1] = (float *)grx_alloc(g, (size_t)g->nv * 4, s);
+        g->pr_c[0] = (float *)grx_alloc(g, (size_t)g->nv * 4 + 16, s);   // + the padding's entry
+        g->pr_c[1] = (float *)grx_alloc(g, (size_t)g->nv * 4 + 16, s);
         g->pr_s = (float *)grx_alloc(g, (size_t)g->nv * 4, s);
         g->pr_fix = (int32_t *)grx_alloc(g, (size_t)(ntiles > 0 ? ntiles : 1) * 4, s);
         if (!g->pr_c[0] || !g->pr_c[1] || !g->pr_s || !g->pr_fix)
@@ -531,6 +542,21 @@ grx_status grx_pr_launch(grx_graph *g, float damping, int iters, float *rank, cu
         base[(size_t)i] = (float)b;
         riso = b;
     }
+    if (!blocked && ntiles > 0 && (g->prs_cols || g->pr_csr_iters + iters >= prs_min_iters(g->ne))) {
+        int ready = 0;
+        grx_status st = grx_prs_build(g, s, &ready);
+        if (st != GRX_OK) return st;
+        if (ready) {
+            grx_prs_init(g, (float)(1.0 / N), g->pr_c[0], g->pr_c[1], s);
+            for (int i = 0; i < iters; ++i)
+                grx_prs_iterate(g, g->pr_c[i & 1], g->pr_c[(i + 1) & 1], i == iters - 1 ? rank : nullptr,
+                                base[(size_t)i], damping, s);
+            k_pr_fill<<<fill_blocks, 256, 0, s>>>(g->nz_bits, g->nv, (float)riso, 0, rank);
+            GRX_CUDA(cudaGetLastError());
+            return GRX_OK;
+        }
+    }
+    g->pr_csr_iters += iters;
     const int init_blocks = (int)((g->n_active + 255) / 256 < 8192 ? (g->n_active + 255) / 256 : 8192);
     if (g->n_active > 0)
         k_pr_init<<<init_blocks > 0 ? init_blocks : 1, 256, 0, s>>>(g->active, g->aoff, g->n_active,
