@@ -48,6 +48,7 @@
 #include <cstring>
 
 #include "grx_internal.cuh"
+#include "narrow.cuh"
 
 namespace {
 
@@ -79,6 +80,8 @@ static_assert(WTILE == 256 && PULL_HSTEP == 256, "warp_tile_rows8 covers 256-pos
 enum { DIR_PUSH = 0, DIR_PULL = 1 };
 enum { OP_QPUSH, OP_BMARK, OP_BFINAL, OP_COMPACT, OP_PULL, OP_PULL_LIST };
 
+enum { NARROW_ON = 1, NARROW_OFF = 2 };
+
 struct LevelState {
     int L;              // level being expanded (frontier = vertices at depth L)
     uint8_t dir;
@@ -96,10 +99,13 @@ struct LevelState {
     uint8_t uin;        // U_L (candidates left unfound by a pull level L-1) exists
     uint8_t lmode;      // pull over the list U_L instead of a sweep of all chunks
     uint8_t uwrite;     // this pull level writes U_{L+1}
+    uint8_t narrow;     // NARROW_ON: the narrow group goes on (the other blocks wait again);
+                        // NARROW_OFF: the whole grid runs this level, whatever its size
     uint32_t seq;       // phases run so far in this traversal (chunk-counter ring index)
     uint32_t ucnt;      // |U_L|
     uint32_t q, T;      // |Q_L| and its edge count
     uint32_t nprev;     // |Q_{L-1}|
+    uint32_t calm;      // push levels in a row that were small enough to be narrow
     unsigned long long vcount;   // visited vertices including Q_L
 };
 
@@ -130,6 +136,8 @@ struct BfsArgs {
     uint32_t ulist_max;           // a pull level works on U_L when |U_L| <= ulist_max
     unsigned long long timeout_ns;
     int32_t src;
+    NarrowBuffers *narrow;        // NULL: no narrow levels
+    uint32_t narrow_levels;       // narrow levels between two grid barriers
 };
 
 template <typename OffT>
@@ -210,19 +218,16 @@ __device__ LevelState initial_state(const BfsArgs<OffT> &a) {
     return s;
 }
 
-// State of the next phase: the same level's next phase, or level L+1 from the
-// counters level L left.
+// State of level L+1 from what level L left: pk = (|Q_{L+1}| << 32 | its edges),
+// ucnt = |U_{L+1}|.
 template <typename OffT>
-__device__ LevelState next_state(const BfsArgs<OffT> &a, const LevelState &st, bool stats) {
+__device__ LevelState next_level(const BfsArgs<OffT> &a, const LevelState &st, unsigned long long pk, uint32_t ucnt,
+                                 bool stats) {
     LevelState ns = st;
     ns.seq = st.seq + 1;
-    if ((int)st.phase + 1 < level_phases(st)) {
-        ns.phase = st.phase + 1;
-        return ns;
-    }
     ns.L = st.L + 1;
     ns.phase = 0;
-    const unsigned long long pk = ld_relaxed_u64(&a.ctl->qpack[(st.L + 1) & 3]);
+    ns.narrow = 0;
     ns.q = (uint32_t)(pk >> 32);
     ns.T = (uint32_t)pk;
     ns.nprev = st.q;
@@ -232,8 +237,9 @@ __device__ LevelState next_state(const BfsArgs<OffT> &a, const LevelState &st, b
     ns.qprev_ok = st.qin || st.compact;
     ns.qin = st.dir == DIR_PUSH || st.lmode;     // a list pull appends what it finds
     ns.uin = st.uwrite;
-    ns.ucnt = st.uwrite ? ld_relaxed_u32(&a.ctl->ucount[(st.L + 1) & 3]) : 0u;
+    ns.ucnt = ucnt;
     if (stats && blockIdx.x == 0 && st.L < GRX_MAX_LEVELS_STATS) a.stats->discovered[st.L] = ns.q;
+    ns.calm = st.dir == DIR_PUSH && st.T <= narrow_max_T() / 2 ? st.calm + 1 : 0u;
     if (ns.q == 0) {
         ns.done = 1;
         return ns;
@@ -257,6 +263,20 @@ __device__ LevelState next_state(const BfsArgs<OffT> &a, const LevelState &st, b
     }
     set_kind(a, ns);
     return ns;
+}
+
+// State of the next phase: the same level's next phase, or level L+1 from the
+// counters level L left.
+template <typename OffT>
+__device__ LevelState next_state(const BfsArgs<OffT> &a, const LevelState &st, bool stats) {
+    if ((int)st.phase + 1 < level_phases(st)) {
+        LevelState ns = st;
+        ns.seq = st.seq + 1;
+        ns.phase = st.phase + 1;
+        return ns;
+    }
+    return next_level(a, st, ld_relaxed_u64(&a.ctl->qpack[(st.L + 1) & 3]),
+                      st.uwrite ? ld_relaxed_u32(&a.ctl->ucount[(st.L + 1) & 3]) : 0u, stats);
 }
 
 // Loads warp tile `tile` of the frontier's edge sequence: the frontier
@@ -998,28 +1018,325 @@ __device__ void init_phase(const BfsArgs<OffT> &a, const LevelState &st0) {
         a.ctl->cpack = 0ull;
         for (int i = 0; i < 4; ++i) a.ctl->wq[i] = 0u;
         for (int i = 0; i < 4; ++i) a.ctl->ucount[i] = 0u;
+        atomicAdd(&a.ctl->narrow_epoch, 1u);     // as does every call: one that gave up left its tags
     }
+}
+
+// ---------------------------------------------------------------------------
+// Narrow levels (narrow.cuh): queue push levels of at most 32,768 edges (512 a
+// block).  On a 4096 x 4096 grid, levels of 15,000 edges took 16.9 us and take
+// 4.0, levels of 20 edges 8.3 and 3.1; the traversal 87 -> 23 ms (28 on
+// another card).  What is left is the chain lines -> piece -> column -> visited -> lines, five trips to L2.
+// ---------------------------------------------------------------------------
+
+// Whether the level st may be run by the narrow group from here on.  The
+// group clears the frontier bitmaps by itself, so it has to be little: a small
+// bitmap, or one whose bits are those of a short queue.  Going in and out costs
+// what two levels save, so three small levels have to have gone before (an
+// R-MAT traversal has two at its start and two or three at its end, and was
+// 12 us slower when one was enough); half the limit to come in, the limit to
+// stay.
+template <typename OffT>
+__device__ bool narrow_may_start(const BfsArgs<OffT> &a, const LevelState &st) {
+    if (!a.narrow || st.narrow == NARROW_OFF || st.done || st.dir != DIR_PUSH || st.phase || st.compact || st.bmp || !st.qin)
+        return false;
+    if (st.calm < 3 || st.T > narrow_max_T() / 2) return false;
+    return a.words <= 65536 || !st.fclear || (st.qprev_ok && st.nprev <= NARROW_MAX_T);
+}
+
+// A found vertex (or none) into the block's segments of level L.
+template <typename OffT>
+__device__ __forceinline__ void bfs_narrow_append(const BfsArgs<OffT> &a, NarrowShared<GRX_NARROW_BLOCKS> &sh, int L,
+                                                  unsigned long long tag, bool has, int32_t v, uint32_t row,
+                                                  uint32_t deg) {
+    narrow_append(sh, a.narrow->pieces[L & 1][blockIdx.x], NARROW_PIECES, a.narrow->verts[L % 3][blockIdx.x],
+                  NARROW_VERTS, tag, has, v, row, deg, a.ctl);
+}
+
+template <typename OffT, typename Ahead>
+__device__ __forceinline__ bool bfs_narrow_exchange(const BfsArgs<OffT> &a, NarrowShared<GRX_NARROW_BLOCKS> &sh,
+                                                    unsigned long long tag, bool fence, Ahead &&ahead) {
+    return narrow_exchange(a.narrow->lines[tag & 1], sh, (int)narrow_group(), tag, fence, a.ctl, a.timeout_ns, ahead);
+}
+
+// One level: a quad of lanes takes a piece, a lane its edge.  The row bounds of
+// the target travel with the atomic on visited (most targets of a sparse
+// frontier are new), and the columns of a found vertex are asked into L2 for the
+// next level.  A lane's last finds are left in row / deg (deg 0: none).
+template <typename OffT, bool PARENT>
+__device__ __forceinline__ void narrow_level(const BfsArgs<OffT> &a, const LevelState &st, NarrowShared<GRX_NARROW_BLOCKS> &sh,
+                                             unsigned long long tag, uint32_t (&row)[2], uint32_t (&deg)[2]) {
+    const int L = st.L;
+    const unsigned int lane = threadIdx.x & 31;
+    const uint32_t group = narrow_group(), step = group * WARPS * 8;
+    const uint32_t mine = ((threadIdx.x >> 5) * group + blockIdx.x) * 8 + (lane >> 2);
+    const uint32_t total = sh.first[GRX_NARROW_BLOCKS];
+    uint32_t *Fout = pick3(a.F[0], a.F[1], a.F[2], (L + 1) % 3);
+    for (uint32_t base = 0; base < total; base += 2 * step) {
+        int32_t v[2], u[2];
+        bool ok[2];
+        OffT rb[2], re[2];
+        uint32_t old[2];
+        const NarrowWord *at[2];
+        NarrowWord w[2];
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+            const uint32_t c = base + k * step + mine;
+            ok[k] = c < total;
+            at[k] = nullptr;
+            if (ok[k]) {
+                uint32_t i;
+                const uint32_t b = narrow_find(sh, c, i);
+                at[k] = &a.narrow->pieces[L & 1][b][i];
+                w[k] = narrow_load(at[k]);
+            }
+        }
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+            v[k] = u[k] = 0;
+            if (ok[k]) ok[k] = narrow_await(at[k], w[k], tag, a.ctl, a.timeout_ns) && (lane & 3) < narrow_len(w[k]);
+            if (ok[k]) {
+                v[k] = __ldg(a.col + narrow_edge(w[k]) + (lane & 3));
+                u[k] = narrow_vertex(w[k]);
+            }
+        }
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+            rb[k] = re[k] = 0;
+            old[k] = 0xffffffffu;
+            if (ok[k]) {
+                old[k] = atomicOr(a.visited + (v[k] >> 5), 1u << (v[k] & 31));
+                rb[k] = __ldg(a.ro + v[k]);
+                re[k] = __ldg(a.ro + v[k] + 1);
+            }
+        }
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+            const bool found = !((old[k] >> (v[k] & 31)) & 1u);
+            const bool has = found && re[k] > rb[k];
+            if (found) {
+                a.depth[v[k]] = L + 1;
+                if (PARENT) a.parent[v[k]] = u[k];
+                if (has) {
+                    asm volatile("prefetch.global.L2 [%0];" ::"l"(a.col + rb[k]));
+                    if (st.fwrite) atomicOr(Fout + (v[k] >> 5), 1u << (v[k] & 31));
+                }
+            }
+            row[k] = (uint32_t)rb[k];
+            deg[k] = has ? (uint32_t)(re[k] - rb[k]) : 0u;
+            bfs_narrow_append(a, sh, L + 1, tag + 1, has, v[k], row[k], deg[k]);
+        }
+    }
+}
+
+// Zeroes the words of F that hold bits of this block's vertices of level l.
+template <typename OffT>
+__device__ __forceinline__ void narrow_clear(const BfsArgs<OffT> &a, int l3, uint32_t own) {
+    uint32_t *F = pick3(a.F[0], a.F[1], a.F[2], l3);
+    for (uint32_t i = threadIdx.x; i < own; i += BFS_BLOCK)
+        F[__ldcg(&a.narrow->verts[l3][blockIdx.x][i]) >> 5] = 0u;
+}
+
+// Runs levels from s_st (in: a queue push level with Q_L) while they stay narrow.
+// Called by the group's blocks; leaves in ctl->hstate the state that every
+// block goes on from after the next grid barrier (with Q_L again, unless done).
+// false: a wait gave up.
+template <typename OffT, bool PARENT, bool STATS>
+__device__ bool narrow_run(const BfsArgs<OffT> &a, LevelState &s_st, NarrowShared<GRX_NARROW_BLOCKS> &sh, FlagBarrier &bar) {
+    // no tag of this stretch was used before: every stretch counts up the epoch
+    unsigned long long tag = (unsigned long long)(ld_relaxed_u32(&a.ctl->narrow_epoch) & 0x7fffffffu) << 32;
+    __shared__ uint32_t own[3];                  // vertices in this block's segments, by level mod 3
+    const uint32_t group = narrow_group();
+    const unsigned int lane = threadIdx.x & 31;
+    LevelState st = s_st;
+    if (threadIdx.x == 0) {
+        sh.got = 0ull;
+        sh.got_edges = 0ull;
+    }
+    __syncthreads();
+    {   // F_{L-1} and F_L hold nothing from here on (a push level reads neither)
+        const uint32_t g0 = blockIdx.x * BFS_BLOCK + threadIdx.x, gs = group * BFS_BLOCK;
+        for (int k = 0; k < 2; ++k) {
+            if (!(k ? st.fprev : st.fclear)) continue;
+            const int l3 = (st.L + 2 + k) % 3;
+            uint32_t *F = pick3(a.F[0], a.F[1], a.F[2], l3);
+            const int32_t *Q = pick3(a.Q[0], a.Q[1], a.Q[2], l3);
+            if (a.words <= 65536)
+                for (uint32_t i = g0; i < a.words; i += gs) F[i] = 0u;
+            else
+                for (uint32_t i = g0; i < (k ? st.q : st.nprev); i += gs) F[__ldcg(Q + i) >> 5] = 0u;
+        }
+    }
+    {   // Q_L into the group's segments
+        const int32_t *Q = pick3(a.Q[0], a.Q[1], a.Q[2], st.L % 3);
+        const OffT *R = pick3(a.R[0], a.R[1], a.R[2], st.L % 3);
+        const uint32_t i0 = (uint32_t)((uint64_t)st.q * blockIdx.x / group);
+        const uint32_t i1 = (uint32_t)((uint64_t)st.q * (blockIdx.x + 1) / group);
+        for (uint32_t base = i0 + (threadIdx.x & ~31u); base < i1; base += BFS_BLOCK) {
+            const uint32_t i = base + lane;
+            int32_t v = 0;
+            OffT row = 0;
+            uint32_t deg = 0;
+            if (i < i1) {
+                v = __ldcg(Q + i);
+                row = __ldcg(R + i);
+                deg = (uint32_t)(__ldg(a.ro + v + 1) - row);
+            }
+            bfs_narrow_append(a, sh, st.L, tag + 1, i < i1, v, (uint32_t)row, deg);
+        }
+    }
+    if (!bfs_narrow_exchange(a, sh, ++tag, true, [] {})) return false;
+    if (threadIdx.x == 0) {
+        own[0] = own[1] = own[2] = 0u;
+        own[st.L % 3] = sh.own;
+        s_st.fclear = 0;
+        s_st.fprev = 0;
+    }
+    __syncthreads();
+    uint32_t ran = 0;
+    for (;;) {
+        st = s_st;
+        if (st.done || st.dir != DIR_PUSH || st.bmp || st.T > narrow_max_T() || sh.most > NARROW_PIECES) break;
+        if (ran == a.narrow_levels) {            // the other blocks' wait is bounded: renew it
+            if (blockIdx.x == 0 && threadIdx.x == 0) {
+                st.narrow = NARROW_ON;
+                memcpy((void *)a.ctl->hstate[(bar.gen + 1) & 1], &st, sizeof st);
+            }
+            if (!flag_barrier(bar)) return false;
+            ran = 0;
+        }
+        ++ran;
+        const int L = st.L;
+        if (STATS && blockIdx.x == 0 && threadIdx.x == 0 && L < GRX_MAX_LEVELS_STATS) {
+            a.stats->level_t0[L] = grx_globaltimer();
+            a.stats->dir[L] = DIR_PUSH;
+            a.stats->frontier[L] = st.q;
+            a.stats->edges_examined[L] = st.T;
+            a.stats->vertices_scanned[L] = st.q;
+            a.stats->levels = L + 1;
+        }
+        if (st.fclear) narrow_clear(a, (L + 2) % 3, own[(L + 2) % 3]);
+        uint32_t row[2] = {0u, 0u}, deg[2] = {0u, 0u};
+        narrow_level<OffT, PARENT>(a, st, sh, tag, row, deg);
+        // The found rows' first targets: their row bounds are asked into L2 while
+        // the lines travel.  (A fence: the frontier bitmaps, where they are kept,
+        // are cleared and set by different blocks.)
+        auto ahead = [&] {
+            int32_t c[2][NARROW_PIECE];
+#pragma unroll
+            for (int k = 0; k < 2; ++k)
+#pragma unroll
+                for (int e = 0; e < NARROW_PIECE; ++e) c[k][e] = (uint32_t)e < deg[k] ? __ldg(a.col + row[k] + e) : -1;
+#pragma unroll
+            for (int k = 0; k < 2; ++k)
+#pragma unroll
+                for (int e = 0; e < NARROW_PIECE; ++e)
+                    if (c[k][e] >= 0) asm volatile("prefetch.global.L2 [%0];" ::"l"(a.ro + c[k][e]));
+        };
+        if (!bfs_narrow_exchange(a, sh, ++tag, st.fwrite || st.fclear, ahead))
+            return false;
+        if (threadIdx.x == 0) {
+            own[(L + 1) % 3] = sh.own;
+            s_st = next_level(a, st, ((unsigned long long)sh.verts << 32) | sh.edges, 0u, STATS);
+        }
+        __syncthreads();
+    }
+    if (!st.done) {                              // back to a queue: vertex, edge prefix, row start
+        if (st.fclear) narrow_clear(a, (st.L + 2) % 3, own[(st.L + 2) % 3]);
+        int32_t *Q = pick3(a.Q[0], a.Q[1], a.Q[2], st.L % 3);
+        uint32_t *E = pick3(a.E[0], a.E[1], a.E[2], st.L % 3);
+        OffT *R = pick3(a.R[0], a.R[1], a.R[2], st.L % 3);
+        const uint32_t n = own[st.L % 3];
+        uint32_t vb = 0, eb = 0;                 // vertices and edges of the blocks before
+        for (uint32_t b = 0; b < blockIdx.x; ++b) {
+            vb += sh.line_verts[b];
+            eb += sh.line_edges[b];
+        }
+        for (uint32_t base = 0; base < n; base += BFS_BLOCK) {
+            const uint32_t i = base + threadIdx.x;
+            int32_t v = 0;
+            OffT rb = 0;
+            uint32_t deg = 0;
+            if (i < n) {
+                v = __ldcg(&a.narrow->verts[st.L % 3][blockIdx.x][i]);
+                rb = __ldg(a.ro + v);
+                deg = (uint32_t)(__ldg(a.ro + v + 1) - rb);
+            }
+            uint32_t e0, x1, x2, esum, t1, t2;
+            block_scan3<BFS_BLOCK>(deg, 0u, 0u, e0, x1, x2, esum, t1, t2);
+            if (i < n) {
+                const uint32_t pos = vb + i;
+                Q[pos] = v;
+                E[pos] = eb + e0;
+                R[pos] = rb;
+            }
+            eb += esum;
+        }
+    }
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        a.ctl->narrow_epoch += 1;                // no block reads it before the next grid barrier
+        for (int i = 0; i < 4; ++i) {            // the rings start afresh
+            a.ctl->qpack[i] = 0ull;
+            a.ctl->ucount[i] = 0u;
+            a.ctl->wq[i] = 0u;
+        }
+        a.ctl->cpack = 0ull;
+        st.fclear = 0;
+        st.narrow = NARROW_OFF;                  // the level it stopped at may look narrow (one long row)
+        memcpy((void *)a.ctl->hstate[(bar.gen + 1) & 1], &st, sizeof st);
+    }
+    return true;
+}
+
+// A stretch of narrow levels, for every block of the grid: from s_st to the s_st
+// that all go on from.  Returns the grid barriers passed so far, 0 when a wait
+// gave up.
+template <typename OffT, bool PARENT, bool STATS>
+__device__ __forceinline__ unsigned int narrow_levels(const BfsArgs<OffT> &a, LevelState &s_st, NarrowShared<GRX_NARROW_BLOCKS> &sh,
+                                                      unsigned int gen) {
+    FlagBarrier bar{a.bar_flags, &a.ctl->bar_release, a.ctl, a.timeout_ns, gen};
+    const bool in = blockIdx.x < narrow_group();
+    if (in && !narrow_run<OffT, PARENT, STATS>(a, s_st, sh, bar)) return 0u;
+    do {
+        if (!flag_barrier(bar, in ? 32 : 500)) return 0u;
+        if (threadIdx.x == 0) {
+            const unsigned long long *h = (const unsigned long long *)a.ctl->hstate[bar.gen & 1];
+            unsigned long long words[8];
+            for (int i = 0; i < 8; ++i) words[i] = __ldcg(h + i);
+            memcpy(&s_st, words, sizeof s_st);
+        }
+        __syncthreads();
+    } while (s_st.narrow == NARROW_ON);
+    return bar.gen;
 }
 
 // The level's state stays in shared memory: a copy in registers made the pull
 // phase spill (R-MAT 16 / 22 / 26: 116 -> 112, 151 -> 144, 1,048 -> 1,018 us,
-// means of three sources).
-template <typename OffT, bool PARENT, bool STATS>
-__global__ void __launch_bounds__(BFS_BLOCK, GRX_BFS_MIN_BLOCKS) k_bfs_persistent(BfsArgs<OffT> a) {
+// means of three sources).  NARROW is a variant of its own because its code
+// costs the 64-bit phases registers again (R-MAT 26: 33 us).
+template <typename OffT, bool PARENT, bool STATS, bool NARROW>
+__global__ void __launch_bounds__(BFS_BLOCK, GRX_BFS_MIN_BLOCKS) k_bfs_persistent(const __grid_constant__ BfsArgs<OffT> a) {
     __shared__ LevelState s_st;
-    WarpSmem<OffT> &w = warp_smem<OffT>();
     FlagBarrier bar{a.bar_flags, &a.ctl->bar_release, a.ctl, a.timeout_ns, 0u};
     if (threadIdx.x == 0) s_st = initial_state(a);
     __syncthreads();
     init_phase<OffT, PARENT>(a, s_st);
     if (!flag_barrier(bar)) return;
     for (;;) {
-        const LevelState &st = s_st;
-        if (st.done) break;
-        run_phase<OffT, PARENT, STATS>(a, st, w);
-        if (!flag_barrier(bar)) return;
-        if (threadIdx.x == 0) s_st = next_state(a, st, STATS);
-        __syncthreads();
+        for (;;) {
+            const LevelState &st = s_st;
+            if (st.done || (NARROW && narrow_may_start(a, st))) break;
+            run_phase<OffT, PARENT, STATS>(a, st, warp_smem<OffT>());
+            if (!flag_barrier(bar)) return;
+            if (threadIdx.x == 0) s_st = next_state(a, st, STATS);
+            __syncthreads();
+        }
+        if (!NARROW || s_st.done) break;
+        if constexpr (NARROW) {
+            __shared__ NarrowShared<GRX_NARROW_BLOCKS> s_narrow;
+            bar.gen = narrow_levels<OffT, PARENT, STATS>(a, s_st, s_narrow, bar.gen);
+            if (bar.gen == 0u) return;
+        }
     }
     if (blockIdx.x == 0 && threadIdx.x == 0) {
         a.ctl->levels_run = s_st.L;
@@ -1093,7 +1410,9 @@ grx_status prepare_kernels() {
     static bool done = false;
     if (done) return GRX_OK;
     const int bytes = (int)bfs_smem_bytes<OffT>();
-    GRX_CUDA(cudaFuncSetAttribute((const void *)k_bfs_persistent<OffT, PARENT, STATS>,
+    GRX_CUDA(cudaFuncSetAttribute((const void *)k_bfs_persistent<OffT, PARENT, STATS, false>,
+                                  cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
+    GRX_CUDA(cudaFuncSetAttribute((const void *)k_bfs_persistent<OffT, PARENT, STATS, true>,
                                   cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
     GRX_CUDA(cudaFuncSetAttribute((const void *)k_bfs_step<OffT, PARENT, STATS>,
                                   cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
@@ -1145,6 +1464,10 @@ BfsArgs<OffT> make_args(grx_graph *g, int32_t src, int32_t *depth, int32_t *pare
     a.ulist_max = (uint32_t)(g->nv / 64 > 0 ? g->nv / 64 : 1);
     a.timeout_ns = grx_timeout_ns(o);
     a.src = src;
+    a.narrow = g->narrow;
+    // a narrow level takes a few microseconds: far less than the bound on a wait
+    const unsigned long long nl = a.timeout_ns >> 16;
+    a.narrow_levels = nl < 1 ? 1u : (nl > 256 ? 256u : (uint32_t)nl);
     return a;
 }
 
@@ -1201,6 +1524,29 @@ grx_status graph_exec(grx_graph *g, cudaGraphExec_t *out) {
     return GRX_OK;
 }
 
+template <typename OffT, bool PARENT, bool STATS, bool NARROW>
+grx_status launch_persistent(grx_graph *g, const BfsArgs<OffT> &a, const grx_opts *o, cudaStream_t s) {
+    const size_t smem = bfs_smem_bytes<OffT>();
+    static int max_blocks_per_sm = -1;
+    if (max_blocks_per_sm < 0) {
+        GRX_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(
+            &max_blocks_per_sm, k_bfs_persistent<OffT, PARENT, STATS, NARROW>, BFS_BLOCK, smem));
+        if (max_blocks_per_sm < 1)
+            return grx_fail(GRX_ECUDA, "bfs: persistent kernel does not fit on an SM");
+    }
+    int max_grid = max_blocks_per_sm * g->ctx->num_sms;
+    if (max_grid > GRX_MAX_GRID) max_grid = GRX_MAX_GRID;
+    int blocks = o->grid_blocks > 0 && o->grid_blocks < max_grid ? o->grid_blocks : max_grid;
+    GRX_CUDA(cudaMemsetAsync(g->bar_flags, 0, sizeof(unsigned int) * (size_t)blocks, s));
+    GRX_CUDA(cudaMemsetAsync(&g->ctl->bar_release, 0, sizeof(unsigned int), s));
+    void *args[] = {(void *)&a};
+    if (o->ev_begin) GRX_CUDA(cudaEventRecord((cudaEvent_t)o->ev_begin, s));
+    GRX_CUDA(cudaLaunchCooperativeKernel((const void *)k_bfs_persistent<OffT, PARENT, STATS, NARROW>,
+                                         dim3(blocks), dim3(BFS_BLOCK), args, smem, s));
+    if (o->ev_end) GRX_CUDA(cudaEventRecord((cudaEvent_t)o->ev_end, s));
+    return GRX_OK;
+}
+
 template <typename OffT, bool PARENT, bool STATS>
 grx_status launch_typed(grx_graph *g, int32_t src, int32_t *depth, int32_t *parent,
                         const grx_opts *o, cudaStream_t s) {
@@ -1245,24 +1591,11 @@ grx_status launch_typed(grx_graph *g, int32_t src, int32_t *depth, int32_t *pare
         GRX_CUDA(cudaGetLastError());
         return GRX_OK;
     }
-    static int max_blocks_per_sm = -1;
-    if (max_blocks_per_sm < 0) {
-        GRX_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-            &max_blocks_per_sm, k_bfs_persistent<OffT, PARENT, STATS>, BFS_BLOCK, smem));
-        if (max_blocks_per_sm < 1)
-            return grx_fail(GRX_ECUDA, "bfs: persistent kernel does not fit on an SM");
-    }
-    int max_grid = max_blocks_per_sm * g->ctx->num_sms;
-    if (max_grid > GRX_MAX_GRID) max_grid = GRX_MAX_GRID;
-    int blocks = o->grid_blocks > 0 && o->grid_blocks < max_grid ? o->grid_blocks : max_grid;
-    GRX_CUDA(cudaMemsetAsync(g->bar_flags, 0, sizeof(unsigned int) * (size_t)blocks, s));
-    GRX_CUDA(cudaMemsetAsync(&g->ctl->bar_release, 0, sizeof(unsigned int), s));
-    void *args[] = {(void *)&a};
-    if (o->ev_begin) GRX_CUDA(cudaEventRecord((cudaEvent_t)o->ev_begin, s));
-    GRX_CUDA(cudaLaunchCooperativeKernel((const void *)k_bfs_persistent<OffT, PARENT, STATS>,
-                                         dim3(blocks), dim3(BFS_BLOCK), args, smem, s));
-    if (o->ev_end) GRX_CUDA(cudaEventRecord((cudaEvent_t)o->ev_end, s));
-    return GRX_OK;
+    // Narrow levels on graphs of few edges a vertex, which may have thousands of
+    // levels; where vertices have more, everything is reached in a few.
+    return a.narrow && g->ne < 8ll * g->nv && o->direction != GRX_DIR_PULL
+               ? launch_persistent<OffT, PARENT, STATS, true>(g, a, o, s)
+               : launch_persistent<OffT, PARENT, STATS, false>(g, a, o, s);
 }
 
 template <typename OffT>

@@ -7,6 +7,7 @@
 #include <cstring>
 
 #include "grx_internal.cuh"
+#include "narrow.cuh"
 
 // ---------------------------------------------------------------------------
 // errors
@@ -331,6 +332,7 @@ grx_status grx_ensure_workspace(grx_graph *g, cudaStream_t s) {
     for (int i = 0; i < 3; ++i) ok = ok && g->fbits[i] && g->qv[i] && g->qe[i] && g->qr[i];
     for (int i = 0; i < 2; ++i) ok = ok && g->ulist[i];
     if (!ok) return grx_fail(GRX_ENOMEM, "traversal workspace allocation failed (nv=%d)", g->nv);
+    g->narrow = (NarrowBuffers *)grx_alloc(g, sizeof(NarrowBuffers), s);   // traversals do without it
     GRX_CUDA(cudaMemsetAsync(g->ctl, 0, sizeof(TravCtl), s));
     GRX_CUDA(cudaMemsetAsync(g->stats, 0, sizeof(DevStats), s));
     grx_status st = grx_build_first2(g, s);
@@ -359,7 +361,7 @@ static size_t workspace_new_bytes(const grx_graph *g, bool multi) {
     size_t b = 0;
     if (!g->ws_ready)
         b += wb + 3 * (wb + nv * 8 + nv * (g->off64 ? 8 : 4)) + 2 * nv * 4 + nv * sizeof(int2) +
-             sizeof(TravCtl) + sizeof(unsigned int) * GRX_MAX_GRID + sizeof(DevStats) + nv * 4;
+             sizeof(TravCtl) + sizeof(unsigned int) * GRX_MAX_GRID + sizeof(DevStats) + nv * 4 + sizeof(NarrowBuffers);
     if (multi && !g->ms_ready) b += 5 * nv * 8;
     return b;
 }

@@ -51,6 +51,7 @@ struct alignas(128) TravCtl {
     unsigned int bar_release;        // flag-barrier release word (own line)
     unsigned int pad4[31];
     unsigned long long pairs[4];     // multi-source: (vertex, lane) pairs discovered, ring
+    unsigned int narrow_epoch;       // stretches that may have used the narrow buffers (never reset)
 };
 
 // Maximum grid of the persistent kernels (size of the barrier flag array).
@@ -145,6 +146,7 @@ struct grx_graph {
     double *bcm_sig, *bcm_acc;       // [nv][64]
     int32_t *bcm_srcs;               // [64] device copy of the sources
     // CUDA-graph level loop of bfs (GRX_LOOP_GRAPH), per parent flag
+    struct NarrowBuffers *narrow;    // narrow levels (narrow.cuh); NULL: none
     cudaGraphExec_t bfs_gexec[2];
     void *bfs_gargs;                 // device copy of the call's arguments
     // 64-bit vertex ids (graph_load_csr64): columns, frontier queues and
@@ -292,7 +294,8 @@ __device__ __forceinline__ bool grid_barrier(TravCtl *ctl, unsigned long long ti
 // one word.  No contended atomic.  `gen` counts barriers within a launch
 // (flags and release word are zeroed before the launch, gen starts at 0).
 // Every wait is bounded by timeout_ns; a block that gives up records
-// GRX_ETIMEOUT and returns false.
+// GRX_ETIMEOUT and returns false.  sleep_ns: pause between two looks at the
+// release word.
 struct FlagBarrier {
     unsigned int *flags;
     unsigned int *release;
@@ -301,7 +304,7 @@ struct FlagBarrier {
     unsigned int gen;
 };
 
-__device__ __forceinline__ bool flag_barrier(FlagBarrier &b) {
+__device__ __forceinline__ bool flag_barrier(FlagBarrier &b, unsigned int sleep_ns = 32) {
     __shared__ int s_ok;
     const unsigned int gen = ++b.gen;
     __syncthreads();
@@ -337,7 +340,7 @@ __device__ __forceinline__ bool flag_barrier(FlagBarrier &b) {
                     ok = 0;
                     break;
                 }
-                __nanosleep(32);
+                __nanosleep(sleep_ns);
             }
         }
         __threadfence();
