@@ -333,6 +333,8 @@ grx_status grx_ensure_workspace(grx_graph *g, cudaStream_t s) {
     for (int i = 0; i < 2; ++i) ok = ok && g->ulist[i];
     if (!ok) return grx_fail(GRX_ENOMEM, "traversal workspace allocation failed (nv=%d)", g->nv);
     g->narrow = (NarrowBuffers *)grx_alloc(g, sizeof(NarrowBuffers), s);   // traversals do without it
+    // (memory of a freed graph could hold words with this graph's first tags)
+    if (g->narrow) GRX_CUDA(cudaMemsetAsync(g->narrow, 0, sizeof(NarrowBuffers), s));
     GRX_CUDA(cudaMemsetAsync(g->ctl, 0, sizeof(TravCtl), s));
     GRX_CUDA(cudaMemsetAsync(g->stats, 0, sizeof(DevStats), s));
     grx_status st = grx_build_first2(g, s);

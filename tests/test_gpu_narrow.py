@@ -64,3 +64,20 @@ def test_bfs_through_narrow_levels(grx, name, off64, direction):
             d, p = d.cpu().numpy(), p.cpu().numpy()
             assert np.array_equal(d, want), (name, src, kw)
             assert oracle.check_bfs(g.row_offsets, g.col_indices, src, d, p) == 0
+
+
+def _weighted(g, wmax, seed):
+    w = inputs.edge_weights(g.row_offsets, g.col_indices, wmax, seed)
+    return inputs.Graph(g.name, g.row_offsets, g.col_indices, w)
+
+
+def test_a_new_graph_in_the_memory_of_a_freed_one(grx):
+    """Words left by a freed graph's traversals are not taken for the new one's."""
+    for k in range(4):
+        g = _weighted(inputs.grid_graph(120 + k, 90, p_del=0.1, seed=k), 50, k)
+        dg = grx.load(g)
+        src = int(inputs.pick_sources(g.row_offsets, 1, seed=k)[0])
+        assert np.array_equal(grx.bfs(dg, src).cpu().numpy(), oracle.bfs(g.row_offsets, g.col_indices, src))
+        d = grx.sssp(dg, src, opts=grx.opts(sssp_delta=200))
+        assert np.array_equal(grx.as_uint32(d), oracle.sssp(g.row_offsets, g.col_indices, g.weights, src))
+        dg.free()
