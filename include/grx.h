@@ -117,7 +117,8 @@ typedef struct {
     float alpha;          /* push->pull when FV > BV * alpha (paper: do_a) */
     float beta;           /* pull->push when FV < BV * beta  (paper: do_b) */
     int loop;             /* GRX_LOOP_* */
-    int grid_blocks;      /* persistent grid size; 0 = SMs x occupancy */
+    int grid_blocks;      /* persistent grid size in units of 256 threads;
+                             0 = SMs x occupancy */
     int block_threads;    /* 0 = library default */
     double timeout_s;     /* bound on every device-side wait; <= 0 = 5 s */
     int collect_stats;    /* record per-level counters for grx_last_stats */

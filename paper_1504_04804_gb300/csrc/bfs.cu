@@ -59,10 +59,11 @@ namespace {
 #define GRX_PUSH_DEDUP 1
 #endif
 
-constexpr int BFS_BLOCK = 256;
-#ifndef GRX_BFS_MIN_BLOCKS
-#define GRX_BFS_MIN_BLOCKS 3                        // resident blocks per SM (register cap)
-#endif
+// Two blocks of 384 threads an SM: as many warps as three of 256, but a third
+// fewer blocks in every grid barrier (R-MAT 16 / 22 / 26, means of three sources:
+// 123 -> 116, 143 -> 141, 1,030 -> 992 us; one block of 768: 112, 148, 993).
+constexpr int BFS_BLOCK = 384;
+constexpr int BFS_MIN_BLOCKS = 2;                   // resident blocks per SM (register cap)
 constexpr int WARPS = BFS_BLOCK / 32;
 constexpr int PUSH_ITEMS = GRX_PUSH_ITEMS;
 constexpr int WTILE = 32 * PUSH_ITEMS;              // edges per warp tile
@@ -1315,7 +1316,7 @@ __device__ __forceinline__ unsigned int narrow_levels(const BfsArgs<OffT> &a, Le
 // means of three sources).  NARROW is a variant of its own because its code
 // costs the 64-bit phases registers again (R-MAT 26: 33 us).
 template <typename OffT, bool PARENT, bool STATS, bool NARROW>
-__global__ void __launch_bounds__(BFS_BLOCK, GRX_BFS_MIN_BLOCKS) k_bfs_persistent(const __grid_constant__ BfsArgs<OffT> a) {
+__global__ void __launch_bounds__(BFS_BLOCK, BFS_MIN_BLOCKS) k_bfs_persistent(const __grid_constant__ BfsArgs<OffT> a) {
     __shared__ LevelState s_st;
     FlagBarrier bar{a.bar_flags, &a.ctl->bar_release, a.ctl, a.timeout_ns, 0u};
     if (threadIdx.x == 0) s_st = initial_state(a);
@@ -1501,7 +1502,7 @@ grx_status graph_exec(grx_graph *g, cudaGraphExec_t *out) {
         cudaKernelNodeParams k1 = {};
         void *a1[] = {(void *)&ap};
         k1.func = (void *)k_bfs_glevel<OffT, PARENT>;
-        k1.gridDim = dim3(g->ctx->num_sms * 3);
+        k1.gridDim = dim3(g->ctx->num_sms * 3 * 256 / BFS_BLOCK);
         k1.blockDim = dim3(BFS_BLOCK);
         k1.sharedMemBytes = (unsigned int)bfs_smem_bytes<OffT>();
         k1.kernelParams = a1;
@@ -1536,7 +1537,7 @@ grx_status launch_persistent(grx_graph *g, const BfsArgs<OffT> &a, const grx_opt
     }
     int max_grid = max_blocks_per_sm * g->ctx->num_sms;
     if (max_grid > GRX_MAX_GRID) max_grid = GRX_MAX_GRID;
-    int blocks = o->grid_blocks > 0 && o->grid_blocks < max_grid ? o->grid_blocks : max_grid;
+    const int blocks = grx_grid(o, BFS_BLOCK, max_grid);
     GRX_CUDA(cudaMemsetAsync(g->bar_flags, 0, sizeof(unsigned int) * (size_t)blocks, s));
     GRX_CUDA(cudaMemsetAsync(&g->ctl->bar_release, 0, sizeof(unsigned int), s));
     void *args[] = {(void *)&a};
@@ -1563,14 +1564,14 @@ grx_status launch_typed(grx_graph *g, int32_t src, int32_t *depth, int32_t *pare
         // initialisation launch and the level loop
         GRX_CUDA(cudaMemcpyAsync(g->bfs_gargs, &a, sizeof a, cudaMemcpyHostToDevice, s));
         if (o->ev_begin) GRX_CUDA(cudaEventRecord((cudaEvent_t)o->ev_begin, s));
-        k_bfs_step<OffT, PARENT, false><<<g->ctx->num_sms * 3, BFS_BLOCK, smem, s>>>(a, 0);
+        k_bfs_step<OffT, PARENT, false><<<g->ctx->num_sms * 3 * 256 / BFS_BLOCK, BFS_BLOCK, smem, s>>>(a, 0);
         GRX_CUDA(cudaGetLastError());
         GRX_CUDA(cudaGraphLaunch(ex, s));
         if (o->ev_end) GRX_CUDA(cudaEventRecord((cudaEvent_t)o->ev_end, s));
         return GRX_OK;
     }
     if (o->loop == GRX_LOOP_HOST) {
-        int blocks = o->grid_blocks > 0 ? o->grid_blocks : g->ctx->num_sms * 4;
+        const int blocks = grx_grid(o, BFS_BLOCK, o->grid_blocks > 0 ? 1 << 30 : g->ctx->num_sms * 4 * 256 / BFS_BLOCK);
         // Poll the done flag every 16 launches; a traversal has at most nv
         // levels of at most 3 phases each.
         long long st_host[8];

@@ -115,6 +115,12 @@ unsigned long long grx_timeout_ns(const grx_opts *o) {
     return (unsigned long long)ns;
 }
 
+int grx_grid(const grx_opts *o, int threads, int max_grid) {
+    if (o->grid_blocks <= 0) return max_grid;
+    const long long b = ((long long)o->grid_blocks * 256 + threads - 1) / threads;
+    return b < max_grid ? (int)b : max_grid;
+}
+
 // ---------------------------------------------------------------------------
 // graph loading
 // ---------------------------------------------------------------------------

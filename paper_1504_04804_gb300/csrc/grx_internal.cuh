@@ -198,6 +198,9 @@ grx_status grx_mssp_launch(grx_graph *g, const int32_t *srcs, int n, uint32_t *d
 // Options resolution.
 void grx_resolve_opts(const grx_opts *in, grx_opts *out);
 unsigned long long grx_timeout_ns(const grx_opts *o);
+// Blocks of `threads` of a persistent grid: opts->grid_blocks (of 256 threads) or
+// max_grid if that is less or none is asked for.
+int grx_grid(const grx_opts *o, int threads, int max_grid);
 
 // Kernel launchers (one per translation unit).
 grx_status grx_bfs_launch(grx_graph *g, int32_t src, int32_t *depth, int32_t *parent,

@@ -26,9 +26,9 @@
 constexpr int NARROW_PIECE = 4;              // edges per piece: a quad of lanes
 constexpr uint32_t NARROW_PIECES = 2048;     // pieces a block's segment holds
 constexpr uint32_t NARROW_MAX_T = 32768;     // edges of a narrow frontier, at most
-// Vertices a block can find in one level: its share of the pieces (whole warp
-// steps of 8), four edges each.
-constexpr uint32_t NARROW_VERTS = NARROW_PIECE * (NARROW_MAX_T / GRX_NARROW_BLOCKS + 8 * 8 * 2);
+// Vertices a block can find in one level: its share of the pieces (whole steps of
+// 12 warps x 8 pieces x 2), four edges each.
+constexpr uint32_t NARROW_VERTS = NARROW_PIECE * (NARROW_MAX_T / GRX_NARROW_BLOCKS + 12 * 8 * 2);
 
 // A 16-byte word that is written and read as one.
 struct alignas(16) NarrowWord {
