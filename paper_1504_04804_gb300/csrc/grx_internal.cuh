@@ -146,6 +146,9 @@ struct grx_graph {
     double *bcm_sig, *bcm_acc;       // [nv][64]
     int32_t *bcm_srcs;               // [64] device copy of the sources
     // CUDA-graph level loop of bfs (GRX_LOOP_GRAPH), per parent flag
+    void *ss_lines;                  // list rounds of sssp: lines, pieces, vertices (first use)
+    uint32_t ss_list_T;              // ... edges of a round per block
+    int ss_list_blocks;              // ... blocks they are laid out for
     struct NarrowBuffers *narrow;    // narrow levels (narrow.cuh); NULL: none
     cudaGraphExec_t bfs_gexec[2];
     void *bfs_gargs;                 // device copy of the call's arguments

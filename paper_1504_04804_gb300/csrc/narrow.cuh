@@ -157,6 +157,61 @@ __device__ __forceinline__ bool narrow_exchange(NarrowWord *lines, NarrowShared<
     return sh.ok != 0;
 }
 
+// The same for a group of up to NT = blockDim.x blocks: every thread waits for a
+// line.  No fence: what the blocks leave for each other beside the pieces has
+// to have reached L2 (atomics whose results were used).
+template <int NT, int NB>
+__device__ __forceinline__ bool narrow_exchange_wide(NarrowWord *lines, NarrowShared<NB> &sh, int group,
+                                                     unsigned long long tag, TravCtl *ctl,
+                                                     unsigned long long timeout_ns) {
+    static_assert(NT <= NB, "a line a thread");
+    __shared__ uint32_t ws[4][NT / 32];              // per warp: pieces, vertices, edges, largest segment
+    __syncthreads();
+    if (threadIdx.x == 0) narrow_publish(lines, sh, tag, false);
+    const unsigned int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    uint32_t q = 0u, p = 0u, e = 0u;
+    bool ok = true;
+    if ((int)threadIdx.x < group) ok = narrow_collect(lines + threadIdx.x, tag, q, p, e, timeout_ns);
+    uint32_t cp = p;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t y = __shfl_up_sync(GRX_FULL_MASK, cp, o);
+        if (lane >= (unsigned)o) cp += y;
+    }
+    const uint32_t verts = __reduce_add_sync(GRX_FULL_MASK, q);
+    const uint32_t edges = __reduce_add_sync(GRX_FULL_MASK, e);
+    const uint32_t most = __reduce_max_sync(GRX_FULL_MASK, p);
+    if (lane == 31) {
+        ws[0][wid] = cp;
+        ws[1][wid] = verts;
+        ws[2][wid] = edges;
+        ws[3][wid] = most;
+    }
+    ok = __syncthreads_and(ok);
+    uint32_t before = 0, tp = 0, tv = 0, te = 0, tm = 0;
+#pragma unroll
+    for (int w = 0; w < NT / 32; ++w) {
+        const uint32_t x = ws[0][w];
+        if ((unsigned)w < wid) before += x;
+        tp += x;
+        tv += ws[1][w];
+        te += ws[2][w];
+        tm = max(tm, ws[3][w]);
+    }
+    sh.first[threadIdx.x] = before + cp - p;
+    sh.line_verts[threadIdx.x] = q;
+    sh.line_edges[threadIdx.x] = e;
+    for (int i = NT + (int)threadIdx.x; i <= NB; i += NT) sh.first[i] = tp;
+    if (threadIdx.x == 0) {
+        sh.verts = tv;
+        sh.edges = te;
+        sh.most = tm;
+        if (!ok) grx_set_status(ctl, GRX_ETIMEOUT);
+    }
+    __syncthreads();
+    return ok;
+}
+
 // Block and place in its segment of piece c of the frontier (c < first[NB]).
 template <int NB>
 __device__ __forceinline__ uint32_t narrow_find(const NarrowShared<NB> &sh, uint32_t c, uint32_t &at) {

@@ -29,14 +29,18 @@
 // entries below the old threshold were relaxed since and are dropped.  High-
 // diameter weighted graphs then relax far fewer edges more than once.
 // Rounds and phases are separated by the bounded grid barrier.
+//
+// On graphs of few edges a vertex, whose shortest paths take thousands of small
+// rounds, rounds that fit run on lists instead (list_round): the whole grid
+// with the exchange and the pieces of the narrow levels (narrow.cuh).
 #include "grx_internal.cuh"
+#include "narrow.cuh"
 
 namespace {
 
-constexpr int SS_BLOCK = 256;
-#ifndef GRX_SS_MIN_BLOCKS
-#define GRX_SS_MIN_BLOCKS 3                         // resident blocks per SM (register cap)
-#endif
+// Two blocks of 384 threads an SM, as in bfs.cu (R-MAT 22: 1,578 -> 1,525 us).
+constexpr int SS_BLOCK = 384;
+constexpr int SS_MIN_BLOCKS = 2;             // resident blocks per SM (register cap)
 constexpr int SS_WARPS = SS_BLOCK / 32;
 constexpr int SS_ITEMS = 8;
 constexpr int SS_WTILE = 32 * SS_ITEMS;
@@ -64,7 +68,18 @@ struct SsspArgs {
     uint32_t bmp_min_T;
     unsigned long long timeout_ns;
     int32_t src;
+    // list rounds (lines NULL: none), per block: pieces by round parity, vertices
+    NarrowWord *lines, *pieces;
+    int32_t *verts;
+    uint32_t list_T;                         // edges of a round, at most, per block
 };
+
+constexpr int SS_LIST_BLOCKS = 512;          // blocks of a list round: at most SS_BLOCK, searched as 512
+// Per block, for rounds of at most t edges a block: pieces a segment holds (a
+// round with a fuller one leaves the list rounds), and vertices a block can
+// find (its whole steps of 192 pieces, four edges each).
+__host__ __device__ inline uint32_t ss_list_pieces(uint32_t t) { return t; }
+__host__ __device__ inline uint32_t ss_list_verts(uint32_t t) { return 4 * (t + SS_WARPS * 8 * 2); }
 
 enum { SOP_RELAX, SOP_FINAL, SOP_FARMIN, SOP_FARSPLIT };
 
@@ -73,6 +88,7 @@ struct SsState {
     int op;
     int bmp;
     int done;
+    int nolist;                              // run this round on the queue, whatever its size
     int fsel;                                // current far pile
     uint32_t q, T;
     uint32_t thr;                            // near-far threshold (UINT32_MAX: no bands)
@@ -326,10 +342,236 @@ __device__ void far_split(const SsspArgs<OffT> &a, const SsState &st) {
     }
 }
 
+// ---------------------------------------------------------------------------
+// List rounds.  Per edge, three dependent trips to memory (piece; column, weight
+// and the source's distance; the target's distance and row bounds) and one for
+// the claim: the minimum and the round stamp are taken at once.  A proposal that
+// beats the distance read means that the target improves in this round, by it or
+// by a smaller one, so whoever sets the stamp may queue the target.  On a weighted
+// 4096 x 4096 grid (rounds of 170,000 edges on average) a round took 22.5 us on the
+// queue (search in the degree prefix, row lookup, global append counter, barrier)
+// and takes 11.6, rounds of 100 edges 13 and 7; the traversal 131 -> 78 ms.
+// ---------------------------------------------------------------------------
+// atomicMin that has taken effect when it returns (the result is waited for).
+__device__ __forceinline__ void ss_min_done(uint32_t *p, uint32_t x) {
+    uint32_t old;
+    asm volatile("atom.relaxed.gpu.global.min.u32 %0, [%1], %2;" : "=r"(old) : "l"(p), "r"(x) : "memory");
+    asm volatile("{\n\t.reg .u32 sink;\n\tmov.u32 sink, %0;\n\t}" ::"r"(old));
+}
+
+template <typename OffT>
+__device__ __forceinline__ void ss_list_append(const SsspArgs<OffT> &a, NarrowShared<SS_LIST_BLOCKS> &sh, int L,
+                                               unsigned long long tag, bool has, int32_t v, uint32_t row,
+                                               uint32_t deg) {
+    const uint32_t cap = ss_list_pieces(a.list_T), vcap = ss_list_verts(a.list_T);
+    const size_t seg = (size_t)(L & 1) * gridDim.x + blockIdx.x;
+    narrow_append(sh, a.pieces + seg * cap, cap, a.verts + seg * vcap, vcap, tag, has, v, row, deg, a.ctl);
+}
+
+template <typename OffT>
+__device__ __forceinline__ void list_round(const SsspArgs<OffT> &a, const SsState &st,
+                                           NarrowShared<SS_LIST_BLOCKS> &sh, unsigned long long tag) {
+    const int L = st.L;
+    const unsigned int lane = threadIdx.x & 31;
+    const uint32_t step = gridDim.x * SS_WARPS * 8;
+    const uint32_t mine = ((threadIdx.x >> 5) * gridDim.x + blockIdx.x) * 8 + (lane >> 2);
+    const uint32_t total = sh.first[SS_LIST_BLOCKS], cap = ss_list_pieces(a.list_T);
+    const NarrowWord *segs = a.pieces + (size_t)(L & 1) * gridDim.x * cap;
+    for (uint32_t base = 0; base < total; base += 2 * step) {
+        const NarrowWord *at[2];
+        NarrowWord w[2];
+        bool ok[2];
+        int32_t v[2];
+        uint32_t wt[2], du[2], nd[2], cur[2];
+        OffT rb[2], re[2];
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+            const uint32_t c = base + k * step + mine;
+            ok[k] = c < total;
+            at[k] = nullptr;
+            if (ok[k]) {
+                uint32_t i;
+                const uint32_t b = narrow_find(sh, c, i);
+                at[k] = segs + (size_t)b * cap + i;
+                w[k] = narrow_load(at[k]);
+            }
+        }
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+            v[k] = 0;
+            wt[k] = 0u;
+            du[k] = 0xffffffffu;
+            if (ok[k]) ok[k] = narrow_await(at[k], w[k], tag, a.ctl, a.timeout_ns) && (lane & 3) < narrow_len(w[k]);
+            if (ok[k]) {
+                v[k] = __ldg(a.col + narrow_edge(w[k]) + (lane & 3));
+                wt[k] = __ldg(a.w + narrow_edge(w[k]) + (lane & 3));
+                du[k] = __ldcg(a.dist + narrow_vertex(w[k]));
+            }
+        }
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+            cur[k] = 0u;
+            rb[k] = re[k] = 0;
+            if (ok[k]) {
+                cur[k] = __ldcg(a.dist + v[k]);
+                rb[k] = __ldg(a.ro + v[k]);
+                re[k] = __ldg(a.ro + v[k] + 1);
+            }
+            nd[k] = 0xffffffffu;
+            if (ok[k] && du[k] != 0xffffffffu) {
+                const uint64_t s64 = (uint64_t)du[k] + wt[k];
+                if (s64 >= 0xffffffffull) grx_set_status(a.ctl, GRX_ERANGE);
+                else nd[k] = (uint32_t)s64;
+            }
+        }
+        int32_t stamp[2];
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+            stamp[k] = L + 1;
+            if (nd[k] < cur[k]) {
+                if (nd[k] < st.thr) stamp[k] = atomicExch(a.stamp + v[k], L + 1);
+                else far_push(a, st, v[k]);
+                ss_min_done(a.dist + v[k], nd[k]);
+            }
+        }
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+            const bool has = stamp[k] != L + 1 && re[k] > rb[k];
+            if (has) {
+                asm volatile("prefetch.global.L2 [%0];" ::"l"(a.col + rb[k]));
+                asm volatile("prefetch.global.L2 [%0];" ::"l"(a.w + rb[k]));
+            }
+            ss_list_append(a, sh, L + 1, tag + 1, has, v[k], (uint32_t)rb[k], (uint32_t)(re[k] - rb[k]));
+        }
+    }
+}
+
+// Whether round st goes on lists (half the limit to come in, the limit to stay).
+template <typename OffT>
+__device__ __forceinline__ bool list_may_start(const SsspArgs<OffT> &a, const SsState &st) {
+    return a.lines && st.op == SOP_RELAX && !st.bmp && !st.nolist && st.T <= a.list_T * gridDim.x / 2;
+}
+
+// Runs rounds from s_st on lists while they fit; s_st is then the next phase of
+// the other kind, with its queue.  Every block calls.  false: a wait gave up.
+template <typename OffT, bool STATS>
+__device__ __forceinline__ bool list_rounds(const SsspArgs<OffT> &a, SsState &s_st, NarrowShared<SS_LIST_BLOCKS> &sh,
+                                            FlagBarrier &bar) {
+    const int group = (int)gridDim.x;
+    const unsigned int lane = threadIdx.x & 31;
+    // no tag of this stretch was used before: every stretch counts up the epoch
+    unsigned long long tag = (unsigned long long)(ld_relaxed_u32(&a.ctl->narrow_epoch) & 0x7fffffffu) << 32;
+    if (threadIdx.x == 0) {
+        sh.got = 0ull;
+        sh.got_edges = 0ull;
+    }
+    __syncthreads();
+    {   // Q_L into the segments
+        const int L = s_st.L;
+        const uint32_t q = s_st.q;
+        const int32_t *Q = pick3(a.Q[0], a.Q[1], a.Q[2], L % 3);
+        const OffT *R = pick3(a.R[0], a.R[1], a.R[2], L % 3);
+        const uint32_t i0 = (uint32_t)((uint64_t)q * blockIdx.x / gridDim.x);
+        const uint32_t i1 = (uint32_t)((uint64_t)q * (blockIdx.x + 1) / gridDim.x);
+        for (uint32_t base = i0 + (threadIdx.x & ~31u); base < i1; base += SS_BLOCK) {
+            const uint32_t i = base + lane;
+            int32_t v = 0;
+            OffT row = 0;
+            uint32_t deg = 0;
+            if (i < i1) {
+                v = __ldcg(Q + i);
+                row = __ldcg(R + i);
+                deg = (uint32_t)(__ldg(a.ro + v + 1) - row);
+            }
+            ss_list_append(a, sh, L, tag + 1, i < i1, v, (uint32_t)row, deg);
+        }
+    }
+    ++tag;
+    if (!narrow_exchange_wide<SS_BLOCK>(a.lines + (tag & 1) * SS_LIST_BLOCKS, sh, group, tag, a.ctl, a.timeout_ns)) return false;
+    for (;;) {
+        if (s_st.q == 0 || s_st.T > a.list_T * gridDim.x || sh.most > ss_list_pieces(a.list_T)) break;
+        const int L = s_st.L;
+        if (STATS && blockIdx.x == 0 && threadIdx.x == 0 && L < GRX_MAX_LEVELS_STATS) {
+            a.stats->level_t0[L] = grx_globaltimer();
+            a.stats->dir[L] = 0;
+            a.stats->frontier[L] = s_st.q;
+            a.stats->edges_examined[L] = s_st.T;
+            a.stats->vertices_scanned[L] = s_st.q;
+            a.stats->discovered[L] = 0;
+            a.stats->levels = L + 1;
+        }
+        list_round(a, s_st, sh, tag);
+        ++tag;
+        if (!narrow_exchange_wide<SS_BLOCK>(a.lines + (tag & 1) * SS_LIST_BLOCKS, sh, group, tag, a.ctl, a.timeout_ns))
+            return false;
+        if (threadIdx.x == 0) {
+            s_st.L = L + 1;
+            s_st.q = sh.verts;
+            s_st.T = sh.edges;
+            if (STATS && blockIdx.x == 0 && L < GRX_MAX_LEVELS_STATS) a.stats->discovered[L] = sh.verts;
+        }
+        __syncthreads();
+    }
+    const int L = s_st.L;
+    if (s_st.q) {                                // back to a queue: vertex, edge prefix, row start
+        uint32_t x0, x1, x2, vb, eb, x3;         // vertices and edges of the blocks before
+        {
+            uint32_t sv = 0, se = 0;
+            for (uint32_t b = threadIdx.x; b < blockIdx.x; b += SS_BLOCK) {
+                sv += sh.line_verts[b];
+                se += sh.line_edges[b];
+            }
+            block_scan3<SS_BLOCK>(sv, se, 0u, x0, x1, x2, vb, eb, x3);
+        }
+        int32_t *Q = pick3(a.Q[0], a.Q[1], a.Q[2], L % 3);
+        uint32_t *E = pick3(a.E[0], a.E[1], a.E[2], L % 3);
+        OffT *R = pick3(a.R[0], a.R[1], a.R[2], L % 3);
+        const int32_t *mine = a.verts + ((size_t)(L & 1) * gridDim.x + blockIdx.x) * ss_list_verts(a.list_T);
+        const uint32_t n = sh.own;
+        for (uint32_t base = 0; base < n; base += SS_BLOCK) {
+            const uint32_t i = base + threadIdx.x;
+            int32_t v = 0;
+            OffT rb = 0;
+            uint32_t deg = 0;
+            if (i < n) {
+                v = __ldcg(mine + i);
+                rb = __ldg(a.ro + v);
+                deg = (uint32_t)(__ldg(a.ro + v + 1) - rb);
+            }
+            uint32_t e0, esum, t1, t2;
+            block_scan3<SS_BLOCK>(deg, 0u, 0u, e0, x1, x2, esum, t1, t2);
+            if (i < n) {
+                Q[vb + i] = v;
+                E[vb + i] = eb + e0;
+                R[vb + i] = rb;
+            }
+            eb += esum;
+        }
+    }
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        a.ctl->narrow_epoch += 1;                // no block reads it before the barrier below
+        for (int i = 0; i < 4; ++i) a.ctl->qpack[i] = 0ull;
+    }
+    if (!flag_barrier(bar)) return false;
+    if (threadIdx.x == 0) {
+        if (s_st.q) {
+            s_st.nolist = 1;                     // the round it stopped at may look small (one long row)
+            ss_set_kind(a, s_st);
+        } else {
+            s_st.nfar = ld_relaxed_u32(&a.ctl->farcnt[s_st.fsel]);
+            if (a.delta && s_st.nfar > 0) s_st.op = SOP_FARMIN;
+            else s_st.done = 1;
+        }
+    }
+    __syncthreads();
+    return true;
+}
+
 // State of the next phase.
 template <typename OffT>
 __device__ SsState ss_next(const SsspArgs<OffT> &a, const SsState &st, bool stats) {
     SsState ns = st;
+    ns.nolist = 0;
     if (st.op == SOP_RELAX && st.bmp) {
         ns.op = SOP_FINAL;
         return ns;
@@ -373,11 +615,20 @@ __device__ SsState ss_next(const SsspArgs<OffT> &a, const SsState &st, bool stat
     return ns;
 }
 
-template <typename OffT, bool STATS>
-__global__ void __launch_bounds__(SS_BLOCK, GRX_SS_MIN_BLOCKS) k_sssp_persistent(SsspArgs<OffT> a) {
+// Shared memory of a block: list rounds and the others do not overlap.
+template <typename OffT>
+union SsSmem {
+    SsWarpSmem<OffT> w[SS_WARPS];
+    NarrowShared<SS_LIST_BLOCKS> list;
+};
+
+// LIST (list rounds) is a variant of its own: other graphs keep their registers.
+template <typename OffT, bool STATS, bool LIST>
+__global__ void __launch_bounds__(SS_BLOCK, SS_MIN_BLOCKS) k_sssp_persistent(const __grid_constant__ SsspArgs<OffT> a) {
     __shared__ SsState s_st;
-    __shared__ SsWarpSmem<OffT> wsm[SS_WARPS];
-    SsWarpSmem<OffT> &w = wsm[threadIdx.x >> 5];
+    extern __shared__ __align__(16) unsigned char ss_dsmem[];
+    SsSmem<OffT> &sm = *reinterpret_cast<SsSmem<OffT> *>(ss_dsmem);
+    SsWarpSmem<OffT> &w = sm.w[threadIdx.x >> 5];
     FlagBarrier bar{a.bar_flags, &a.ctl->bar_release, a.ctl, a.timeout_ns, 0u};
     if (threadIdx.x == 0) {
         SsState s;
@@ -393,28 +644,33 @@ __global__ void __launch_bounds__(SS_BLOCK, GRX_SS_MIN_BLOCKS) k_sssp_persistent
     }
     __syncthreads();
     for (;;) {
-        const SsState st = s_st;
-        if (st.done) break;
-        const int L = st.L;
-        if (st.op == SOP_RELAX && blockIdx.x == 0 && threadIdx.x == 0) {
-            a.ctl->qpack[(L + 2) & 3] = 0ull;
-            if (STATS && L < GRX_MAX_LEVELS_STATS) {
-                a.stats->level_t0[L] = grx_globaltimer();
-                a.stats->dir[L] = 0;
-                a.stats->frontier[L] = st.q;
-                a.stats->edges_examined[L] = st.T;
-                a.stats->vertices_scanned[L] = st.q;
-                a.stats->levels = L + 1;
+        for (;;) {
+            const SsState &st = s_st;
+            if (st.done || (LIST && list_may_start(a, st))) break;
+            const int L = st.L;
+            if (st.op == SOP_RELAX && blockIdx.x == 0 && threadIdx.x == 0) {
+                a.ctl->qpack[(L + 2) & 3] = 0ull;
+                if (STATS && L < GRX_MAX_LEVELS_STATS) {
+                    a.stats->level_t0[L] = grx_globaltimer();
+                    a.stats->dir[L] = 0;
+                    a.stats->frontier[L] = st.q;
+                    a.stats->edges_examined[L] = st.T;
+                    a.stats->vertices_scanned[L] = st.q;
+                    a.stats->levels = L + 1;
+                }
             }
+            if (st.op == SOP_FINAL) changed_to_queue<OffT>(a, st, w.list);
+            else if (st.op == SOP_FARMIN) far_min<OffT>(a, st);
+            else if (st.op == SOP_FARSPLIT) far_split<OffT>(a, st);
+            else if (st.bmp) relax_round<OffT, true>(a, st, w);
+            else relax_round<OffT, false>(a, st, w);
+            if (!flag_barrier(bar)) return;
+            if (threadIdx.x == 0) s_st = ss_next(a, st, STATS);
+            __syncthreads();
         }
-        if (st.op == SOP_FINAL) changed_to_queue<OffT>(a, st, w.list);
-        else if (st.op == SOP_FARMIN) far_min<OffT>(a, st);
-        else if (st.op == SOP_FARSPLIT) far_split<OffT>(a, st);
-        else if (st.bmp) relax_round<OffT, true>(a, st, w);
-        else relax_round<OffT, false>(a, st, w);
-        if (!flag_barrier(bar)) return;
-        if (threadIdx.x == 0) s_st = ss_next(a, st, STATS);
-        __syncthreads();
+        if (!LIST || s_st.done) break;
+        if constexpr (LIST)
+            if (!list_rounds<OffT, STATS>(a, s_st, sm.list, bar)) return;
     }
     if (blockIdx.x == 0 && threadIdx.x == 0) {
         a.ctl->levels_run = s_st.L;
@@ -437,7 +693,73 @@ __global__ void k_sssp_init(int32_t src, const OffT *ro, uint32_t *dist, int32_t
     ctl->farcnt[1] = 0u;
     ctl->farmin[0] = 0xffffffffu;
     ctl->farmin[1] = 0xffffffffu;
+    ctl->narrow_epoch += 1;                  // as does every stretch of list rounds: a call that gave up left its tags
     if (stats_on) stats->levels = 0;
+}
+
+// The list rounds' buffers of g for grids of up to `blocks` (once; NULL without
+// memory, or while s is captured: the rounds then run on the queue).
+grx_status ss_list_buffers(grx_graph *g, int blocks, cudaStream_t s) {
+    if (g->ss_lines || blocks > SS_BLOCK) return GRX_OK;
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(s, &cap) != cudaSuccess) {
+        cudaGetLastError();
+        return GRX_OK;
+    }
+    if (cap != cudaStreamCaptureStatusNone) return GRX_OK;
+    // rounds of up to 3,072 edges a block, a quarter of the graph's at most
+    const int64_t share = g->ne / 4 / blocks;
+    const uint32_t t = (uint32_t)(share < 192 ? 192 : (share > 3072 ? 3072 : share));
+    const size_t lines = 2 * SS_LIST_BLOCKS * sizeof(NarrowWord);
+    const size_t pieces = 2 * (size_t)blocks * ss_list_pieces(t) * sizeof(NarrowWord);
+    const size_t verts = 2 * (size_t)blocks * ss_list_verts(t) * sizeof(int32_t);
+    char *p = (char *)grx_alloc(g, lines + pieces + verts, s);
+    if (!p) return GRX_OK;
+    GRX_CUDA(cudaMemsetAsync(p, 0, lines + pieces, s));           // tag 0 is never used
+    g->ss_lines = p;
+    g->ss_list_T = t;
+    g->ss_list_blocks = blocks;
+    return GRX_OK;
+}
+
+template <typename OffT, bool STATS, bool LIST>
+grx_status launch_persistent(grx_graph *g, SsspArgs<OffT> &a, int32_t src, uint32_t *dist, const grx_opts *o,
+                             cudaStream_t s) {
+    k_sssp_init<OffT><<<1, 1, 0, s>>>(src, a.ro, dist, g->qv[0], g->qe[0], a.R[0], g->ctl, g->stats,
+                                      o->collect_stats);
+    GRX_CUDA(cudaGetLastError());
+    constexpr int smem = (int)sizeof(SsSmem<OffT>);
+    static int per_sm = -1;
+    if (per_sm < 0) {
+        GRX_CUDA(cudaFuncSetAttribute((const void *)k_sssp_persistent<OffT, STATS, LIST>,
+                                      cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+        GRX_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_sssp_persistent<OffT, STATS, LIST>,
+                                                               SS_BLOCK, smem));
+        if (per_sm < 1) return grx_fail(GRX_ECUDA, "sssp: persistent kernel does not fit on an SM");
+    }
+    int max_grid = per_sm * g->ctx->num_sms;
+    if (max_grid > GRX_MAX_GRID) max_grid = GRX_MAX_GRID;
+    const int blocks = grx_grid(o, SS_BLOCK, max_grid);
+    if (LIST) {
+        const grx_status st = ss_list_buffers(g, max_grid, s);
+        if (st != GRX_OK) return st;
+        if (g->ss_lines && blocks <= g->ss_list_blocks) {
+            const uint32_t t = g->ss_list_T;
+            a.lines = (NarrowWord *)g->ss_lines;
+            a.pieces = a.lines + 2 * SS_LIST_BLOCKS;
+            a.verts = (int32_t *)(a.pieces + 2 * (size_t)g->ss_list_blocks * ss_list_pieces(t));
+            a.list_T = t;
+            if (o->push_bitmap == 0.f && a.bmp_min_T <= t * (uint32_t)blocks) a.bmp_min_T = t * (uint32_t)blocks + 1;
+        }
+    }
+    GRX_CUDA(cudaMemsetAsync(g->bar_flags, 0, sizeof(unsigned int) * (size_t)blocks, s));
+    GRX_CUDA(cudaMemsetAsync(&g->ctl->bar_release, 0, sizeof(unsigned int), s));
+    void *args[] = {(void *)&a};
+    if (o->ev_begin) GRX_CUDA(cudaEventRecord((cudaEvent_t)o->ev_begin, s));
+    GRX_CUDA(cudaLaunchCooperativeKernel((const void *)k_sssp_persistent<OffT, STATS, LIST>, dim3(blocks),
+                                         dim3(SS_BLOCK), args, smem, s));
+    if (o->ev_end) GRX_CUDA(cudaEventRecord((cudaEvent_t)o->ev_end, s));
+    return GRX_OK;
 }
 
 template <typename OffT, bool STATS>
@@ -466,31 +788,19 @@ grx_status launch_typed(grx_graph *g, int32_t src, uint32_t *dist, const grx_opt
     a.stats = g->stats;
     a.timeout_ns = grx_timeout_ns(o);
     a.src = src;
+    a.lines = a.pieces = nullptr;
+    a.verts = nullptr;
+    a.list_T = 0;
     {   // reduction rounds when a round's edges reach push_bitmap * nv (0 = 1/8, < 0 = never)
         const double pb = o->push_bitmap == 0.f ? 0.125 : (double)o->push_bitmap;
         const double t = pb * (double)g->nv;
         a.bmp_min_T = pb < 0 ? 0xffffffffu : (t < 1.0 ? 1u : (t > 4294967295.0 ? 0xffffffffu : (uint32_t)t));
     }
-    k_sssp_init<OffT><<<1, 1, 0, s>>>(src, a.ro, dist, g->qv[0], g->qe[0], a.R[0], g->ctl, g->stats,
-                                      o->collect_stats);
-    GRX_CUDA(cudaGetLastError());
-    static int per_sm = -1;
-    if (per_sm < 0) {
-        GRX_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_sssp_persistent<OffT, STATS>,
-                                                               SS_BLOCK, 0));
-        if (per_sm < 1) return grx_fail(GRX_ECUDA, "sssp: persistent kernel does not fit on an SM");
-    }
-    int max_grid = per_sm * g->ctx->num_sms;
-    if (max_grid > GRX_MAX_GRID) max_grid = GRX_MAX_GRID;
-    int blocks = o->grid_blocks > 0 && o->grid_blocks < max_grid ? o->grid_blocks : max_grid;
-    GRX_CUDA(cudaMemsetAsync(g->bar_flags, 0, sizeof(unsigned int) * (size_t)blocks, s));
-    GRX_CUDA(cudaMemsetAsync(&g->ctl->bar_release, 0, sizeof(unsigned int), s));
-    void *args[] = {(void *)&a};
-    if (o->ev_begin) GRX_CUDA(cudaEventRecord((cudaEvent_t)o->ev_begin, s));
-    GRX_CUDA(cudaLaunchCooperativeKernel((const void *)k_sssp_persistent<OffT, STATS>, dim3(blocks),
-                                         dim3(SS_BLOCK), args, 0, s));
-    if (o->ev_end) GRX_CUDA(cudaEventRecord((cudaEvent_t)o->ev_end, s));
-    return GRX_OK;
+    // List rounds on graphs of few edges a vertex (see narrow levels of bfs.cu);
+    // only where they are the better form of a large round too: lists up to the
+    // limit, the changed bitmap past it, unless the caller set the line.
+    return g->ne < 8ll * g->nv ? launch_persistent<OffT, STATS, true>(g, a, src, dist, o, s)
+                               : launch_persistent<OffT, STATS, false>(g, a, src, dist, o, s);
 }
 
 }  // namespace

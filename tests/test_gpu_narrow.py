@@ -71,6 +71,21 @@ def _weighted(g, wmax, seed):
     return inputs.Graph(g.name, g.row_offsets, g.col_indices, w)
 
 
+@pytest.mark.parametrize("name", list(GRAPHS))
+@pytest.mark.parametrize("off64", [False, True])
+@pytest.mark.parametrize("wmax", [1, 300])
+def test_sssp_through_list_rounds(grx, name, off64, wmax):
+    g = _weighted(GRAPHS[name](), wmax, 7)
+    dg = grx.load(g, offsets64=off64)
+    for src in (0, g.nv // 2, int(inputs.pick_sources(g.row_offsets, 1, seed=3)[0])):
+        want = oracle.sssp(g.row_offsets, g.col_indices, g.weights, src)
+        for delta in (0, 1, 150, 5000):
+            for kw in ({}, {"grid_blocks": 1}, {"grid_blocks": 5}, {"push_bitmap": 0.001}):
+                d = grx.sssp(dg, src, opts=grx.opts(sssp_delta=delta, **kw))
+                grx.graph_status(dg)
+                assert np.array_equal(grx.as_uint32(d), want), (name, src, delta, kw)
+
+
 def test_a_new_graph_in_the_memory_of_a_freed_one(grx):
     """Words left by a freed graph's traversals are not taken for the new one's."""
     for k in range(4):
