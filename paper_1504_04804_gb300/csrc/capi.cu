@@ -53,8 +53,13 @@ void grx_ctx_free(grx_ctx *c, void *p, size_t bytes, cudaStream_t s) {
 void *grx_alloc(grx_graph *g, size_t bytes, cudaStream_t s) {
     if (g->nallocs >= (int)(sizeof g->allocs / sizeof g->allocs[0])) return nullptr;
     void *p = grx_ctx_alloc(g->ctx, bytes, s);
+    if (p && ((uintptr_t)p & 15)) {              // 16-byte loads; CUDA's own allocators align to 256
+        grx_ctx_free(g->ctx, p, bytes, s);
+        bytes += 16;
+        p = grx_ctx_alloc(g->ctx, bytes, s);
+    }
     if (p) g->allocs[g->nallocs++] = {p, bytes};
-    return p;
+    return p ? (void *)(((uintptr_t)p + 15) & ~(uintptr_t)15) : nullptr;
 }
 
 // ---------------------------------------------------------------------------

@@ -2,13 +2,13 @@
 // min combiner of Sec. 3, per lane).
 //
 //  * Distances live vertex-major inside the library, D[v][lane] (64 uint32
-//    per vertex), so a warp relaxes one edge (u, v, w) for 32 lanes at once
-//    with coalesced 128-byte reads of D[u][*] and D[v][*]; lanes that improve
-//    use atomicMin on their own word.  The output is transposed to the
+//    per vertex), so a few threads relax an edge (u, v, w) for all lanes with
+//    16-byte reads of D[u][*] and D[v][*]; lanes that improve use atomicMin on
+//    their own word.  The output is transposed to the
 //    caller's lane-major layout at the end.
 //  * A vertex's "changed" mask lists the lanes whose distance improved in the
 //    last round; only those lanes relax its edges.  A warp stages a tile's 64
-//    edges in shared memory (coalesced) and relaxes 8 of them at a time, all
+//    edges in shared memory (coalesced) and relaxes a few at a time, all
 //    their distance loads in flight.  Improved lanes are OR-ed into next[v]
 //    (one atomic per warp and edge); the first toucher lists v -- or, in
 //    rounds with at least push_bitmap * V edges, the min and the OR are
@@ -25,7 +25,6 @@ namespace {
 constexpr int MP_BLOCK = 256;
 constexpr int MP_WARPS = MP_BLOCK / 32;
 constexpr int MP_WTILE = 64;                 // edges per warp tile
-constexpr int MP_UNROLL = 8;                 // edges relaxed together by a warp
 
 template <typename OffT>
 struct MpArgs {
@@ -111,146 +110,84 @@ __device__ void mp_seed(const MpArgs<OffT> &a) {
 
 namespace {
 
-// Relaxes a staged tile of `len` edges for every lane of the batch: one edge
-// at a time across the warp, thread = lane b (and b + 32 with two halves).
-// Improved lanes go to next[v] (and the touched bitmap in reduction rounds,
-// or the tile's touched list tbuf / nt otherwise).
-template <typename OffT>
+// Relaxes a staged tile of `len` edges for the batch's lanes.  TPE threads take an
+// edge, four lanes each: one 16-byte load of D[u] and one of D[v] where a thread
+// per lane would take eight, so a warp instruction serves 32 / TPE edges.  Improved
+// lanes go to next[v] (and the touched bitmap in reduction rounds, or the tile's
+// touched list tbuf / nt otherwise).  Lanes that do not take part, because the
+// edge's source did not improve there, have mask bit 0.
+// (It is issue-bound: with a thread per lane, R-MAT 20 took 7.1 / 14.9 / 23.9 ms for
+// 16 / 32 / 64 sources, now 4.2 / 6.6 / 12.5; two edges in flight instead of four
+// 4.6 / 7.2 / 13.7.)
+template <typename OffT, int TPE>
 __device__ __forceinline__ void relax_lanes(const MpArgs<OffT> &a, MpWarpSmem<OffT> &w, int len, bool bmp,
-                                            int32_t *tbuf, int &nt, int halves) {
+                                            int32_t *tbuf, int &nt) {
+    constexpr int EPW = 32 / TPE;                 // edges per warp instruction
+    constexpr int UN = 4;                         // edges a thread has in flight
     const unsigned int lane = threadIdx.x & 31;
-        for (int eb = 0; eb < len; eb += MP_UNROLL) {
-        int32_t vv[MP_UNROLL], uu[MP_UNROLL];
-        uint32_t ww[MP_UNROLL];
-        unsigned long long mm[MP_UNROLL];
+    const int gi = (int)lane / TPE;               // the thread's edge within a step
+    const int b0 = ((int)lane % TPE) * 4;         // its first SSSP lane
+    for (int eb = 0; eb < len; eb += UN * EPW) {
+        int32_t vv[UN];
+        uint32_t ww[UN], act[UN];
+        uint4 du[UN], dv[UN];
 #pragma unroll
-        for (int k = 0; k < MP_UNROLL; ++k) {
-            const bool ok = eb + k < len;
-            const int j = ok ? w.er[eb + k] : 0;
-            vv[k] = ok ? w.ev[eb + k] : 0;
-            ww[k] = ok ? w.ew[eb + k] : 0u;
-            uu[k] = ok ? w.u[j] : 0;
-            mm[k] = ok ? w.cm[j] : 0ull;
-        }
-        unsigned long long imp[MP_UNROLL];
-#pragma unroll
-        for (int k = 0; k < MP_UNROLL; ++k) imp[k] = 0ull;
-        for (int h = 0; h < halves; ++h) {
-            const int b = (int)lane + 32 * h;
-            uint32_t du[MP_UNROLL], dv[MP_UNROLL];
-#pragma unroll
-            for (int k = 0; k < MP_UNROLL; ++k) {
-                const bool act = (mm[k] >> b) & 1ull;
-                du[k] = act ? __ldcg(a.D + (int64_t)uu[k] * 64 + b) : 0xffffffffu;
-                dv[k] = act ? __ldcg(a.D + (int64_t)vv[k] * 64 + b) : 0u;
-            }
-#pragma unroll
-            for (int k = 0; k < MP_UNROLL; ++k) {
-                bool improved = false;
-                if (du[k] != 0xffffffffu) {
-                    const uint64_t nd = (uint64_t)du[k] + ww[k];
-                    if (nd >= 0xffffffffull) {
-                        grx_set_status(a.ctl, GRX_ERANGE);
-                    } else if ((uint32_t)nd < dv[k]) {
-                        if (bmp) {
-                            // a reduction: the lane improves in this round,
-                            // by this proposal or a smaller one
-                            atomicMin(a.D + (int64_t)vv[k] * 64 + b, (uint32_t)nd);
-                            improved = true;
-                        } else {
-                            const uint32_t old = atomicMin(a.D + (int64_t)vv[k] * 64 + b, (uint32_t)nd);
-                            improved = (uint32_t)nd < old;
-                        }
-                    }
-                }
-                imp[k] |= (unsigned long long)__ballot_sync(GRX_FULL_MASK, improved) << (32 * h);
-            }
-        }
-        if (bmp) {
-#pragma unroll
-            for (int k = 0; k < MP_UNROLL; ++k) {
-                if (lane == (unsigned)k && imp[k]) {
-                    atomicOr(a.next + vv[k], imp[k]);                // results unused: reductions
-                    atomicOr(a.tbits + (vv[k] >> 5), 1u << (vv[k] & 31));
-                }
-            }
-        } else {
-#pragma unroll
-            for (int k = 0; k < MP_UNROLL; ++k) {
-                bool first = false;
-                if (lane == (unsigned)k && imp[k]) first = atomicOr(a.next + vv[k], imp[k]) == 0ull;
-                const unsigned int fm = __ballot_sync(GRX_FULL_MASK, first);
-                if (first) tbuf[nt + __popc(fm & lanemask_lt())] = vv[k];
-                nt += __popc(fm);
-            }
-        }
-    }
-}
-
-// The same for batches of at most G lanes (G = 8 or 16): the warp splits into
-// 32 / G groups and each group relaxes its own edge, thread = lane b of its
-// group's edge, so one warp instruction serves 32 / G edges.
-template <typename OffT, int G>
-__device__ __forceinline__ void relax_groups(const MpArgs<OffT> &a, MpWarpSmem<OffT> &w, int len, bool bmp,
-                                             int32_t *tbuf, int &nt) {
-    static_assert(G == 8 || G == 16, "lane groups of 8 or 16");
-    constexpr int EPW = 32 / G;                   // edges per warp instruction
-    const unsigned int lane = threadIdx.x & 31;
-    const int gi = (int)lane / G;                 // the thread's edge within a step
-    const int b = (int)lane % G;                  // its SSSP lane
-    const unsigned int gmask = (1u << G) - 1u;
-    for (int eb = 0; eb < len; eb += MP_UNROLL * EPW) {
-        int32_t vv[MP_UNROLL], uu[MP_UNROLL];
-        uint32_t ww[MP_UNROLL];
-        bool act[MP_UNROLL];
-#pragma unroll
-        for (int k = 0; k < MP_UNROLL; ++k) {
+        for (int k = 0; k < UN; ++k) {
             const int e = eb + k * EPW + gi;
             const bool ok = e < len;
             const int j = ok ? w.er[e] : 0;
             vv[k] = ok ? w.ev[e] : 0;
             ww[k] = ok ? w.ew[e] : 0u;
-            uu[k] = ok ? w.u[j] : 0;
-            act[k] = ok && ((w.cm[j] >> b) & 1ull);
+            act[k] = ok ? (uint32_t)(w.cm[j] >> b0) & 15u : 0u;
+            du[k] = make_uint4(0xffffffffu, 0xffffffffu, 0xffffffffu, 0xffffffffu);
+            dv[k] = make_uint4(0u, 0u, 0u, 0u);
+            if (act[k]) {
+                du[k] = __ldcg(reinterpret_cast<const uint4 *>(a.D + (int64_t)w.u[j] * 64 + b0));
+                dv[k] = __ldcg(reinterpret_cast<const uint4 *>(a.D + (int64_t)vv[k] * 64 + b0));
+            }
         }
-        uint32_t du[MP_UNROLL], dv[MP_UNROLL];
 #pragma unroll
-        for (int k = 0; k < MP_UNROLL; ++k) {
-            du[k] = act[k] ? __ldcg(a.D + (int64_t)uu[k] * 64 + b) : 0xffffffffu;
-            dv[k] = act[k] ? __ldcg(a.D + (int64_t)vv[k] * 64 + b) : 0u;
-        }
+        for (int k = 0; k < UN; ++k) {
+            const uint32_t us[4] = {du[k].x, du[k].y, du[k].z, du[k].w};
+            const uint32_t vs[4] = {dv[k].x, dv[k].y, dv[k].z, dv[k].w};
+            uint32_t imp = 0;
 #pragma unroll
-        for (int k = 0; k < MP_UNROLL; ++k) {
-            bool improved = false;
-            if (du[k] != 0xffffffffu) {
-                const uint64_t nd = (uint64_t)du[k] + ww[k];
+            for (int i = 0; i < 4; ++i) {
+                if (!(act[k] >> i & 1u) || us[i] == 0xffffffffu) continue;
+                const uint64_t nd = (uint64_t)us[i] + ww[k];
                 if (nd >= 0xffffffffull) {
                     grx_set_status(a.ctl, GRX_ERANGE);
-                } else if ((uint32_t)nd < dv[k]) {
+                } else if ((uint32_t)nd < vs[i]) {
+                    uint32_t *p = a.D + (int64_t)vv[k] * 64 + b0 + i;
                     if (bmp) {
-                        atomicMin(a.D + (int64_t)vv[k] * 64 + b, (uint32_t)nd);
-                        improved = true;
-                    } else {
-                        const uint32_t old = atomicMin(a.D + (int64_t)vv[k] * 64 + b, (uint32_t)nd);
-                        improved = (uint32_t)nd < old;
+                        // a reduction: the lane improves in this round, by this
+                        // proposal or a smaller one
+                        atomicMin(p, (uint32_t)nd);
+                        imp |= 1u << i;
+                    } else if ((uint32_t)nd < atomicMin(p, (uint32_t)nd)) {
+                        imp |= 1u << i;
                     }
                 }
             }
-            // the group's improved lanes; its first thread publishes them
-            const unsigned int imp = (__ballot_sync(GRX_FULL_MASK, improved) >> (gi * G)) & gmask;
-            bool first = false;
-            if (b == 0 && imp) {
-                if (bmp) {
-                    atomicOr(a.next + vv[k], (unsigned long long)imp);        // results unused: reductions
-                    atomicOr(a.tbits + (vv[k] >> 5), 1u << (vv[k] & 31));
-                } else {
-                    first = atomicOr(a.next + vv[k], (unsigned long long)imp) == 0ull;
+            // the edge's improved lanes; its first thread publishes them
+            unsigned long long m = (unsigned long long)imp << b0;
+            if (__any_sync(GRX_FULL_MASK, imp != 0u)) {
+#pragma unroll
+                for (int o = TPE / 2; o > 0; o >>= 1) m |= __shfl_xor_sync(GRX_FULL_MASK, m, o);
+                bool first = false;
+                if (b0 == 0 && m) {
+                    if (bmp) {
+                        atomicOr(a.next + vv[k], m);                     // results unused: reductions
+                        atomicOr(a.tbits + (vv[k] >> 5), 1u << (vv[k] & 31));
+                    } else {
+                        first = atomicOr(a.next + vv[k], m) == 0ull;
+                    }
                 }
-            }
-            if (!bmp) {
-                const unsigned int fm = __ballot_sync(GRX_FULL_MASK, first);
-                if (first) tbuf[nt + __popc(fm & lanemask_lt())] = vv[k];
-                nt += __popc(fm);
+                if (!bmp) {
+                    const unsigned int fm = __ballot_sync(GRX_FULL_MASK, first);
+                    if (first) tbuf[nt + __popc(fm & lanemask_lt())] = vv[k];
+                    nt += __popc(fm);
+                }
             }
         }
     }
@@ -272,7 +209,6 @@ __device__ void mp_expand(const MpArgs<OffT> &a, int L, uint32_t q, uint64_t T, 
     const uint64_t tb0 = gw * per;
     const uint64_t tb1 = min(ntiles, tb0 + per);
     if (tb0 >= tb1) return;
-    const int halves = a.n > 32 ? 2 : 1;
     int64_t i0 = warp_upper_index_cg(Qe, (int64_t)q, (uint32_t)(tb0 * MP_WTILE));
     for (uint64_t tile = tb0; tile < tb1; ++tile) {
         const uint64_t e0 = tile * MP_WTILE;
@@ -316,9 +252,10 @@ __device__ void mp_expand(const MpArgs<OffT> &a, int L, uint32_t q, uint64_t T, 
         __syncwarp();
         const int len = (int)(e1 - (uint32_t)e0);
         int nt = 0;                                   // touched vertices of this tile (list rounds)
-        if (a.n <= 8) relax_groups<OffT, 8>(a, w, len, bmp, tbuf, nt);
-        else if (a.n <= 16) relax_groups<OffT, 16>(a, w, len, bmp, tbuf, nt);
-        else relax_lanes<OffT>(a, w, len, bmp, tbuf, nt, halves);
+        if (a.n <= 8) relax_lanes<OffT, 2>(a, w, len, bmp, tbuf, nt);
+        else if (a.n <= 16) relax_lanes<OffT, 4>(a, w, len, bmp, tbuf, nt);
+        else if (a.n <= 32) relax_lanes<OffT, 8>(a, w, len, bmp, tbuf, nt);
+        else relax_lanes<OffT, 16>(a, w, len, bmp, tbuf, nt);
         __syncwarp();
         // one append of the tile's touched vertices
         unsigned int base = 0;
