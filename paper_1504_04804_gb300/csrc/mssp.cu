@@ -25,6 +25,7 @@ namespace {
 constexpr int MP_BLOCK = 256;
 constexpr int MP_WARPS = MP_BLOCK / 32;
 constexpr int MP_WTILE = 64;                 // edges per warp tile
+constexpr int MP_BATCH = 4;                  // tiles a warp takes at a time
 
 template <typename OffT>
 struct MpArgs {
@@ -69,10 +70,11 @@ template <typename OffT>
 __device__ void mp_init_fill(const MpArgs<OffT> &a) {
     const int64_t tid = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    // only the batch's lanes (rounded up to a 32-byte sector) are ever read
-    const int nl = (a.n + 7) & ~7;
-    const int64_t total = (int64_t)a.nv * nl;
-    for (int64_t i = tid; i < total; i += stride) a.D[(i / nl) * 64 + (i % nl)] = 0xffffffffu;
+    // only the batch's lanes (8, 16, 32 or 64) are ever read
+    const int quads = a.n <= 8 ? 1 : (a.n <= 16 ? 2 : (a.n <= 32 ? 3 : 4));   // log2 of their 16-byte words
+    const uint4 far = make_uint4(0xffffffffu, 0xffffffffu, 0xffffffffu, 0xffffffffu);
+    for (int64_t i = tid; i < (int64_t)a.nv << quads; i += stride)
+        reinterpret_cast<uint4 *>(a.D)[(i >> quads) * 16 + (i & ((1 << quads) - 1))] = far;
     for (int64_t v = tid; v < a.nv; v += stride) {
         a.next[v] = 0ull;
         a.cur[0][v] = 0ull;
@@ -104,6 +106,7 @@ __device__ void mp_seed(const MpArgs<OffT> &a) {
     a.ctl->qpack[0] = ((unsigned long long)cnt << 32) | edges;
     for (int i = 1; i < 4; ++i) a.ctl->qpack[i] = 0ull;
     for (int i = 0; i < 4; ++i) a.ctl->ucount[i] = 0u;
+    for (int i = 0; i < 4; ++i) a.ctl->wq[i] = 0u;
 }
 
 }  // namespace
@@ -117,11 +120,11 @@ namespace {
 // touched list tbuf / nt otherwise).  Lanes that do not take part, because the
 // edge's source did not improve there, have mask bit 0.
 // (It is issue-bound: with a thread per lane, R-MAT 20 took 7.1 / 14.9 / 23.9 ms for
-// 16 / 32 / 64 sources, now 4.2 / 6.6 / 12.5; two edges in flight instead of four
-// 4.6 / 7.2 / 13.7.)
-template <typename OffT, int TPE>
-__device__ __forceinline__ void relax_lanes(const MpArgs<OffT> &a, MpWarpSmem<OffT> &w, int len, bool bmp,
-                                            int32_t *tbuf, int &nt) {
+// 16 / 32 / 64 sources, now 3.5 / 5.3 / 9.6; two edges in flight instead of four
+// cost 10 % more.  Reading D[u] through L1 changes nothing.)
+template <typename OffT, int TPE, bool BMP>
+__device__ __forceinline__ void relax_lanes(const MpArgs<OffT> &a, MpWarpSmem<OffT> &w, int len, int32_t *tbuf,
+                                            int &nt) {
     constexpr int EPW = 32 / TPE;                 // edges per warp instruction
     constexpr int UN = 4;                         // edges a thread has in flight
     const unsigned int lane = threadIdx.x & 31;
@@ -150,25 +153,26 @@ __device__ __forceinline__ void relax_lanes(const MpArgs<OffT> &a, MpWarpSmem<Of
         for (int k = 0; k < UN; ++k) {
             const uint32_t us[4] = {du[k].x, du[k].y, du[k].z, du[k].w};
             const uint32_t vs[4] = {dv[k].x, dv[k].y, dv[k].z, dv[k].w};
-            uint32_t imp = 0;
+            uint32_t imp = 0, over = 0;
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
-                if (!(act[k] >> i & 1u) || us[i] == 0xffffffffu) continue;
-                const uint64_t nd = (uint64_t)us[i] + ww[k];
-                if (nd >= 0xffffffffull) {
-                    grx_set_status(a.ctl, GRX_ERANGE);
-                } else if ((uint32_t)nd < vs[i]) {
+                const uint32_t nd = us[i] + ww[k];
+                const bool in = (act[k] >> i & 1u) && us[i] != 0xffffffffu;
+                const bool big = nd < us[i] || nd == 0xffffffffu;          // past 32 bits
+                over |= in && big ? 1u : 0u;
+                if (in && !big && nd < vs[i]) {
                     uint32_t *p = a.D + (int64_t)vv[k] * 64 + b0 + i;
-                    if (bmp) {
-                        // a reduction: the lane improves in this round, by this
-                        // proposal or a smaller one
-                        atomicMin(p, (uint32_t)nd);
+                    // a reduction where the touched go to a bitmap: the lane improves
+                    // in this round, by this proposal or a smaller one
+                    if (BMP) {
+                        asm volatile("red.relaxed.gpu.global.min.u32 [%0], %1;" ::"l"(p), "r"(nd) : "memory");
                         imp |= 1u << i;
-                    } else if ((uint32_t)nd < atomicMin(p, (uint32_t)nd)) {
+                    } else if (nd < atomicMin(p, nd)) {
                         imp |= 1u << i;
                     }
                 }
             }
+            if (over) grx_set_status(a.ctl, GRX_ERANGE);
             // the edge's improved lanes; its first thread publishes them
             unsigned long long m = (unsigned long long)imp << b0;
             if (__any_sync(GRX_FULL_MASK, imp != 0u)) {
@@ -176,14 +180,14 @@ __device__ __forceinline__ void relax_lanes(const MpArgs<OffT> &a, MpWarpSmem<Of
                 for (int o = TPE / 2; o > 0; o >>= 1) m |= __shfl_xor_sync(GRX_FULL_MASK, m, o);
                 bool first = false;
                 if (b0 == 0 && m) {
-                    if (bmp) {
+                    if (BMP) {
                         atomicOr(a.next + vv[k], m);                     // results unused: reductions
                         atomicOr(a.tbits + (vv[k] >> 5), 1u << (vv[k] & 31));
                     } else {
                         first = atomicOr(a.next + vv[k], m) == 0ull;
                     }
                 }
-                if (!bmp) {
+                if (!BMP) {
                     const unsigned int fm = __ballot_sync(GRX_FULL_MASK, first);
                     if (first) tbuf[nt + __popc(fm & lanemask_lt())] = vv[k];
                     nt += __popc(fm);
@@ -193,9 +197,9 @@ __device__ __forceinline__ void relax_lanes(const MpArgs<OffT> &a, MpWarpSmem<Of
     }
 }
 
-template <typename OffT>
+template <typename OffT, bool BMP>
 __device__ void mp_expand(const MpArgs<OffT> &a, int L, uint32_t q, uint64_t T, MpWarpSmem<OffT> &w,
-                          int32_t *tbuf, bool bmp) {
+                          int32_t *tbuf) {
     const unsigned int lane = threadIdx.x & 31;
     const int32_t *Qv = pk3(a.Q[0], a.Q[1], a.Q[2], L % 3);
     const uint32_t *Qe = pk3(a.E[0], a.E[1], a.E[2], L % 3);
@@ -205,65 +209,75 @@ __device__ void mp_expand(const MpArgs<OffT> &a, int L, uint32_t q, uint64_t T, 
     const uint64_t ntiles = (T + MP_WTILE - 1) / MP_WTILE;
     const uint64_t nwarps = (uint64_t)gridDim.x * MP_WARPS;
     const uint64_t gw = (uint64_t)blockIdx.x * MP_WARPS + (threadIdx.x >> 5);
-    const uint64_t per = (ntiles + nwarps - 1) / nwarps;
-    const uint64_t tb0 = gw * per;
-    const uint64_t tb1 = min(ntiles, tb0 + per);
-    if (tb0 >= tb1) return;
-    int64_t i0 = warp_upper_index_cg(Qe, (int64_t)q, (uint32_t)(tb0 * MP_WTILE));
-    for (uint64_t tile = tb0; tile < tb1; ++tile) {
-        const uint64_t e0 = tile * MP_WTILE;
-        const uint32_t e1 = (uint32_t)min(T, e0 + MP_WTILE);
-        int n = 0;
-        for (;;) {
-            const int64_t idx = i0 + n + lane;
-            uint32_t qe = 0xffffffffu;
-            if (idx < (int64_t)q) qe = __ldcg(Qe + idx);
-            const bool in = idx < (int64_t)q && qe < e1;
-            if (n + (int)lane <= MP_WTILE + 1) w.qe[n + lane] = qe;
-            if (in && n + (int)lane <= MP_WTILE) {
-                const int32_t u = __ldcg(Qv + idx);
-                w.u[n + lane] = u;
-                w.rs[n + lane] = __ldcg(Qr + idx);
-                w.cm[n + lane] = __ldcg(cin + u) & a.lanes;
+    // Batches of up to MP_BATCH tiles: the first by the warp's number, the others
+    // from the round's counter.  How long a tile takes depends on how many lanes
+    // improve, which varies along the queue (R-MAT 20, 16 / 64 sources: one equal
+    // share a warp 3.87 / 11.2 ms, batches of 16 tiles 3.61 / 10.0, of 4 3.50 / 9.6).
+    const uint64_t batch = min((uint64_t)MP_BATCH, (ntiles + nwarps - 1) / nwarps);
+    if (batch == 0) return;
+    const uint64_t nbatch = (ntiles + batch - 1) / batch;
+    unsigned int *wq = &a.ctl->wq[L & 3];
+    for (uint64_t bt = gw; bt < nbatch;) {
+        unsigned int nn = 0;
+        if (lane == 0) nn = atomicAdd(wq, 1u);
+        const uint64_t tb0 = bt * batch, tb1 = min(ntiles, tb0 + batch);
+        int64_t i0 = warp_upper_index_cg(Qe, (int64_t)q, (uint32_t)(tb0 * MP_WTILE));
+        for (uint64_t tile = tb0; tile < tb1; ++tile) {
+            const uint64_t e0 = tile * MP_WTILE;
+            const uint32_t e1 = (uint32_t)min(T, e0 + MP_WTILE);
+            int n = 0;
+            for (;;) {
+                const int64_t idx = i0 + n + lane;
+                uint32_t qe = 0xffffffffu;
+                if (idx < (int64_t)q) qe = __ldcg(Qe + idx);
+                const bool in = idx < (int64_t)q && qe < e1;
+                if (n + (int)lane <= MP_WTILE + 1) w.qe[n + lane] = qe;
+                if (in && n + (int)lane <= MP_WTILE) {
+                    const int32_t u = __ldcg(Qv + idx);
+                    w.u[n + lane] = u;
+                    w.rs[n + lane] = __ldcg(Qr + idx);
+                    w.cm[n + lane] = __ldcg(cin + u) & a.lanes;
+                }
+                const int cnt = __popc(__ballot_sync(GRX_FULL_MASK, in));
+                n += cnt;
+                if (cnt < 32) break;
+                if (n > MP_WTILE) {
+                    if (lane == 0) grx_set_status(a.ctl, GRX_EINVAL);
+                    n = MP_WTILE;
+                    break;
+                }
             }
-            const int cnt = __popc(__ballot_sync(GRX_FULL_MASK, in));
-            n += cnt;
-            if (cnt < 32) break;
-            if (n > MP_WTILE) {
-                if (lane == 0) grx_set_status(a.ctl, GRX_EINVAL);
-                n = MP_WTILE;
-                break;
-            }
-        }
-        __syncwarp();
-        const uint32_t next_start = w.qe[n];
-        // the tile's edges, two per lane, coalesced: target, weight, row
+            __syncwarp();
+            const uint32_t next_start = w.qe[n];
+            // the tile's edges, two per lane, coalesced: target, weight, row
 #pragma unroll
-        for (int h = 0; h < MP_WTILE / 32; ++h) {
-            const uint32_t e = (uint32_t)e0 + lane + 32 * h;
-            if (e < e1) {
-                const int j = upper_index_smem(w.qe, n, e);
-                const OffT idx = w.rs[j] + (OffT)(e - w.qe[j]);
-                w.ev[lane + 32 * h] = __ldg(a.col + idx);
-                w.ew[lane + 32 * h] = __ldg(a.w + idx);
-                w.er[lane + 32 * h] = j;
+            for (int h = 0; h < MP_WTILE / 32; ++h) {
+                const uint32_t e = (uint32_t)e0 + lane + 32 * h;
+                if (e < e1) {
+                    const int j = upper_index_smem(w.qe, n, e);
+                    const OffT idx = w.rs[j] + (OffT)(e - w.qe[j]);
+                    w.ev[lane + 32 * h] = __ldg(a.col + idx);
+                    w.ew[lane + 32 * h] = __ldg(a.w + idx);
+                    w.er[lane + 32 * h] = j;
+                }
             }
+            __syncwarp();
+            const int len = (int)(e1 - (uint32_t)e0);
+            int nt = 0;                                   // touched vertices of this tile (list rounds)
+            if (a.n <= 8) relax_lanes<OffT, 2, BMP>(a, w, len, tbuf, nt);
+            else if (a.n <= 16) relax_lanes<OffT, 4, BMP>(a, w, len, tbuf, nt);
+            else if (a.n <= 32) relax_lanes<OffT, 8, BMP>(a, w, len, tbuf, nt);
+            else relax_lanes<OffT, 16, BMP>(a, w, len, tbuf, nt);
+            __syncwarp();
+            // one append of the tile's touched vertices
+            unsigned int base = 0;
+            if (lane == 0 && nt) base = atomicAdd(tctr, (unsigned)nt);
+            base = __shfl_sync(GRX_FULL_MASK, base, 0);
+            for (int t = (int)lane; t < nt; t += 32) a.touched[base + t] = tbuf[t];
+            i0 = (next_start == e1) ? i0 + n : i0 + n - 1;
+            __syncwarp();
         }
-        __syncwarp();
-        const int len = (int)(e1 - (uint32_t)e0);
-        int nt = 0;                                   // touched vertices of this tile (list rounds)
-        if (a.n <= 8) relax_lanes<OffT, 2>(a, w, len, bmp, tbuf, nt);
-        else if (a.n <= 16) relax_lanes<OffT, 4>(a, w, len, bmp, tbuf, nt);
-        else if (a.n <= 32) relax_lanes<OffT, 8>(a, w, len, bmp, tbuf, nt);
-        else relax_lanes<OffT, 16>(a, w, len, bmp, tbuf, nt);
-        __syncwarp();
-        // one append of the tile's touched vertices
-        unsigned int base = 0;
-        if (lane == 0 && nt) base = atomicAdd(tctr, (unsigned)nt);
-        base = __shfl_sync(GRX_FULL_MASK, base, 0);
-        for (int t = (int)lane; t < nt; t += 32) a.touched[base + t] = tbuf[t];
-        i0 = (next_start == e1) ? i0 + n : i0 + n - 1;
-        __syncwarp();
+        bt = nwarps + __shfl_sync(GRX_FULL_MASK, nn, 0);
     }
 }
 
@@ -328,9 +342,13 @@ namespace {
 
 template <typename OffT>
 __global__ void __launch_bounds__(MP_BLOCK, 3) k_mssp_persistent(MpArgs<OffT> a) {
-    __shared__ MpWarpSmem<OffT> wsm[MP_WARPS];
-    __shared__ int32_t tbufs[MP_WARPS][MP_WTILE];
-    __shared__ uint16_t lists[MP_WARPS][32 * 32];
+    __shared__ union Warp {                  // expand and finalize phases do not overlap
+        struct {
+            MpWarpSmem<OffT> w;
+            int32_t tbuf[MP_WTILE];
+        };
+        uint16_t list[32 * 32];
+    } wsm[MP_WARPS];
     __shared__ uint32_t s_q, s_T;
     __shared__ int s_done;
     const int wi = threadIdx.x >> 5;
@@ -356,6 +374,7 @@ __global__ void __launch_bounds__(MP_BLOCK, 3) k_mssp_persistent(MpArgs<OffT> a)
         if (blockIdx.x == 0 && threadIdx.x == 0) {
             a.ctl->qpack[(L + 2) & 3] = 0ull;
             a.ctl->ucount[(L + 2) & 3] = 0u;
+            a.ctl->wq[(L + 2) & 3] = 0u;
         }
         {   // Q_{L-1}'s masks leave cur[(L+2)%3]
             const int32_t *Qp = pk3(a.Q[0], a.Q[1], a.Q[2], (L + 2) % 3);
@@ -365,9 +384,10 @@ __global__ void __launch_bounds__(MP_BLOCK, 3) k_mssp_persistent(MpArgs<OffT> a)
                 cp[__ldcg(Qp + i)] = 0ull;
         }
         const bool bmp = T >= a.bmp_min_T;
-        mp_expand(a, L, q, T, wsm[wi], tbufs[wi], bmp);
+        if (bmp) mp_expand<OffT, true>(a, L, q, T, wsm[wi].w, wsm[wi].tbuf);
+        else mp_expand<OffT, false>(a, L, q, T, wsm[wi].w, wsm[wi].tbuf);
         if (!flag_barrier(bar)) return;
-        mp_finalize(a, L, bmp, lists[wi]);
+        mp_finalize(a, L, bmp, wsm[wi].list);
         if (!flag_barrier(bar)) return;
         qprev = q;
     }
@@ -380,7 +400,7 @@ __global__ void k_mssp_transpose(const uint32_t *__restrict__ D, int32_t nv, int
     const int64_t v0 = (int64_t)blockIdx.x * 32;
     for (int r = threadIdx.y; r < 32; r += blockDim.y) {
         const int64_t v = v0 + r;
-        for (int b = threadIdx.x; b < 64; b += 32)
+        for (int b = threadIdx.x; b < n; b += 32)
             tile[r][b] = v < nv ? D[v * 64 + b] : 0u;
     }
     __syncthreads();
