@@ -44,6 +44,7 @@ constexpr int SS_MIN_BLOCKS = 2;             // resident blocks per SM (register
 constexpr int SS_WARPS = SS_BLOCK / 32;
 constexpr int SS_ITEMS = 8;
 constexpr int SS_WTILE = 32 * SS_ITEMS;
+constexpr int SS_BATCH = 4;                  // tiles a warp takes at a time
 constexpr int SS_RPL = 4;                    // finalize: vertices per lane per round
 
 template <typename OffT>
@@ -140,106 +141,116 @@ __device__ void relax_round(const SsspArgs<OffT> &a, const SsState &st, SsWarpSm
     const uint64_t ntiles = (T + SS_WTILE - 1) / SS_WTILE;
     const uint64_t nwarps = (uint64_t)gridDim.x * SS_WARPS;
     const uint64_t gw = (uint64_t)blockIdx.x * SS_WARPS + (threadIdx.x >> 5);
-    const uint64_t per = (ntiles + nwarps - 1) / nwarps;
-    const uint64_t tb0 = gw * per;
-    const uint64_t tb1 = min(ntiles, tb0 + per);
-    if (tb0 >= tb1) return;
-    int64_t i0 = warp_upper_index_cg(Qe, q, (uint32_t)(tb0 * SS_WTILE));
-    for (uint64_t tile = tb0; tile < tb1; ++tile) {
-        const uint64_t e0 = tile * SS_WTILE;
-        const uint32_t e1 = (uint32_t)min(T, e0 + SS_WTILE);
-        // frontier elements starting before e1, 32 per round
-        int n = 0;
-        for (;;) {
-            const int64_t idx = i0 + n + lane;
-            uint32_t qe = 0xffffffffu;
-            if (idx < q) qe = __ldcg(Qe + idx);
-            const bool in = idx < q && qe < e1;
-            if (n + (int)lane <= SS_WTILE + 1) w.qe[n + lane] = qe;
-            if (in && n + (int)lane <= SS_WTILE) {
-                const int32_t u = __ldcg(Qv + idx);
-                w.u[n + lane] = u;
-                w.rs[n + lane] = __ldcg(Qr + idx);
-                w.du[n + lane] = __ldcg(a.dist + u);
-            }
-            const int cnt = __popc(__ballot_sync(GRX_FULL_MASK, in));
-            n += cnt;
-            if (cnt < 32) break;
-            if (n > SS_WTILE) {              // only possible with a malformed graph
-                if (lane == 0) grx_set_status(a.ctl, GRX_EINVAL);
-                n = SS_WTILE;
-                break;
-            }
-        }
-        __syncwarp();
-        const uint32_t next_start = w.qe[n];
-        int row[SS_ITEMS];
-        warp_tile_rows8_strided(w.rid, w.qe, (uint32_t)e0, n, row);   // item k at position k*32 + lane
-        int32_t v[SS_ITEMS];
-        uint32_t wt[SS_ITEMS], du[SS_ITEMS];
-#pragma unroll
-        for (int k = 0; k < SS_ITEMS; ++k) {
-            const uint32_t e = (uint32_t)e0 + (uint32_t)k * 32 + lane;
-            const int j = row[k];
-            const bool ok = e < e1;
-            const OffT idx = ok ? w.rs[j] + (OffT)(e - w.qe[j]) : (OffT)0;
-            v[k] = ok ? __ldg(a.col + idx) : -1;
-            wt[k] = ok ? __ldg(a.w + idx) : 0u;
-            du[k] = ok ? w.du[j] : 0xffffffffu;
-        }
-        __syncwarp();
-        uint32_t nd[SS_ITEMS], cur[SS_ITEMS];
-#pragma unroll
-        for (int k = 0; k < SS_ITEMS; ++k) {
-            nd[k] = 0xffffffffu;
-            if (v[k] >= 0 && du[k] != 0xffffffffu) {
-                const uint64_t s64 = (uint64_t)du[k] + wt[k];
-                if (s64 >= 0xffffffffull) grx_set_status(a.ctl, GRX_ERANGE);
-                else nd[k] = (uint32_t)s64;
-            }
-            cur[k] = nd[k] != 0xffffffffu ? __ldcg(a.dist + v[k]) : 0u;
-        }
-        if (BMP) {
-#pragma unroll
-            for (int k = 0; k < SS_ITEMS; ++k) {
-                if (nd[k] < cur[k]) {
-                    atomicMin(a.dist + v[k], nd[k]);                     // results unused: reductions
-                    atomicOr(a.cbits + (v[k] >> 5), 1u << (v[k] & 31));
+    // Batches of up to SS_BATCH tiles: the first by the warp's number, the others
+    // from the round's counter.  What a tile costs varies along the queue (R-MAT 22,
+    // mean of three sources: one equal share a warp 1,824 us, batches of 16 / 8 / 4 / 2
+    // tiles 1,618 / 1,577 / 1,569 / 1,744; a batch costs a search).
+    const uint64_t batch = min((uint64_t)SS_BATCH, (ntiles + nwarps - 1) / nwarps);
+    if (batch == 0) return;
+    const uint64_t nbatch = (ntiles + batch - 1) / batch;
+    unsigned int *wq = &a.ctl->wq[L & 3];
+    for (uint64_t bt = gw; bt < nbatch;) {
+        unsigned int nn = 0;
+        if (lane == 0) nn = atomicAdd(wq, 1u);
+        const uint64_t tb0 = bt * batch, tb1 = min(ntiles, tb0 + batch);
+        int64_t i0 = warp_upper_index_cg(Qe, q, (uint32_t)(tb0 * SS_WTILE));
+        for (uint64_t tile = tb0; tile < tb1; ++tile) {
+            const uint64_t e0 = tile * SS_WTILE;
+            const uint32_t e1 = (uint32_t)min(T, e0 + SS_WTILE);
+            // frontier elements starting before e1, 32 per round
+            int n = 0;
+            for (;;) {
+                const int64_t idx = i0 + n + lane;
+                uint32_t qe = 0xffffffffu;
+                if (idx < q) qe = __ldcg(Qe + idx);
+                const bool in = idx < q && qe < e1;
+                if (n + (int)lane <= SS_WTILE + 1) w.qe[n + lane] = qe;
+                if (in && n + (int)lane <= SS_WTILE) {
+                    const int32_t u = __ldcg(Qv + idx);
+                    w.u[n + lane] = u;
+                    w.rs[n + lane] = __ldcg(Qr + idx);
+                    w.du[n + lane] = __ldcg(a.dist + u);
+                }
+                const int cnt = __popc(__ballot_sync(GRX_FULL_MASK, in));
+                n += cnt;
+                if (cnt < 32) break;
+                if (n > SS_WTILE) {              // only possible with a malformed graph
+                    if (lane == 0) grx_set_status(a.ctl, GRX_EINVAL);
+                    n = SS_WTILE;
+                    break;
                 }
             }
-        } else {
-            uint32_t improved = 0;
+            __syncwarp();
+            const uint32_t next_start = w.qe[n];
+            int row[SS_ITEMS];
+            warp_tile_rows8_strided(w.rid, w.qe, (uint32_t)e0, n, row);   // item k at position k*32 + lane
+            int32_t v[SS_ITEMS];
+            uint32_t wt[SS_ITEMS], du[SS_ITEMS];
 #pragma unroll
             for (int k = 0; k < SS_ITEMS; ++k) {
-                if (nd[k] < cur[k]) {
-                    const uint32_t old = atomicMin(a.dist + v[k], nd[k]);
-                    if (nd[k] < old) improved |= 1u << k;
+                const uint32_t e = (uint32_t)e0 + (uint32_t)k * 32 + lane;
+                const int j = row[k];
+                const bool ok = e < e1;
+                const OffT idx = ok ? w.rs[j] + (OffT)(e - w.qe[j]) : (OffT)0;
+                v[k] = ok ? __ldg(a.col + idx) : -1;
+                wt[k] = ok ? __ldg(a.w + idx) : 0u;
+                du[k] = ok ? w.du[j] : 0xffffffffu;
+            }
+            __syncwarp();
+            uint32_t nd[SS_ITEMS], cur[SS_ITEMS];
+#pragma unroll
+            for (int k = 0; k < SS_ITEMS; ++k) {
+                nd[k] = 0xffffffffu;
+                if (v[k] >= 0 && du[k] != 0xffffffffu) {
+                    const uint64_t s64 = (uint64_t)du[k] + wt[k];
+                    if (s64 >= 0xffffffffull) grx_set_status(a.ctl, GRX_ERANGE);
+                    else nd[k] = (uint32_t)s64;
                 }
+                cur[k] = nd[k] != 0xffffffffu ? __ldcg(a.dist + v[k]) : 0u;
             }
-            uint32_t queued = 0;
+            if (BMP) {
 #pragma unroll
-            for (int k = 0; k < SS_ITEMS; ++k) {
-                if (!(improved >> k & 1u)) continue;
-                if (nd[k] >= st.thr) far_push(a, st, v[k]);
-                else if (atomicExch(a.stamp + v[k], L + 1) != L + 1) queued |= 1u << k;
-            }
-            uint32_t deg[SS_ITEMS];
-            OffT rb[SS_ITEMS];
-            uint32_t app = 0;
-#pragma unroll
-            for (int k = 0; k < SS_ITEMS; ++k) {
-                rb[k] = 0;
-                deg[k] = 0;
-                if (queued >> k & 1u) {
-                    rb[k] = __ldg(a.ro + v[k]);
-                    deg[k] = (uint32_t)(__ldg(a.ro + v[k] + 1) - rb[k]);
-                    if (deg[k]) app |= 1u << k;
+                for (int k = 0; k < SS_ITEMS; ++k) {
+                    if (nd[k] < cur[k]) {
+                        atomicMin(a.dist + v[k], nd[k]);                     // results unused: reductions
+                        atomicOr(a.cbits + (v[k] >> 5), 1u << (v[k] & 31));
+                    }
                 }
+            } else {
+                uint32_t improved = 0;
+#pragma unroll
+                for (int k = 0; k < SS_ITEMS; ++k) {
+                    if (nd[k] < cur[k]) {
+                        const uint32_t old = atomicMin(a.dist + v[k], nd[k]);
+                        if (nd[k] < old) improved |= 1u << k;
+                    }
+                }
+                uint32_t queued = 0;
+#pragma unroll
+                for (int k = 0; k < SS_ITEMS; ++k) {
+                    if (!(improved >> k & 1u)) continue;
+                    if (nd[k] >= st.thr) far_push(a, st, v[k]);
+                    else if (atomicExch(a.stamp + v[k], L + 1) != L + 1) queued |= 1u << k;
+                }
+                uint32_t deg[SS_ITEMS];
+                OffT rb[SS_ITEMS];
+                uint32_t app = 0;
+#pragma unroll
+                for (int k = 0; k < SS_ITEMS; ++k) {
+                    rb[k] = 0;
+                    deg[k] = 0;
+                    if (queued >> k & 1u) {
+                        rb[k] = __ldg(a.ro + v[k]);
+                        deg[k] = (uint32_t)(__ldg(a.ro + v[k] + 1) - rb[k]);
+                        if (deg[k]) app |= 1u << k;
+                    }
+                }
+                warp_append_items<SS_ITEMS, OffT>(v, deg, rb, app, Qv_out, Qe_out, Qr_out, ctr);
             }
-            warp_append_items<SS_ITEMS, OffT>(v, deg, rb, app, Qv_out, Qe_out, Qr_out, ctr);
+            i0 = (next_start == e1) ? i0 + n : i0 + n - 1;
+            __syncwarp();
         }
-        i0 = (next_start == e1) ? i0 + n : i0 + n - 1;
-        __syncwarp();
+        bt = nwarps + __shfl_sync(GRX_FULL_MASK, nn, 0);
     }
 }
 
@@ -550,7 +561,10 @@ __device__ __forceinline__ bool list_rounds(const SsspArgs<OffT> &a, SsState &s_
     }
     if (blockIdx.x == 0 && threadIdx.x == 0) {
         a.ctl->narrow_epoch += 1;                // no block reads it before the barrier below
-        for (int i = 0; i < 4; ++i) a.ctl->qpack[i] = 0ull;
+        for (int i = 0; i < 4; ++i) {
+            a.ctl->qpack[i] = 0ull;
+            a.ctl->wq[i] = 0u;
+        }
     }
     if (!flag_barrier(bar)) return false;
     if (threadIdx.x == 0) {
@@ -650,6 +664,7 @@ __global__ void __launch_bounds__(SS_BLOCK, SS_MIN_BLOCKS) k_sssp_persistent(con
             const int L = st.L;
             if (st.op == SOP_RELAX && blockIdx.x == 0 && threadIdx.x == 0) {
                 a.ctl->qpack[(L + 2) & 3] = 0ull;
+                a.ctl->wq[(L + 2) & 3] = 0u;
                 if (STATS && L < GRX_MAX_LEVELS_STATS) {
                     a.stats->level_t0[L] = grx_globaltimer();
                     a.stats->dir[L] = 0;
@@ -689,6 +704,7 @@ __global__ void k_sssp_init(int32_t src, const OffT *ro, uint32_t *dist, int32_t
     R0[0] = b;
     ctl->qpack[0] = deg ? ((1ull << 32) | deg) : 0ull;
     for (int i = 1; i < 4; ++i) ctl->qpack[i] = 0ull;
+    for (int i = 0; i < 4; ++i) ctl->wq[i] = 0u;
     ctl->farcnt[0] = 0u;
     ctl->farcnt[1] = 0u;
     ctl->farmin[0] = 0xffffffffu;
