@@ -1593,10 +1593,19 @@ grx_status launch_typed(grx_graph *g, int32_t src, int32_t *depth, int32_t *pare
         return GRX_OK;
     }
     // Narrow levels on graphs of few edges a vertex, which may have thousands of
-    // levels; where vertices have more, everything is reached in a few.
-    return a.narrow && g->ne < 8ll * g->nv && o->direction != GRX_DIR_PULL
-               ? launch_persistent<OffT, PARENT, STATS, true>(g, a, o, s)
-               : launch_persistent<OffT, PARENT, STATS, false>(g, a, o, s);
+    // levels; where vertices have more, everything is reached in a few.  Their
+    // buffers are allocated by the first call that uses them, and start zeroed:
+    // memory of a freed graph could hold words with this graph's first tags.
+    // Without memory there are no narrow levels.
+    if (g->ne >= 8ll * g->nv || o->direction == GRX_DIR_PULL)
+        return launch_persistent<OffT, PARENT, STATS, false>(g, a, o, s);
+    if (!g->narrow && !g->fixed_scratch && !grx_capturing(s)) {
+        g->narrow = (NarrowBuffers *)grx_alloc(g, sizeof(NarrowBuffers), s);
+        if (g->narrow) GRX_CUDA(cudaMemsetAsync(g->narrow, 0, sizeof(NarrowBuffers), s));
+        a.narrow = g->narrow;
+    }
+    return a.narrow ? launch_persistent<OffT, PARENT, STATS, true>(g, a, o, s)
+                    : launch_persistent<OffT, PARENT, STATS, false>(g, a, o, s);
 }
 
 template <typename OffT>

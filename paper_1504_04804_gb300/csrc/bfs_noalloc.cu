@@ -154,6 +154,7 @@ extern "C" grx_status bfs_noalloc(int64_t nv, int64_t ne, const int32_t *row_off
     g.ctl = &sc->ctl;
     g.bar_flags = sc->bar_flags;
     g.ws_ready = 1;
+    g.fixed_scratch = 1;
     st = grx_bfs_launch(&g, src, depth_out, parent_out, &o, s);
     if (st != GRX_OK) return st;
     if (status_out)

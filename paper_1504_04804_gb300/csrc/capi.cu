@@ -7,7 +7,6 @@
 #include <cstring>
 
 #include "grx_internal.cuh"
-#include "narrow.cuh"
 
 // ---------------------------------------------------------------------------
 // errors
@@ -48,6 +47,13 @@ void grx_ctx_free(grx_ctx *c, void *p, size_t bytes, cudaStream_t s) {
     if (bytes == 0) bytes = 16;
     if (c->has_alloc) c->alloc.free(p, bytes, (void *)s, c->alloc.user);
     else cudaFreeAsync(p, s);
+}
+
+bool grx_capturing(cudaStream_t s) {
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(s, &cap) == cudaSuccess) return cap != cudaStreamCaptureStatusNone;
+    cudaGetLastError();
+    return true;
 }
 
 void *grx_alloc(grx_graph *g, size_t bytes, cudaStream_t s) {
@@ -343,9 +349,6 @@ grx_status grx_ensure_workspace(grx_graph *g, cudaStream_t s) {
     for (int i = 0; i < 3; ++i) ok = ok && g->fbits[i] && g->qv[i] && g->qe[i] && g->qr[i];
     for (int i = 0; i < 2; ++i) ok = ok && g->ulist[i];
     if (!ok) return grx_fail(GRX_ENOMEM, "traversal workspace allocation failed (nv=%d)", g->nv);
-    g->narrow = (NarrowBuffers *)grx_alloc(g, sizeof(NarrowBuffers), s);   // traversals do without it
-    // (memory of a freed graph could hold words with this graph's first tags)
-    if (g->narrow) GRX_CUDA(cudaMemsetAsync(g->narrow, 0, sizeof(NarrowBuffers), s));
     GRX_CUDA(cudaMemsetAsync(g->ctl, 0, sizeof(TravCtl), s));
     GRX_CUDA(cudaMemsetAsync(g->stats, 0, sizeof(DevStats), s));
     grx_status st = grx_build_first2(g, s);
@@ -374,7 +377,7 @@ static size_t workspace_new_bytes(const grx_graph *g, bool multi) {
     size_t b = 0;
     if (!g->ws_ready)
         b += wb + 3 * (wb + nv * 8 + nv * (g->off64 ? 8 : 4)) + 2 * nv * 4 + nv * sizeof(int2) +
-             sizeof(TravCtl) + sizeof(unsigned int) * GRX_MAX_GRID + sizeof(DevStats) + nv * 4 + sizeof(NarrowBuffers);
+             sizeof(TravCtl) + sizeof(unsigned int) * GRX_MAX_GRID + sizeof(DevStats) + nv * 4;
     if (multi && !g->ms_ready) b += 5 * nv * 8;
     return b;
 }

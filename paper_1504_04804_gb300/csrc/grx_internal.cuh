@@ -149,7 +149,8 @@ struct grx_graph {
     void *ss_lines;                  // list rounds of sssp: lines, pieces, vertices (first use)
     uint32_t ss_list_T;              // ... edges of a round per block
     int ss_list_blocks;              // ... blocks they are laid out for
-    struct NarrowBuffers *narrow;    // narrow levels (narrow.cuh); NULL: none
+    struct NarrowBuffers *narrow;    // narrow levels of bfs (narrow.cuh), first use
+    int fixed_scratch;               // bfs_noalloc's view: nothing may be allocated
     cudaGraphExec_t bfs_gexec[2];
     void *bfs_gargs;                 // device copy of the call's arguments
     // 64-bit vertex ids (graph_load_csr64): columns, frontier queues and
@@ -165,6 +166,9 @@ struct grx_graph {
     int nallocs;
 };
 
+// Whether s is being captured (or may not be asked): no time to allocate what a
+// call can do without.
+bool grx_capturing(cudaStream_t s);
 // Allocation through the context allocator (or cudaMallocAsync).
 void *grx_alloc(grx_graph *g, size_t bytes, cudaStream_t s);
 void *grx_ctx_alloc(grx_ctx *c, size_t bytes, cudaStream_t s);

@@ -412,12 +412,7 @@ PrsRows prs_rows(const grx_graph *g) {
 grx_status grx_prs_build(grx_graph *g, cudaStream_t s, int *ready) {
     *ready = g->prs_cols != nullptr;
     if (*ready || g->n_active == 0) return GRX_OK;
-    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-    if (cudaStreamIsCapturing(s, &cap) != cudaSuccess) {
-        cudaGetLastError();
-        return GRX_OK;
-    }
-    if (cap != cudaStreamCaptureStatusNone) return GRX_OK;
+    if (grx_capturing(s)) return GRX_OK;
     const int64_t n = g->n_active, ne = g->ne;
     // chunks of 1,024 edges on large graphs; smaller ones on small graphs, where
     // a warp's whole share is a few hundred edges.  Rows past eight chunks are

@@ -716,13 +716,7 @@ __global__ void k_sssp_init(int32_t src, const OffT *ro, uint32_t *dist, int32_t
 // The list rounds' buffers of g for grids of up to `blocks` (once; NULL without
 // memory, or while s is captured: the rounds then run on the queue).
 grx_status ss_list_buffers(grx_graph *g, int blocks, cudaStream_t s) {
-    if (g->ss_lines || blocks > SS_BLOCK) return GRX_OK;
-    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-    if (cudaStreamIsCapturing(s, &cap) != cudaSuccess) {
-        cudaGetLastError();
-        return GRX_OK;
-    }
-    if (cap != cudaStreamCaptureStatusNone) return GRX_OK;
+    if (g->ss_lines || blocks > SS_BLOCK || grx_capturing(s)) return GRX_OK;
     // rounds of up to 3,072 edges a block, a quarter of the graph's at most
     const int64_t share = g->ne / 4 / blocks;
     const uint32_t t = (uint32_t)(share < 192 ? 192 : (share > 3072 ? 3072 : share));
