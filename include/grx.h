@@ -318,7 +318,8 @@ typedef struct {
 /* Synchronise `stream` and copy the counters of the graph's last traversal
  * that ran with collect_stats = 1.  After cc (which always counts), only
  * `levels` is set: the number of hooking rounds.  For multi-source BFS pull
- * levels, vertices_scanned counts the rows of the edge tiles not skipped. */
+ * levels, vertices_scanned counts the rows not skipped, edges_examined the
+ * neighbours read. */
 grx_status grx_last_stats(grx_graph *g, void *stream, grx_trav_stats *out);
 
 /* ---- seeded input generation (device twins of the host generators) ------ */

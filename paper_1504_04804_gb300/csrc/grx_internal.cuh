@@ -85,8 +85,7 @@ struct grx_graph {
     int32_t *active;
     uint32_t *aoff;
     int64_t n_active;
-    // static row ranges of all-edges tiles (CC hooking, PageRank, multi-source
-    // pull), per tile size
+    // static row ranges of all-edges tiles (PageRank in CSR order), per tile size
     int2 *etiles[4];
     int etile_size[4];
     void *last_stream;
@@ -132,9 +131,9 @@ struct grx_graph {
     // multi-source
     unsigned long long *ms_cur[3], *ms_next, *ms_seen;   // [nv] each
     unsigned long long *ms_hist[6];  // multi-source BFS: pull levels' new lanes, [nv] each
-    int32_t *ms_fix;                 // multi-source BFS: per pull tile, the crossing row it finishes
+    int2 *ms_rest;                   // multi-source BFS: pieces of rows a pull level leaves open
     uint32_t *ms_tbits;              // multi-source BFS: touched bitmap of bitmap push levels
-    uint8_t *ms_sat;                 // multi-source BFS: per pull tile, all lanes seen
+    uint8_t *ms_sat;                 // multi-source BFS: per 128 rows, all lanes seen
     uint32_t *ms_dist;               // batched SSSP, vertex-major [nv][64]
     int ms_ready;
     // betweenness centrality (allocated on first use)

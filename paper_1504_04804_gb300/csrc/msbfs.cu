@@ -15,13 +15,12 @@
 //    scan).  A finalize phase turns each touched vertex's next mask into its
 //    new lanes, labels them (scattered depth writes: few), and appends the
 //    vertex to the next queue.
-//  * Pull level (dense frontier): static tiles of equal edge count over the
-//    non-isolated vertices (their edge prefix is the CSR offsets).  A block
-//    stages a tile's rows, drops the rows whose lanes are all seen, gathers
-//    cur[u] over the remaining rows' edges into a per-row OR in shared
-//    memory, and finishes the rows that lie inside the tile; a row that
-//    crosses tiles ORs its partials into a global accumulator and is
-//    finished by a fix-up phase.
+//  * Pull level (dense frontier): warps take the non-isolated vertices 128 at a
+//    time and gather cur[u] over a row only until every lane the row misses is
+//    found (edge skipping, for all lanes at once): its first two neighbours
+//    (first2), a lane per row; then eight lanes per row, 32 edges a step.  Rows
+//    still open after MS_HEAD edges leave the rest to a second phase, in pieces
+//    of 1,024 edges over the grid, and are finished by a third.
 //  * Depths found by pull levels are not written per level: the level's new
 //    lane masks go to one of MS_HSLOTS history slots, and a flush pass
 //    writes them lane-major with coalesced stores (and, at the end, -1 for
@@ -33,8 +32,8 @@
 //    pull ANDs the gathered lanes with the row's missing lanes, and a push
 //    reads cur only for queue entries, which the previous level wrote.  The
 //    queue of a push after a pull comes from the pull's history slot.
-//  * A pull tile whose rows have every lane seen stays so: it is flagged and
-//    skipped by later pull levels.
+//  * 128 rows that have every lane seen stay so: they are flagged and skipped by
+//    later pull levels.
 //  * One cooperative persistent kernel; levels and their phases are
 //    separated by the bounded flag barrier.
 #include <cstring>
@@ -47,15 +46,19 @@ constexpr int MS_BLOCK = 256;
 constexpr int MS_WARPS = MS_BLOCK / 32;
 constexpr int MS_ITEMS = 8;
 constexpr int MS_WTILE = 32 * MS_ITEMS;             // push: edges per warp tile
-constexpr int MS_PITEMS = 7;
-constexpr int MS_PTILE = MS_BLOCK * MS_PITEMS;      // pull: edges per block tile
+constexpr int MS_ROWS = 128;                        // pull: rows a warp takes at a time
+// Pull: edges of a row in the first phase, after its first two (64 sources, R-MAT
+// 24 / 22 / 20: 30 7.58 / 2.27 / 0.82 ms, 126 7.02 / 2.16 / 0.89, 254 7.12 / 2.30 /
+// 0.98, 510 7.37 / 2.57 / 1.16).
+constexpr uint32_t MS_HEAD = 126;
+constexpr uint32_t MS_PIECE = 1024;                 // pull: edges of a piece of the second phase
 constexpr int MS_HSLOTS = 6;                        // history slots of pull levels
 #ifndef GRX_MS_MIN_BLOCKS
 #define GRX_MS_MIN_BLOCKS 3                         // resident blocks per SM (register cap)
 #endif
 
 enum { DIR_PUSH = 0, DIR_PULL = 1 };
-enum { MOP_COMPACT, MOP_EXPAND, MOP_FINAL, MOP_FLUSH, MOP_PULL, MOP_FIXUP };
+enum { MOP_COMPACT, MOP_EXPAND, MOP_FINAL, MOP_FLUSH, MOP_PULL, MOP_REST, MOP_FIXUP };
 
 template <typename OffT>
 struct MsArgs {
@@ -65,17 +68,17 @@ struct MsArgs {
     const int32_t *col;
     const int32_t *active;
     const uint32_t *aoff;
-    const int2 *tiles;                // pull tiles: (first active row, rows)
-    int64_t ntiles;
+    const int2 *first2;               // first two neighbours of every vertex (-1: none)
+    int64_t n_active;
     int n;
     unsigned long long lanes;         // active lane mask
     int32_t src[64];
     unsigned long long *seen;
-    unsigned long long *next;         // push: lane OR per touched vertex; pull: cross-tile OR
+    unsigned long long *next;         // push: lane OR per touched vertex; pull: OR of rows in pieces
     unsigned long long *cur[3];
     unsigned long long *hist[MS_HSLOTS];
-    int32_t *fix;                     // per pull tile: the crossing row it finishes (-1: none)
-    uint8_t *sat;                     // per pull tile: every row has all lanes seen
+    int2 *rest;                       // pieces of open rows: (active row, piece)
+    uint8_t *sat;                     // per MS_ROWS rows: every one has all lanes seen
     int32_t *Q[3];
     uint32_t *E[3];
     OffT *R[3];
@@ -115,24 +118,24 @@ union MsWarpSmem {
     uint16_t list[32 * 32];           // bitmap finalize: set bits of a 32-word chunk
 };
 
+// A warp's open rows: first edge, degree, active row, vertex; lanes missing, found.
 struct MsPullSmem {
-    uint32_t qe[MS_PTILE + 2];
-    int32_t vid[MS_PTILE + 1];
-    unsigned long long miss[MS_PTILE + 1];
-    unsigned long long acc[MS_PTILE + 1];
+    uint32_t s[MS_ROWS], deg[MS_ROWS];
+    int32_t i[MS_ROWS], v[MS_ROWS];
+    unsigned long long miss[MS_ROWS], acc[MS_ROWS];
 };
 
 template <typename OffT>
 union MsSmem {
     MsWarpSmem<OffT> w[MS_WARPS];
-    MsPullSmem p;
+    MsPullSmem p[MS_WARPS];
 };
 
 template <typename T>
 __device__ __forceinline__ T pk3(T a, T b, T c, int i) { return i == 0 ? a : (i == 1 ? b : c); }
 
 __device__ __forceinline__ int ms_phases(const MsState &s) {
-    return s.dir == DIR_PUSH ? 2 + s.compact : 2 + s.flush;
+    return s.dir == DIR_PUSH ? 2 + s.compact : 3 + s.flush;
 }
 
 __device__ __forceinline__ int ms_op(const MsState &s) {
@@ -141,7 +144,7 @@ __device__ __forceinline__ int ms_op(const MsState &s) {
         return p < 0 ? MOP_COMPACT : (p == 0 ? MOP_EXPAND : MOP_FINAL);
     }
     const int p = (int)s.phase - (int)s.flush;
-    return p < 0 ? MOP_FLUSH : (p == 0 ? MOP_PULL : MOP_FIXUP);
+    return p < 0 ? MOP_FLUSH : MOP_PULL + p;
 }
 
 template <typename OffT>
@@ -164,7 +167,9 @@ __device__ __forceinline__ void write_depths(int32_t *depth, int32_t nv, int32_t
 template <typename OffT>
 __device__ MsState ms_next_state(const MsArgs<OffT> &a, const MsState &st, bool stats) {
     MsState ns = st;
-    if ((int)st.phase + 1 < ms_phases(st)) {
+    // a pull that left no pieces is over after its first phase
+    const bool over = ms_op(st) == MOP_PULL && ld_relaxed_u32(&a.ctl->ucount[(st.L + 1) & 3]) == 0u;
+    if ((int)st.phase + 1 < ms_phases(st) && !over) {
         ns.phase = st.phase + 1;
         return ns;
     }
@@ -226,7 +231,7 @@ __device__ void ms_init_fill(const MsArgs<OffT> &a, bool dirty) {
     }
     if (dirty)
         for (int64_t w = tid; w < a.words; w += stride) a.tbits[w] = 0u;
-    for (int64_t t = tid; t < a.ntiles; t += stride) a.sat[t] = 0;
+    for (int64_t t = tid; t < (a.n_active + MS_ROWS - 1) / MS_ROWS; t += stride) a.sat[t] = 0;
 }
 
 // Phase 1 (one thread): seed the lanes (depth 0), the first frontier
@@ -256,6 +261,7 @@ __device__ void ms_seed(const MsArgs<OffT> &a) {
     for (int i = 1; i < 4; ++i) a.ctl->qpack[i] = 0ull;
     for (int i = 0; i < 4; ++i) a.ctl->pairs[i] = 0ull;
     a.ctl->ucount[1] = 0u;
+    for (int i = 0; i < 4; ++i) a.ctl->wq[i] = 0u;
     a.ctl->cpack = 0ull;
     a.ctl->ms_grid = gridDim.x;
     a.ctl->ms_done = 0u;
@@ -466,174 +472,175 @@ __device__ __forceinline__ void ms_pull_finish(unsigned long long *seen, unsigne
     c.pairs += (unsigned long long)__popcll(nw);
 }
 
-// Pull, phase 1: one block per static tile of the active list's edges.
-// ORs each item's lane mask into its row's shared accumulator.  A thread's
-// items are consecutive positions with non-decreasing rows, and a warp's
-// threads hold consecutive runs of positions, so a row's items within a warp
-// sit in consecutive lanes.  A row strictly inside one lane's items is stored
-// by that lane alone; rows at lane boundaries are OR-ed across the warp by a
-// segmented shuffle scan and added once per warp by the lane where they end
-// (a hub row filling a tile costs one shared atomic per warp, not one per
-// thread).  All 32 lanes call; valid = the lane's item count (0..MS_PITEMS).
-__device__ __forceinline__ void or_runs(unsigned long long *acc, const int (&row)[MS_PITEMS],
-                                        const unsigned long long (&g)[MS_PITEMS], int valid) {
-    const unsigned int lane = threadIdx.x & 31;
-    int fk = -1, lk = -1;          // rows of the lane's first run (when it ends inside the lane) and last run
-    unsigned long long fs = 0ull, ls = 0ull;
-    if (valid > 0) {
-        int cj = row[0];
-        unsigned long long part = 0ull;
-        bool first = true;
-#pragma unroll
-        for (int k = 0; k < MS_PITEMS; ++k) {
-            if (k < valid) {
-                if (row[k] != cj) {
-                    if (first) {
-                        fk = cj;
-                        fs = part;
-                        first = false;
-                    } else if (part) {
-                        acc[cj] = part;           // a row inside this lane's items
-                    }
-                    part = 0ull;
-                    cj = row[k];
-                }
-                part |= g[k];
-            }
-        }
-        lk = cj;
-        ls = part;
-    }
-    const int pk = __shfl_up_sync(GRX_FULL_MASK, lk, 1);
-    const bool prev_same = lane > 0 && pk == lk && lk >= 0;
-    unsigned long long m = ls;
-    int head = (fk >= 0 || !prev_same) ? 1 : 0;
-    // segmented inclusive OR-scan of the last runs (Hillis-Steele with head flags)
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const unsigned long long m2 = __shfl_up_sync(GRX_FULL_MASK, m, o);
-        const int h2 = __shfl_up_sync(GRX_FULL_MASK, head, o);
-        if (lane >= (unsigned)o && !head) {
-            m |= m2;
-            head |= h2;
-        }
-    }
-    const unsigned long long pm = __shfl_up_sync(GRX_FULL_MASK, m, 1);
-    if (fk >= 0) {
-        const unsigned long long x = fs | ((lane > 0 && pk == fk) ? pm : 0ull);
-        if (x) atomicOr(&acc[fk], x);
-    }
-    const int nfk = __shfl_down_sync(GRX_FULL_MASK, fk, 1);
-    const int nlk = __shfl_down_sync(GRX_FULL_MASK, lk, 1);
-    const bool next_cont = lane < 31 && ((nfk >= 0 && nfk == lk) || (nfk < 0 && nlk == lk));
-    if (lk >= 0 && !next_cont && m) atomicOr(&acc[lk], m);
-}
-
+// Pull, phase 1 (see the head of the file).  With every open row's edges gathered
+// (in equal tiles), the three pull levels of 64 sources on R-MAT 24 took 3.80,
+// 3.43 and 1.02 ms, and take 2.64 (88 % of the neighbours read: few rows find all
+// their lanes so early), 0.25 (6 %) and 0.13.
 template <typename OffT, bool STATS>
-__device__ void ms_pull(const MsArgs<OffT> &a, const MsState &st, MsPullSmem &p, MsCounts &c) {
+__device__ void ms_pull(const MsArgs<OffT> &a, const MsState &st, MsPullSmem &w, MsCounts &c) {
+    constexpr int PER = MS_ROWS / 32;
     const int L = st.L;
+    const unsigned int lane = threadIdx.x & 31;
     const unsigned long long *cin = pk3(a.cur[0], a.cur[1], a.cur[2], L % 3);
     unsigned long long *cout = pk3(a.cur[0], a.cur[1], a.cur[2], (L + 1) % 3);
     unsigned long long *hs = a.hist[st.flush ? 0 : st.hslots];
-    __shared__ int s_open;
-    for (int64_t tile = blockIdx.x; tile < a.ntiles; tile += gridDim.x) {
-        if (__ldcg(a.sat + tile)) continue;                  // uniform in the block
-        const uint64_t e0 = (uint64_t)tile * MS_PTILE;
-        const uint64_t e1 = min((uint64_t)a.ne, e0 + MS_PTILE);
-        const int len = (int)(e1 - e0);
-        const int2 tr = __ldg(a.tiles + tile);
-        const int64_t i0 = tr.x;
-        const int n = tr.y;
-        for (int j = threadIdx.x; j <= n; j += MS_BLOCK) {   // n+1 prefixes: qe[n] = end of last row
-            p.qe[j] = __ldg(a.aoff + i0 + j);
-            if (j < n) {
-                const int32_t v = __ldg(a.active + i0 + j);
-                p.vid[j] = v;
-                p.miss[j] = a.lanes & ~__ldcg(a.seen + v);
-                p.acc[j] = 0ull;
-            }
-        }
-        if (threadIdx.x == 0) {
-            a.fix[tile] = -1;
-            s_open = 0;
-            if (STATS) c.rows += (unsigned long long)n;
-        }
-        __syncthreads();
-        // a run of MS_PITEMS consecutive edges per thread: rows first, then
-        // every column and every gather in flight together; rows with every
-        // lane seen gather nothing
-        const int t0 = threadIdx.x * MS_PITEMS;
-        int rj[MS_PITEMS];
-        unsigned long long gv[MS_PITEMS];
+    unsigned int *wq = &a.ctl->wq[L & 3], *rctr = &a.ctl->ucount[(L + 1) & 3];
+    const int64_t nch = (a.n_active + MS_ROWS - 1) / MS_ROWS;
+    const int64_t nwarps = (int64_t)gridDim.x * MS_WARPS;
+    for (int64_t ch = (int64_t)blockIdx.x * MS_WARPS + (threadIdx.x >> 5); ch < nch;) {
+        unsigned int nn = 0;
+        if (lane == 0) nn = atomicAdd(wq, 1u);
+        if (!__ldcg(a.sat + ch)) {
+            int32_t v[PER];
+            uint32_t s[PER], deg[PER];
+            unsigned long long miss[PER], acc[PER];
+            int2 f2[PER];
 #pragma unroll
-        for (int k = 0; k < MS_PITEMS; ++k) {
-            rj[k] = 0;
-            gv[k] = 0ull;
-        }
-        if (t0 < len) {
-            int j = upper_index_smem(p.qe, n, (uint32_t)(e0 + t0));
-#pragma unroll
-            for (int k = 0; k < MS_PITEMS; ++k) {
-                const uint32_t e = (uint32_t)(e0 + t0 + k);
-                if (t0 + k < len)
-                    while (p.qe[j + 1] <= e) ++j;
-                rj[k] = j;
-            }
-            int32_t u[MS_PITEMS];
-#pragma unroll
-            for (int k = 0; k < MS_PITEMS; ++k)
-                u[k] = (t0 + k < len && p.miss[rj[k]]) ? __ldg(a.col + e0 + t0 + k) : -1;
-#pragma unroll
-            for (int k = 0; k < MS_PITEMS; ++k) gv[k] = u[k] >= 0 ? __ldca(cin + u[k]) : 0ull;
-            if (STATS) {
-#pragma unroll
-                for (int k = 0; k < MS_PITEMS; ++k) c.gathered += u[k] >= 0 ? 1ull : 0ull;
-            }
-        }
-        or_runs(p.acc, rj, gv, t0 < len ? min(MS_PITEMS, len - t0) : 0);
-        __syncthreads();
-        int open = 0;
-        for (int j = threadIdx.x; j < n; j += MS_BLOCK) {
-            const int32_t v = p.vid[j];
-            const uint32_t start = p.qe[j], end = p.qe[j + 1];
-            const unsigned long long nw = p.acc[j] & p.miss[j];
-            if (p.miss[j] & ~nw) open = 1;                    // lanes still missing after this level
-            if (start >= e0 && end <= e1) {
-                if (nw) {
-                    cout[v] = nw;
-                    ms_pull_finish(a.seen, hs, v, a.lanes & ~p.miss[j], nw, end - start, c);
+            for (int k = 0; k < PER; ++k) {
+                const int64_t i = ch * MS_ROWS + k * 32 + lane;
+                v[k] = -1;
+                s[k] = deg[k] = 0u;
+                if (i < a.n_active) {
+                    v[k] = __ldg(a.active + i);
+                    s[k] = __ldg(a.aoff + i);
+                    deg[k] = __ldg(a.aoff + i + 1) - s[k];
                 }
-            } else {
-                if (nw) atomicOr(a.next + v, nw);
-                if (end <= e1) a.fix[tile] = v;               // this tile holds the row's last edge
             }
+#pragma unroll
+            for (int k = 0; k < PER; ++k) {
+                miss[k] = v[k] >= 0 ? a.lanes & ~__ldcg(a.seen + v[k]) : 0ull;
+                f2[k] = miss[k] ? __ldg(a.first2 + v[k]) : make_int2(-1, -1);
+            }
+#pragma unroll
+            for (int k = 0; k < PER; ++k) {
+                acc[k] = f2[k].x >= 0 ? __ldca(cin + f2[k].x) : 0ull;
+                acc[k] |= f2[k].y >= 0 ? __ldca(cin + f2[k].y) : 0ull;
+                if (STATS) c.gathered += (f2[k].x >= 0 ? 1 : 0) + (f2[k].y >= 0 ? 1 : 0);
+            }
+            if (STATS && lane == 0) c.rows += (unsigned long long)min((int64_t)MS_ROWS, a.n_active - ch * MS_ROWS);
+            bool open = false;
+            int nh = 0;
+#pragma unroll
+            for (int k = 0; k < PER; ++k) {
+                acc[k] &= miss[k];
+                const bool more = (miss[k] & ~acc[k]) != 0ull && deg[k] > 2;
+                const unsigned int m = __ballot_sync(GRX_FULL_MASK, more);
+                if (more) {
+                    const int h = nh + __popc(m & lanemask_lt());
+                    w.s[h] = s[k];
+                    w.deg[h] = deg[k];
+                    w.i[h] = (int32_t)(ch * MS_ROWS + k * 32 + lane);
+                    w.v[h] = v[k];
+                    w.miss[h] = miss[k];
+                    w.acc[h] = acc[k];
+                } else {
+                    if (miss[k] & ~acc[k]) open = true;          // lanes still missing after this level
+                    if (acc[k]) {
+                        cout[v[k]] = acc[k];
+                        ms_pull_finish(a.seen, hs, v[k], a.lanes & ~miss[k], acc[k], deg[k], c);
+                    }
+                }
+                nh += __popc(m);
+            }
+            __syncwarp();
+            // the open rows: eight lanes a row, 32 edges a step
+            const unsigned int gi = lane >> 3, gl = lane & 7, gmask = 0xffu << (gi * 8);
+            for (int h = (int)gi; h < nh; h += 4) {
+                const uint32_t len = w.deg[h], end = min(len, 2 + MS_HEAD);
+                const int64_t e0 = w.s[h];
+                const unsigned long long ms = w.miss[h];
+                unsigned long long ac = w.acc[h];
+                for (uint32_t at = 2; at < end && (ms & ~ac); at += 32) {
+                    int32_t u[4];
+                    unsigned long long g[4];
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) u[j] = at + j * 8 + gl < end ? __ldg(a.col + e0 + at + j * 8 + gl) : -1;
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) g[j] = u[j] >= 0 ? __ldca(cin + u[j]) : 0ull;
+                    if (STATS) {
+#pragma unroll
+                        for (int j = 0; j < 4; ++j) c.gathered += u[j] >= 0 ? 1ull : 0ull;
+                    }
+                    unsigned long long x = (g[0] | g[1]) | (g[2] | g[3]);
+#pragma unroll
+                    for (int o = 4; o > 0; o >>= 1) x |= __shfl_xor_sync(gmask, x, o);
+                    ac |= x & ms;
+                }
+                const bool left = (ms & ~ac) != 0ull;
+                if (left) open = true;
+                if (gl == 0) {
+                    const int32_t vv = w.v[h];
+                    if (left && len > end) {                     // the rest of the row, in pieces
+                        const uint32_t np = (len - end + MS_PIECE - 1) / MS_PIECE;
+                        const unsigned int base = atomicAdd(rctr, np);
+                        for (uint32_t k = 0; k < np; ++k) a.rest[base + k] = make_int2(w.i[h], (int)k);
+                        if (ac) a.next[vv] = ac;
+                    } else if (ac) {
+                        cout[vv] = ac;
+                        ms_pull_finish(a.seen, hs, vv, a.lanes & ~ms, ac, len, c);
+                    }
+                }
+            }
+            // a row that goes on in pieces counts as open: the flag may stay clear
+            // one level longer than needed, never the other way
+            open = __any_sync(GRX_FULL_MASK, open);
+            if (lane == 0 && !open) a.sat[ch] = 1;
         }
-        if (open) s_open = 1;
-        __syncthreads();
-        // a crossing row's lanes from other tiles are not known here: the flag
-        // may stay clear one level longer than needed, never the other way
-        if (threadIdx.x == 0 && !s_open) a.sat[tile] = 1;
+        ch = nwarps + __shfl_sync(GRX_FULL_MASK, nn, 0);
     }
 }
 
-// Pull, phase 2: rows that cross tiles, finished by the tile holding their
-// last edge.
+// Pull, phase 2: the pieces of rows that are still open; what other pieces found
+// meanwhile is taken into account.
+template <typename OffT, bool STATS>
+__device__ void ms_pull_rest(const MsArgs<OffT> &a, const MsState &st, MsCounts &c) {
+    const unsigned int lane = threadIdx.x & 31;
+    const unsigned long long *cin = pk3(a.cur[0], a.cur[1], a.cur[2], st.L % 3);
+    const int64_t n = ld_relaxed_u32(&a.ctl->ucount[(st.L + 1) & 3]);
+    const int64_t nwarps = (int64_t)gridDim.x * MS_WARPS;
+    for (int64_t t = (int64_t)blockIdx.x * MS_WARPS + (threadIdx.x >> 5); t < n; t += nwarps) {
+        const int2 r = __ldcg(a.rest + t);
+        const int32_t v = __ldg(a.active + r.x);
+        const int64_t e0 = (int64_t)__ldg(a.aoff + r.x) + 2 + MS_HEAD + (int64_t)r.y * MS_PIECE;
+        const int64_t e1 = min((int64_t)__ldg(a.aoff + r.x + 1), e0 + MS_PIECE);
+        const unsigned long long ms = a.lanes & ~__ldcg(a.seen + v) & ~__ldcg(a.next + v);
+        unsigned long long ac = 0ull;
+        for (int64_t at = e0; at < e1 && (ms & ~ac); at += 256) {
+            int32_t u[8];
+            unsigned long long x = 0ull;
+#pragma unroll
+            for (int j = 0; j < 8; ++j) u[j] = at + j * 32 + lane < e1 ? __ldg(a.col + at + j * 32 + lane) : -1;
+#pragma unroll
+            for (int j = 0; j < 8; ++j) {
+                x |= u[j] >= 0 ? __ldca(cin + u[j]) : 0ull;
+                if (STATS) c.gathered += u[j] >= 0 ? 1ull : 0ull;
+            }
+            const uint32_t lo = __reduce_or_sync(GRX_FULL_MASK, (uint32_t)x);
+            const uint32_t hi = __reduce_or_sync(GRX_FULL_MASK, (uint32_t)(x >> 32));
+            ac |= (((unsigned long long)hi << 32) | lo) & ms;
+        }
+        if (lane == 0 && ac) atomicOr(a.next + v, ac);
+    }
+}
+
+// Pull, phase 3: the rows of the pieces, finished at their first one.
 template <typename OffT>
 __device__ void ms_pull_fixup(const MsArgs<OffT> &a, const MsState &st, MsCounts &c) {
     const int L = st.L;
     unsigned long long *cout = pk3(a.cur[0], a.cur[1], a.cur[2], (L + 1) % 3);
     unsigned long long *hs = a.hist[st.flush ? 0 : st.hslots];
-    for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < a.ntiles;
-         t += (int64_t)gridDim.x * blockDim.x) {
-        const int32_t v = __ldcg(a.fix + t);
-        if (v < 0) continue;
+    const int64_t n = ld_relaxed_u32(&a.ctl->ucount[(L + 1) & 3]);
+    for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < n; t += (int64_t)gridDim.x * blockDim.x) {
+        const int2 r = __ldcg(a.rest + t);
+        if (r.y != 0) continue;
+        const int32_t v = __ldg(a.active + r.x);
         const unsigned long long acc = __ldcg(a.next + v);
         if (acc) a.next[v] = 0ull;
         const unsigned long long sv = __ldcg(a.seen + v);
         const unsigned long long nw = acc & a.lanes & ~sv;
         if (nw) {
             cout[v] = nw;
-            ms_pull_finish(a.seen, hs, v, sv, nw, (uint32_t)(__ldg(a.ro + v + 1) - __ldg(a.ro + v)), c);
+            ms_pull_finish(a.seen, hs, v, sv, nw, __ldg(a.aoff + r.x + 1) - __ldg(a.aoff + r.x), c);
         }
     }
 }
@@ -643,18 +650,21 @@ __device__ void ms_pull_fixup(const MsArgs<OffT> &a, const MsState &st, MsCounts
 // the slots are cleared.  The final flush also writes -1 for every pair that
 // was never reached.  Masks are split into 32-bit halves so the per-lane
 // tests are single-word operations.
-template <typename OffT>
-__device__ void ms_flush(const MsArgs<OffT> &a, int nslots, const int32_t *slot_depth, bool final) {
-    int32_t sd[MS_HSLOTS];
+// NS: history slots looked at (a lane's depth takes a test per slot, and the
+// output's 4 * lanes * V bytes leave time for few of them).
+template <typename OffT, int NS>
+__device__ __forceinline__ void ms_flush_slots(const MsArgs<OffT> &a, int nslots, const int32_t *slot_depth,
+                                               bool final) {
+    int32_t sd[NS];
 #pragma unroll
-    for (int s = 0; s < MS_HSLOTS; ++s) sd[s] = s < nslots ? slot_depth[s] : 0;
+    for (int s = 0; s < NS; ++s) sd[s] = s < nslots ? slot_depth[s] : 0;
     const int nlo = min(a.n, 32);
     for (int64_t v = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; v < a.nv;
          v += (int64_t)gridDim.x * blockDim.x) {
-        uint32_t hl[MS_HSLOTS], hh[MS_HSLOTS];
+        uint32_t hl[NS], hh[NS];
         unsigned long long any = 0ull;
 #pragma unroll
-        for (int s = 0; s < MS_HSLOTS; ++s) {
+        for (int s = 0; s < NS; ++s) {
             const unsigned long long h = s < nslots ? __ldcg(a.hist[s] + v) : 0ull;
             if (h) a.hist[s][v] = 0ull;
             hl[s] = (uint32_t)h;
@@ -672,16 +682,24 @@ __device__ void ms_flush(const MsArgs<OffT> &a, int nslots, const int32_t *slot_
         for (int b = 0; b < nlo; ++b) {
             int d = (ul >> b & 1u) ? -1 : -2;
 #pragma unroll
-            for (int s = 0; s < MS_HSLOTS; ++s) d = (hl[s] >> b & 1u) ? sd[s] : d;
+            for (int s = 0; s < NS; ++s) d = (hl[s] >> b & 1u) ? sd[s] : d;
             if (d != -2) out[(int64_t)b * a.nv] = d;
         }
         for (int b = 32; b < a.n; ++b) {
             int d = (uh >> (b - 32) & 1u) ? -1 : -2;
 #pragma unroll
-            for (int s = 0; s < MS_HSLOTS; ++s) d = (hh[s] >> (b - 32) & 1u) ? sd[s] : d;
+            for (int s = 0; s < NS; ++s) d = (hh[s] >> (b - 32) & 1u) ? sd[s] : d;
             if (d != -2) out[(int64_t)b * a.nv] = d;
         }
     }
+}
+
+template <typename OffT>
+__device__ void ms_flush(const MsArgs<OffT> &a, int nslots, const int32_t *slot_depth, bool final) {
+    if (nslots <= 2) ms_flush_slots<OffT, 2>(a, nslots, slot_depth, final);
+    else if (nslots <= 3) ms_flush_slots<OffT, 3>(a, nslots, slot_depth, final);
+    else if (nslots <= 4) ms_flush_slots<OffT, 4>(a, nslots, slot_depth, final);
+    else ms_flush_slots<OffT, MS_HSLOTS>(a, nslots, slot_depth, final);
 }
 
 template <typename OffT, bool STATS>
@@ -717,7 +735,7 @@ __global__ void __launch_bounds__(MS_BLOCK, GRX_MS_MIN_BLOCKS) k_msbfs_persisten
     }
     __syncthreads();
     for (;;) {
-        const MsState st = s_st;
+        const MsState &st = s_st;
         if (st.done) break;
         const int L = st.L;
         const int op = ms_op(st);
@@ -726,6 +744,7 @@ __global__ void __launch_bounds__(MS_BLOCK, GRX_MS_MIN_BLOCKS) k_msbfs_persisten
             if (st.phase == 0) {
                 a.ctl->qpack[(L + 2) & 3] = 0ull;
                 a.ctl->ucount[(L + 2) & 3] = 0u;
+                a.ctl->wq[(L + 2) & 3] = 0u;
                 a.ctl->pairs[(L + 2) & 3] = 0ull;
                 if (STATS && L < GRX_MAX_LEVELS_STATS) {
                     a.stats->level_t0[L] = grx_globaltimer();
@@ -749,7 +768,8 @@ __global__ void __launch_bounds__(MS_BLOCK, GRX_MS_MIN_BLOCKS) k_msbfs_persisten
             ms_flush<OffT>(a, MS_HSLOTS, st.slot_depth, false);
         } else {
             MsCounts c = {0ull, 0ull, 0ull, 0ull, 0ull};
-            if (op == MOP_PULL) ms_pull<OffT, STATS>(a, st, sm.p, c);
+            if (op == MOP_PULL) ms_pull<OffT, STATS>(a, st, sm.p[threadIdx.x >> 5], c);
+            else if (op == MOP_REST) ms_pull_rest<OffT, STATS>(a, st, c);
             else ms_pull_fixup<OffT>(a, st, c);
             c.q = warp_sum(c.q);
             c.T = warp_sum(c.T);
@@ -764,7 +784,7 @@ __global__ void __launch_bounds__(MS_BLOCK, GRX_MS_MIN_BLOCKS) k_msbfs_persisten
                 if (STATS && c.gathered && L < GRX_MAX_LEVELS_STATS)
                     atomicAdd(&a.stats->edges_examined[L], c.gathered);
                 if (STATS && c.rows && L < GRX_MAX_LEVELS_STATS)
-                    atomicAdd(&a.stats->vertices_scanned[L], c.rows);   // rows of the tiles not skipped
+                    atomicAdd(&a.stats->vertices_scanned[L], c.rows);   // rows not skipped
             }
         }
         if (!flag_barrier(bar)) return;
@@ -784,6 +804,13 @@ __global__ void __launch_bounds__(MS_BLOCK, GRX_MS_MIN_BLOCKS) k_msbfs_persisten
     }
 }
 
+size_t ms_sat_bytes(const grx_graph *g) { return (size_t)((g->n_active + MS_ROWS - 1) / MS_ROWS) + 1; }
+
+// Pieces of the rows longer than 2 + MS_HEAD, at most.
+size_t ms_rest_bytes(const grx_graph *g) {
+    return (size_t)(g->ne / (MS_HEAD + 3) + g->ne / MS_PIECE + 1) * sizeof(int2);
+}
+
 template <typename OffT, bool STATS>
 grx_status ms_launch_typed(grx_graph *g, const int32_t *srcs, int n, int32_t *depth,
                            const grx_opts *o, cudaStream_t s) {
@@ -794,22 +821,18 @@ grx_status ms_launch_typed(grx_graph *g, const int32_t *srcs, int n, int32_t *de
     a.col = g->col;
     a.active = g->active;
     a.aoff = g->aoff;
-    a.ntiles = (g->ne + MS_PTILE - 1) / MS_PTILE;
-    a.tiles = nullptr;
-    if (a.ntiles > 0) {
-        grx_status st = grx_edge_tiles(g, MS_PTILE, s, &a.tiles);
-        if (st != GRX_OK) return st;
-    }
-    if (!g->ms_fix) {
-        g->ms_sat = (uint8_t *)grx_alloc(g, (size_t)(a.ntiles > 0 ? a.ntiles : 1), s);
-        g->ms_fix = g->ms_sat ? (int32_t *)grx_alloc(g, (size_t)(a.ntiles > 0 ? a.ntiles : 1) * 4, s) : nullptr;
-        for (int i = 0; i < MS_HSLOTS && g->ms_fix; ++i) {
+    a.first2 = g->first2;
+    a.n_active = g->n_active;
+    if (!g->ms_rest) {
+        g->ms_sat = (uint8_t *)grx_alloc(g, ms_sat_bytes(g), s);
+        g->ms_rest = g->ms_sat ? (int2 *)grx_alloc(g, ms_rest_bytes(g), s) : nullptr;
+        for (int i = 0; i < MS_HSLOTS && g->ms_rest; ++i) {
             g->ms_hist[i] = (unsigned long long *)grx_alloc(g, (size_t)g->nv * 8, s);
             if (!g->ms_hist[i]) return grx_fail(GRX_ENOMEM, "bfs_multi: history slot allocation failed");
         }
-        if (!g->ms_fix) return grx_fail(GRX_ENOMEM, "bfs_multi: workspace allocation failed");
+        if (!g->ms_rest) return grx_fail(GRX_ENOMEM, "bfs_multi: workspace allocation failed");
     }
-    a.fix = g->ms_fix;
+    a.rest = g->ms_rest;
     a.sat = g->ms_sat;
     for (int i = 0; i < MS_HSLOTS; ++i) a.hist[i] = g->ms_hist[i];
     a.n = n;
@@ -868,13 +891,7 @@ grx_status ms_launch_typed(grx_graph *g, const int32_t *srcs, int n, int32_t *de
 
 size_t grx_msbfs_new_bytes(const grx_graph *g) {
     size_t b = 0;
-    const int64_t ntiles = (g->ne + MS_PTILE - 1) / MS_PTILE;
-    const size_t nt = (size_t)(ntiles > 0 ? ntiles : 1);
-    bool have_tiles = false;
-    for (int i = 0; i < (int)(sizeof g->etiles / sizeof g->etiles[0]); ++i)
-        if (g->etiles[i] && g->etile_size[i] == MS_PTILE) have_tiles = true;
-    if (ntiles > 0 && !have_tiles) b += nt * sizeof(int2);
-    if (!g->ms_fix) b += nt + nt * 4 + (size_t)MS_HSLOTS * (size_t)g->nv * 8;
+    if (!g->ms_rest) b += ms_sat_bytes(g) + ms_rest_bytes(g) + (size_t)MS_HSLOTS * (size_t)g->nv * 8;
     if (!g->ms_tbits) b += (size_t)g->words * 4 + 16;
     return b;
 }
