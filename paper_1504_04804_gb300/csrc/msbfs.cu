@@ -21,8 +21,8 @@
 //    (first2), a lane per row; then eight lanes per row, 32 edges a step.  Rows
 //    still open after MS_HEAD edges leave the rest to a second phase, in pieces
 //    of 1,024 edges over the grid, and are finished by a third.
-//  * Depths found by pull levels are not written per level: the level's new
-//    lane masks go to one of MS_HSLOTS history slots, and a flush pass
+//  * Depths found by pull levels and large push levels are not written per level:
+//    the level's new lane masks go to one of MS_HSLOTS history slots, and a flush pass
 //    writes them lane-major with coalesced stores (and, at the end, -1 for
 //    every pair never reached, so the output needs no initial fill).
 //  * cur rotates through three buffers: level L reads cur[L%3] and writes
@@ -42,7 +42,7 @@
 
 namespace {
 
-constexpr int MS_BLOCK = 256;
+constexpr int MS_BLOCK = 384;
 constexpr int MS_WARPS = MS_BLOCK / 32;
 constexpr int MS_ITEMS = 8;
 constexpr int MS_WTILE = 32 * MS_ITEMS;             // push: edges per warp tile
@@ -53,9 +53,8 @@ constexpr int MS_ROWS = 128;                        // pull: rows a warp takes a
 constexpr uint32_t MS_HEAD = 126;
 constexpr uint32_t MS_PIECE = 1024;                 // pull: edges of a piece of the second phase
 constexpr int MS_HSLOTS = 6;                        // history slots of pull levels
-#ifndef GRX_MS_MIN_BLOCKS
-#define GRX_MS_MIN_BLOCKS 3                         // resident blocks per SM (register cap)
-#endif
+constexpr int MS_MIN_BLOCKS = 2;                    // resident blocks per SM (register cap; two of 384 threads
+                                                    // against three of 256: 1 % at R-MAT 20 to 24)
 
 enum { DIR_PUSH = 0, DIR_PULL = 1 };
 enum { MOP_COMPACT, MOP_EXPAND, MOP_FINAL, MOP_FLUSH, MOP_PULL, MOP_REST, MOP_FIXUP };
@@ -103,6 +102,7 @@ struct MsState {
     uint8_t hslots;     // history slots holding pull levels' masks
     uint8_t flush;      // this pull level starts with a flush (slots full)
     uint8_t bmp;        // push level that marks touched vertices in a bitmap
+    uint8_t keep;       // push level whose new lanes go to a history slot
     int32_t slot_depth[MS_HSLOTS];
     uint32_t q, T;      // |Q_L| and its edge count
     unsigned long long seen_pairs;    // (vertex, lane) pairs labelled so far
@@ -152,6 +152,7 @@ __device__ __forceinline__ void ms_set_kind(const MsArgs<OffT> &a, MsState &s) {
     s.compact = s.dir == DIR_PUSH && !s.qin;
     s.flush = s.dir == DIR_PULL && s.hslots >= MS_HSLOTS;
     s.bmp = s.dir == DIR_PUSH && s.T >= a.bmp_min_T;
+    s.keep = s.bmp && !s.back && s.hslots < MS_HSLOTS;   // after the pulls little is found
 }
 
 // Label the new lanes of v at depth d in the lane-major depth output.
@@ -179,7 +180,7 @@ __device__ MsState ms_next_state(const MsArgs<OffT> &a, const MsState &st, bool 
     ns.q = (uint32_t)(pk >> 32);
     ns.T = (uint32_t)pk;
     ns.qin = st.dir == DIR_PUSH;
-    if (st.dir == DIR_PULL) {
+    if (st.dir == DIR_PULL || st.keep) {
         const int h = st.flush ? 0 : st.hslots;
         ns.slot_depth[h] = st.L + 1;
         ns.hslots = (uint8_t)(h + 1);
@@ -362,9 +363,10 @@ __device__ void ms_push_expand(const MsArgs<OffT> &a, const MsState &st, MsWarpS
 }
 
 // A touched vertex v (or -1): its next mask becomes its new lanes (labelled
-// here) and, with edges, a slot of the next frontier.  All 32 lanes call.
+// here, or left in the history slot hs) and, with edges, a slot of the next
+// frontier.  All 32 lanes call.
 template <typename OffT>
-__device__ __forceinline__ void ms_touched(const MsArgs<OffT> &a, int L, int32_t vv,
+__device__ __forceinline__ void ms_touched(const MsArgs<OffT> &a, int L, int32_t vv, unsigned long long *hs,
                                            unsigned long long *cout, int32_t *Qv_out,
                                            uint32_t *Qe_out, OffT *Qr_out, unsigned long long *ctr,
                                            unsigned long long &found) {
@@ -380,7 +382,8 @@ __device__ __forceinline__ void ms_touched(const MsArgs<OffT> &a, int L, int32_t
         if (nw) {
             a.seen[vv] = sv | nw;
             cout[vv] = nw;
-            write_depths(a.depth, a.nv, vv, nw, L + 1);
+            if (hs) hs[vv] = nw;
+            else write_depths(a.depth, a.nv, vv, nw, L + 1);
             found += (unsigned long long)__popcll(nw);
             rb[0] = __ldg(a.ro + vv);
             deg[0] = (uint32_t)(__ldg(a.ro + vv + 1) - rb[0]);
@@ -400,6 +403,7 @@ __device__ void ms_push_finalize(const MsArgs<OffT> &a, const MsState &st, uint1
     uint32_t *Qe_out = pk3(a.E[0], a.E[1], a.E[2], (L + 1) % 3);
     OffT *Qr_out = pk3(a.R[0], a.R[1], a.R[2], (L + 1) % 3);
     unsigned long long *ctr = &a.ctl->qpack[(L + 1) & 3];
+    unsigned long long *hs = st.keep ? a.hist[st.hslots] : nullptr;
     unsigned long long found = 0;
     if (st.bmp) {
         const unsigned int lane = threadIdx.x & 31;
@@ -412,7 +416,7 @@ __device__ void ms_push_finalize(const MsArgs<OffT> &a, const MsState &st, uint1
             const int n = warp_compact_bits(bits, list);
             for (int base = 0; base < n; base += 32) {
                 const int i = base + (int)lane;
-                ms_touched<OffT>(a, L, i < n ? (int32_t)(sc * 1024 + list[i]) : -1, cout, Qv_out, Qe_out,
+                ms_touched<OffT>(a, L, i < n ? (int32_t)(sc * 1024 + list[i]) : -1, hs, cout, Qv_out, Qe_out,
                                  Qr_out, ctr, found);
             }
             __syncwarp();
@@ -422,7 +426,7 @@ __device__ void ms_push_finalize(const MsArgs<OffT> &a, const MsState &st, uint1
         const int64_t span = (count + 31) & ~(int64_t)31;
         for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < span;
              i += (int64_t)gridDim.x * blockDim.x)
-            ms_touched<OffT>(a, L, i < count ? __ldcg(a.touched + i) : -1, cout, Qv_out, Qe_out, Qr_out,
+            ms_touched<OffT>(a, L, i < count ? __ldcg(a.touched + i) : -1, hs, cout, Qv_out, Qe_out, Qr_out,
                              ctr, found);
     }
     found = warp_sum(found);
@@ -652,58 +656,71 @@ __device__ void ms_pull_fixup(const MsArgs<OffT> &a, const MsState &st, MsCounts
 // tests are single-word operations.
 // NS: history slots looked at (a lane's depth takes a test per slot, and the
 // output's 4 * lanes * V bytes leave time for few of them).
-template <typename OffT, int NS>
+template <typename OffT, int NS, int VW>
 __device__ __forceinline__ void ms_flush_slots(const MsArgs<OffT> &a, int nslots, const int32_t *slot_depth,
                                                bool final) {
     int32_t sd[NS];
 #pragma unroll
     for (int s = 0; s < NS; ++s) sd[s] = s < nslots ? slot_depth[s] : 0;
-    const int nlo = min(a.n, 32);
-    for (int64_t v = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; v < a.nv;
-         v += (int64_t)gridDim.x * blockDim.x) {
-        uint32_t hl[NS], hh[NS];
-        unsigned long long any = 0ull;
+    // VW consecutive vertices a thread: 16-byte stores where every lane's row of the
+    // output starts on such a boundary
+    for (int64_t v0 = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) * VW; v0 < a.nv;
+         v0 += (int64_t)gridDim.x * blockDim.x * VW) {
+        for (int half = 0; half * 32 < a.n; ++half) {    // 32 lanes at a time
+            uint32_t h[NS][VW], un[VW], any = 0u;
 #pragma unroll
-        for (int s = 0; s < NS; ++s) {
-            const unsigned long long h = s < nslots ? __ldcg(a.hist[s] + v) : 0ull;
-            if (h) a.hist[s][v] = 0ull;
-            hl[s] = (uint32_t)h;
-            hh[s] = (uint32_t)(h >> 32);
-            any |= h;
-        }
-        const unsigned long long unseen = final ? (a.lanes & ~__ldcg(a.seen + v)) : 0ull;
-        if (!(any | unseen)) continue;
-        int32_t *out = a.depth + v;
-        if (!any && unseen == a.lanes) {             // reached by no lane
-            for (int b = 0; b < a.n; ++b) out[(int64_t)b * a.nv] = -1;
-            continue;
-        }
-        const uint32_t ul = (uint32_t)unseen, uh = (uint32_t)(unseen >> 32);
-        for (int b = 0; b < nlo; ++b) {
-            int d = (ul >> b & 1u) ? -1 : -2;
+            for (int i = 0; i < VW; ++i) {
+                un[i] = final ? (uint32_t)(a.lanes >> (32 * half)) & ~__ldcg((const uint32_t *)(a.seen + v0 + i) + half)
+                              : 0u;
+                any |= un[i];
 #pragma unroll
-            for (int s = 0; s < NS; ++s) d = (hl[s] >> b & 1u) ? sd[s] : d;
-            if (d != -2) out[(int64_t)b * a.nv] = d;
-        }
-        for (int b = 32; b < a.n; ++b) {
-            int d = (uh >> (b - 32) & 1u) ? -1 : -2;
+                for (int s = 0; s < NS; ++s) {
+                    uint32_t *p = (uint32_t *)(a.hist[s] + v0 + i) + half;
+                    h[s][i] = s < nslots ? __ldcg(p) : 0u;
+                    any |= h[s][i];
+                    if (h[s][i]) *p = 0u;
+                }
+            }
+            if (!any) continue;
+            const int last = min(a.n, 32 * half + 32);
+            int32_t *out = a.depth + (int64_t)(32 * half) * a.nv + v0;
+            for (int b = 32 * half; b < last; ++b, out += a.nv) {
+                int d[VW];
+                bool all = true;
 #pragma unroll
-            for (int s = 0; s < NS; ++s) d = (hh[s] >> (b - 32) & 1u) ? sd[s] : d;
-            if (d != -2) out[(int64_t)b * a.nv] = d;
+                for (int i = 0; i < VW; ++i) {
+                    d[i] = (un[i] & 1u) ? -1 : -2;       // -2: written by a push level
+                    un[i] >>= 1;
+#pragma unroll
+                    for (int s = 0; s < NS; ++s) {
+                        d[i] = (h[s][i] & 1u) ? sd[s] : d[i];
+                        h[s][i] >>= 1;
+                    }
+                    all = all && d[i] != -2;
+                }
+                if (VW == 4 && all) {
+                    *reinterpret_cast<int4 *>(out) = make_int4(d[0], d[1 % VW], d[2 % VW], d[3 % VW]);
+                } else {
+#pragma unroll
+                    for (int i = 0; i < VW; ++i)
+                        if (d[i] != -2) out[i] = d[i];
+                }
+            }
         }
     }
 }
 
 template <typename OffT>
 __device__ void ms_flush(const MsArgs<OffT> &a, int nslots, const int32_t *slot_depth, bool final) {
-    if (nslots <= 2) ms_flush_slots<OffT, 2>(a, nslots, slot_depth, final);
-    else if (nslots <= 3) ms_flush_slots<OffT, 3>(a, nslots, slot_depth, final);
-    else if (nslots <= 4) ms_flush_slots<OffT, 4>(a, nslots, slot_depth, final);
-    else ms_flush_slots<OffT, MS_HSLOTS>(a, nslots, slot_depth, final);
+    const bool wide = (a.nv & 3) == 0 && ((uintptr_t)a.depth & 15) == 0;
+    if (!wide) ms_flush_slots<OffT, MS_HSLOTS, 1>(a, nslots, slot_depth, final);
+    else if (nslots <= 3) ms_flush_slots<OffT, 3, 4>(a, nslots, slot_depth, final);
+    else if (nslots <= 4) ms_flush_slots<OffT, 4, 4>(a, nslots, slot_depth, final);
+    else ms_flush_slots<OffT, MS_HSLOTS, 4>(a, nslots, slot_depth, final);
 }
 
 template <typename OffT, bool STATS>
-__global__ void __launch_bounds__(MS_BLOCK, GRX_MS_MIN_BLOCKS) k_msbfs_persistent(MsArgs<OffT> a) {
+__global__ void __launch_bounds__(MS_BLOCK, MS_MIN_BLOCKS) k_msbfs_persistent(MsArgs<OffT> a) {
     __shared__ MsState s_st;
     __shared__ int s_dirty;
     __shared__ MsSmem<OffT> sm;
@@ -875,7 +892,7 @@ grx_status ms_launch_typed(grx_graph *g, const int32_t *srcs, int n, int32_t *de
     }
     int max_grid = per_sm * g->ctx->num_sms;
     if (max_grid > GRX_MAX_GRID) max_grid = GRX_MAX_GRID;
-    int blocks = o->grid_blocks > 0 && o->grid_blocks < max_grid ? o->grid_blocks : max_grid;
+    const int blocks = grx_grid(o, MS_BLOCK, max_grid);
     GRX_CUDA(cudaMemsetAsync(g->bar_flags, 0, sizeof(unsigned int) * (size_t)blocks, s));
     GRX_CUDA(cudaMemsetAsync(&g->ctl->bar_release, 0, sizeof(unsigned int), s));
     if (o->collect_stats) GRX_CUDA(cudaMemsetAsync(g->stats, 0, sizeof(DevStats), s));
