@@ -46,11 +46,12 @@ constexpr int MS_BLOCK = 384;
 constexpr int MS_WARPS = MS_BLOCK / 32;
 constexpr int MS_ITEMS = 8;
 constexpr int MS_WTILE = 32 * MS_ITEMS;             // push: edges per warp tile
-constexpr int MS_ROWS = 128;                        // pull: rows a warp takes at a time
+constexpr int MS_ROWS = 128;                        // pull: rows a warp takes at a time, at most
 // Pull: edges of a row in the first phase, after its first two (64 sources, R-MAT
 // 24 / 22 / 20: 30 7.58 / 2.27 / 0.82 ms, 126 7.02 / 2.16 / 0.89, 254 7.12 / 2.30 /
 // 0.98, 510 7.37 / 2.57 / 1.16).
 constexpr uint32_t MS_HEAD = 126;
+constexpr uint32_t MS_WARP_ROW = 2048;              // pull, small graphs: rows up to this stay in the first phase
 constexpr uint32_t MS_PIECE = 1024;                 // pull: edges of a piece of the second phase
 constexpr int MS_HSLOTS = 6;                        // history slots of pull levels
 constexpr int MS_MIN_BLOCKS = 2;                    // resident blocks per SM (register cap; two of 384 threads
@@ -77,7 +78,8 @@ struct MsArgs {
     unsigned long long *cur[3];
     unsigned long long *hist[MS_HSLOTS];
     int2 *rest;                       // pieces of open rows: (active row, piece)
-    uint8_t *sat;                     // per MS_ROWS rows: every one has all lanes seen
+    int rows;                         // pull: rows a warp takes at a time
+    uint8_t *sat;                     // per `rows` rows: every one has all lanes seen
     int32_t *Q[3];
     uint32_t *E[3];
     OffT *R[3];
@@ -232,7 +234,7 @@ __device__ void ms_init_fill(const MsArgs<OffT> &a, bool dirty) {
     }
     if (dirty)
         for (int64_t w = tid; w < a.words; w += stride) a.tbits[w] = 0u;
-    for (int64_t t = tid; t < (a.n_active + MS_ROWS - 1) / MS_ROWS; t += stride) a.sat[t] = 0;
+    for (int64_t t = tid; t < (a.n_active + a.rows - 1) / a.rows; t += stride) a.sat[t] = 0;
 }
 
 // Phase 1 (one thread): seed the lanes (depth 0), the first frontier
@@ -476,6 +478,25 @@ __device__ __forceinline__ void ms_pull_finish(unsigned long long *seen, unsigne
     c.pairs += (unsigned long long)__popcll(nw);
 }
 
+// OR of the masks of up to 256 neighbours (edges at to e1), by a whole warp.
+template <bool STATS>
+__device__ __forceinline__ unsigned long long ms_gather256(const int32_t *col, const unsigned long long *cin,
+                                                           int64_t at, int64_t e1, MsCounts &c) {
+    const unsigned int lane = threadIdx.x & 31;
+    int32_t u[8];
+    unsigned long long x = 0ull;
+#pragma unroll
+    for (int j = 0; j < 8; ++j) u[j] = at + j * 32 + lane < e1 ? __ldg(col + at + j * 32 + lane) : -1;
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+        x |= u[j] >= 0 ? __ldca(cin + u[j]) : 0ull;
+        if (STATS) c.gathered += u[j] >= 0 ? 1ull : 0ull;
+    }
+    const uint32_t lo = __reduce_or_sync(GRX_FULL_MASK, (uint32_t)x);
+    const uint32_t hi = __reduce_or_sync(GRX_FULL_MASK, (uint32_t)(x >> 32));
+    return ((unsigned long long)hi << 32) | lo;
+}
+
 // Pull, phase 1 (see the head of the file).  With every open row's edges gathered
 // (in equal tiles), the three pull levels of 64 sources on R-MAT 24 took 3.80,
 // 3.43 and 1.02 ms, and take 2.64 (88 % of the neighbours read: few rows find all
@@ -489,7 +510,9 @@ __device__ void ms_pull(const MsArgs<OffT> &a, const MsState &st, MsPullSmem &w,
     unsigned long long *cout = pk3(a.cur[0], a.cur[1], a.cur[2], (L + 1) % 3);
     unsigned long long *hs = a.hist[st.flush ? 0 : st.hslots];
     unsigned int *wq = &a.ctl->wq[L & 3], *rctr = &a.ctl->ucount[(L + 1) & 3];
-    const int64_t nch = (a.n_active + MS_ROWS - 1) / MS_ROWS;
+    const int R = a.rows;
+    const bool small = R < MS_ROWS;              // few rows a warp: it finishes its longer ones itself
+    const int64_t nch = (a.n_active + R - 1) / R;
     const int64_t nwarps = (int64_t)gridDim.x * MS_WARPS;
     for (int64_t ch = (int64_t)blockIdx.x * MS_WARPS + (threadIdx.x >> 5); ch < nch;) {
         unsigned int nn = 0;
@@ -501,10 +524,10 @@ __device__ void ms_pull(const MsArgs<OffT> &a, const MsState &st, MsPullSmem &w,
             int2 f2[PER];
 #pragma unroll
             for (int k = 0; k < PER; ++k) {
-                const int64_t i = ch * MS_ROWS + k * 32 + lane;
+                const int64_t i = ch * R + k * 32 + lane;
                 v[k] = -1;
                 s[k] = deg[k] = 0u;
-                if (i < a.n_active) {
+                if (k * 32 + (int)lane < R && i < a.n_active) {
                     v[k] = __ldg(a.active + i);
                     s[k] = __ldg(a.aoff + i);
                     deg[k] = __ldg(a.aoff + i + 1) - s[k];
@@ -521,7 +544,7 @@ __device__ void ms_pull(const MsArgs<OffT> &a, const MsState &st, MsPullSmem &w,
                 acc[k] |= f2[k].y >= 0 ? __ldca(cin + f2[k].y) : 0ull;
                 if (STATS) c.gathered += (f2[k].x >= 0 ? 1 : 0) + (f2[k].y >= 0 ? 1 : 0);
             }
-            if (STATS && lane == 0) c.rows += (unsigned long long)min((int64_t)MS_ROWS, a.n_active - ch * MS_ROWS);
+            if (STATS && lane == 0) c.rows += (unsigned long long)min((int64_t)R, a.n_active - ch * R);
             bool open = false;
             int nh = 0;
 #pragma unroll
@@ -533,7 +556,7 @@ __device__ void ms_pull(const MsArgs<OffT> &a, const MsState &st, MsPullSmem &w,
                     const int h = nh + __popc(m & lanemask_lt());
                     w.s[h] = s[k];
                     w.deg[h] = deg[k];
-                    w.i[h] = (int32_t)(ch * MS_ROWS + k * 32 + lane);
+                    w.i[h] = (int32_t)(ch * R + k * 32 + lane);
                     w.v[h] = v[k];
                     w.miss[h] = miss[k];
                     w.acc[h] = acc[k];
@@ -570,7 +593,13 @@ __device__ void ms_pull(const MsArgs<OffT> &a, const MsState &st, MsPullSmem &w,
                     for (int o = 4; o > 0; o >>= 1) x |= __shfl_xor_sync(gmask, x, o);
                     ac |= x & ms;
                 }
+                __syncwarp(gmask);                               // the group has read its entry
                 const bool left = (ms & ~ac) != 0ull;
+                if (left && len > end && small && len <= MS_WARP_ROW) {
+                    if (gl == 0) w.acc[h] = ac;                  // the warp together, below
+                    continue;
+                }
+                if (gl == 0) w.deg[h] = 0u;                      // nothing left to do here
                 if (left) open = true;
                 if (gl == 0) {
                     const int32_t vv = w.v[h];
@@ -583,6 +612,21 @@ __device__ void ms_pull(const MsArgs<OffT> &a, const MsState &st, MsPullSmem &w,
                         cout[vv] = ac;
                         ms_pull_finish(a.seen, hs, vv, a.lanes & ~ms, ac, len, c);
                     }
+                }
+            }
+            __syncwarp();
+            for (int h = 0; small && h < nh; ++h) {
+                const uint32_t len = w.deg[h];
+                if (len == 0) continue;
+                const int64_t e0 = w.s[h];
+                const unsigned long long ms = w.miss[h];
+                unsigned long long ac = w.acc[h];
+                for (uint32_t at = 2 + MS_HEAD; at < len && (ms & ~ac); at += 256)
+                    ac |= ms_gather256<STATS>(a.col, cin, e0 + at, e0 + len, c) & ms;
+                if (ms & ~ac) open = true;
+                if (lane == 0 && ac) {
+                    cout[w.v[h]] = ac;
+                    ms_pull_finish(a.seen, hs, w.v[h], a.lanes & ~ms, ac, len, c);
                 }
             }
             // a row that goes on in pieces counts as open: the flag may stay clear
@@ -609,20 +653,8 @@ __device__ void ms_pull_rest(const MsArgs<OffT> &a, const MsState &st, MsCounts 
         const int64_t e1 = min((int64_t)__ldg(a.aoff + r.x + 1), e0 + MS_PIECE);
         const unsigned long long ms = a.lanes & ~__ldcg(a.seen + v) & ~__ldcg(a.next + v);
         unsigned long long ac = 0ull;
-        for (int64_t at = e0; at < e1 && (ms & ~ac); at += 256) {
-            int32_t u[8];
-            unsigned long long x = 0ull;
-#pragma unroll
-            for (int j = 0; j < 8; ++j) u[j] = at + j * 32 + lane < e1 ? __ldg(a.col + at + j * 32 + lane) : -1;
-#pragma unroll
-            for (int j = 0; j < 8; ++j) {
-                x |= u[j] >= 0 ? __ldca(cin + u[j]) : 0ull;
-                if (STATS) c.gathered += u[j] >= 0 ? 1ull : 0ull;
-            }
-            const uint32_t lo = __reduce_or_sync(GRX_FULL_MASK, (uint32_t)x);
-            const uint32_t hi = __reduce_or_sync(GRX_FULL_MASK, (uint32_t)(x >> 32));
-            ac |= (((unsigned long long)hi << 32) | lo) & ms;
-        }
+        for (int64_t at = e0; at < e1 && (ms & ~ac); at += 256)
+            ac |= ms_gather256<STATS>(a.col, cin, at, e1, c) & ms;
         if (lane == 0 && ac) atomicOr(a.next + v, ac);
     }
 }
@@ -821,7 +853,20 @@ __global__ void __launch_bounds__(MS_BLOCK, MS_MIN_BLOCKS) k_msbfs_persistent(Ms
     }
 }
 
-size_t ms_sat_bytes(const grx_graph *g) { return (size_t)((g->n_active + MS_ROWS - 1) / MS_ROWS) + 1; }
+// Rows a warp of the pull takes at a time: 128, or on small graphs what gives
+// every warp some, down to four (one per eight lanes).  3,800 vertices, 48 sources:
+// 294 us with 128, 191 so, and 157 since these warps finish rows of up to 2,048
+// edges themselves instead of leaving them to two more phases.
+int ms_rows(const grx_graph *g, int blocks) {
+    int r = MS_ROWS;
+    while (r > 4 && g->n_active < (int64_t)blocks * MS_WARPS * r) r /= 2;
+    return r;
+}
+
+// One flag per ms_rows rows: fewer than two per warp where these are not MS_ROWS.
+size_t ms_sat_bytes(const grx_graph *g) {
+    return (size_t)(g->n_active / MS_ROWS) + 1 + 2 * (size_t)GRX_MAX_GRID * MS_WARPS;
+}
 
 // Pieces of the rows longer than 2 + MS_HEAD, at most.
 size_t ms_rest_bytes(const grx_graph *g) {
@@ -893,6 +938,7 @@ grx_status ms_launch_typed(grx_graph *g, const int32_t *srcs, int n, int32_t *de
     int max_grid = per_sm * g->ctx->num_sms;
     if (max_grid > GRX_MAX_GRID) max_grid = GRX_MAX_GRID;
     const int blocks = grx_grid(o, MS_BLOCK, max_grid);
+    a.rows = ms_rows(g, blocks);
     GRX_CUDA(cudaMemsetAsync(g->bar_flags, 0, sizeof(unsigned int) * (size_t)blocks, s));
     GRX_CUDA(cudaMemsetAsync(&g->ctl->bar_release, 0, sizeof(unsigned int), s));
     if (o->collect_stats) GRX_CUDA(cudaMemsetAsync(g->stats, 0, sizeof(DevStats), s));
