@@ -22,7 +22,7 @@
 
 namespace {
 
-constexpr int CC_BLOCK = 256;
+constexpr int CC_BLOCK = 1024;                // (1,216 blocks of 256 in every grid barrier: R-MAT 22 138 -> 116 us)
 constexpr int CC_SAMPLES = 1024;              // vertices sampled for the largest component
 
 struct CcArgs {
@@ -39,24 +39,14 @@ struct CcArgs {
     unsigned long long timeout_ns;
 };
 
-__device__ __forceinline__ int32_t find_root(int32_t *label, int32_t x) {
-    int32_t p = __ldcg(label + x);
-    while (p != x) {
-        x = p;
-        p = __ldcg(label + x);
-    }
-    return x;
-}
-
 // Joins the trees of u and v: the larger root goes under the smaller one.
 // Every failed attempt means some parent decreased, so the loop ends; the cap
 // only guards against a corrupted label array (then the status is set).
-__device__ __forceinline__ void hook(int32_t *label, int32_t u, int32_t v, TravCtl *ctl) {
-    // The first parents may come from L1 (a hub's label is read by most of its
-    // neighbours' hooks): a stale parent is still an ancestor, and the
-    // compare-and-swap below reads the larger root's parent fresh before it
-    // writes, so a stale start only costs a retry.
-    int32_t p1 = __ldca(label + u), p2 = __ldca(label + v);
+// p1, p2: parents of theirs, which may come from L1 (a hub's label is read by most
+// of its neighbours' hooks): a stale parent is still an ancestor, and the
+// compare-and-swap below reads the larger root's parent fresh before it
+// writes, so a stale start only costs a retry.
+__device__ __forceinline__ void hook(int32_t *label, int32_t p1, int32_t p2, TravCtl *ctl) {
     for (int tries = 0; p1 != p2; ++tries) {
         if (tries > (1 << 24)) {
             grx_set_status(ctl, GRX_ETIMEOUT);
@@ -87,33 +77,62 @@ __device__ __forceinline__ int32_t find_root_ca(const int32_t *label, int32_t x)
 }
 
 // Every vertex points at its root.
+template <int CC_FLIGHT>
 __device__ void compress(const CcArgs &a) {
-    for (int64_t v = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; v < a.nv;
-         v += (int64_t)gridDim.x * blockDim.x) {
-        const int32_t p = __ldcg(a.label + v);
-        if (p == v) continue;
-        const int32_t r = find_root_ca(a.label, p);
-        if (r != p) a.label[v] = r;
+    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+    for (int64_t v0 = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; v0 < a.nv; v0 += CC_FLIGHT * stride) {
+        int32_t p[CC_FLIGHT], g[CC_FLIGHT];
+#pragma unroll
+        for (int j = 0; j < CC_FLIGHT; ++j) {
+            const int64_t v = v0 + j * stride;
+            p[j] = v < a.nv ? __ldcg(a.label + v) : -1;
+        }
+#pragma unroll
+        for (int j = 0; j < CC_FLIGHT; ++j) {
+            g[j] = p[j];
+            if (p[j] >= 0 && p[j] != v0 + j * stride) g[j] = __ldca(a.label + p[j]);
+        }
+#pragma unroll
+        for (int j = 0; j < CC_FLIGHT; ++j)
+            if (g[j] != p[j]) a.label[v0 + j * stride] = find_root_ca(a.label, g[j]);
     }
 }
 
 // Hooks every non-isolated vertex to its k-th neighbour (k = 0 or 1), read
 // from the pair array of first neighbours: 8 bytes per vertex in vertex
 // order instead of a row start and a scattered column sector.
+template <int CC_FLIGHT>
 __device__ void hook_kth(const CcArgs &a, uint32_t k) {
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < a.n_active;
-         i += (int64_t)gridDim.x * blockDim.x) {
-        const int32_t v = __ldg(a.active + i);
-        const int2 f = __ldg(a.first2 + v);
-        const int32_t u = k == 0 ? f.x : f.y;
-        if (u >= 0) hook(a.label, v, u, a.ctl);
+    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+    for (int64_t i0 = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i0 < a.n_active; i0 += CC_FLIGHT * stride) {
+        int32_t v[CC_FLIGHT], u[CC_FLIGHT], p1[CC_FLIGHT], p2[CC_FLIGHT];
+#pragma unroll
+        for (int j = 0; j < CC_FLIGHT; ++j) {
+            const int64_t i = i0 + j * stride;
+            v[j] = i < a.n_active ? __ldg(a.active + i) : -1;
+        }
+#pragma unroll
+        for (int j = 0; j < CC_FLIGHT; ++j) {
+            const int2 f = v[j] >= 0 ? __ldg(a.first2 + v[j]) : make_int2(-1, -1);
+            u[j] = k == 0 ? f.x : f.y;
+        }
+#pragma unroll
+        for (int j = 0; j < CC_FLIGHT; ++j) {
+            p1[j] = p2[j] = 0;
+            if (u[j] >= 0) {
+                p1[j] = __ldca(a.label + v[j]);
+                p2[j] = __ldca(a.label + u[j]);
+            }
+        }
+#pragma unroll
+        for (int j = 0; j < CC_FLIGHT; ++j) hook(a.label, p1[j], p2[j], a.ctl);
     }
 }
 
 // Block 0: the most frequent root among CC_SAMPLES vertices spread over the
 // active list (ties go to the smaller root).
 __device__ void find_giant(const CcArgs &a) {
-    __shared__ int32_t roots[CC_SAMPLES];
+    __shared__ __align__(16) int32_t roots[CC_SAMPLES];
     __shared__ unsigned long long best;
     if (threadIdx.x == 0) best = 0ull;
     for (int s = threadIdx.x; s < CC_SAMPLES; s += blockDim.x) {
@@ -124,7 +143,11 @@ __device__ void find_giant(const CcArgs &a) {
     __syncthreads();
     for (int s = threadIdx.x; s < CC_SAMPLES; s += blockDim.x) {
         int c = 0;
-        for (int t = 0; t < CC_SAMPLES; ++t) c += roots[t] == roots[s];
+        const int32_t r = roots[s];
+        for (int t = 0; t < CC_SAMPLES; t += 4) {
+            const int4 x = *reinterpret_cast<const int4 *>(roots + t);
+            c += (x.x == r) + (x.y == r) + (x.z == r) + (x.w == r);
+        }
         atomicMax(&best, ((unsigned long long)c << 32) | (unsigned)(0x7fffffff - roots[s]));
     }
     __syncthreads();
@@ -132,22 +155,37 @@ __device__ void find_giant(const CcArgs &a) {
 }
 
 // Vertices outside the largest component hook their remaining edges.
+template <int CC_FLIGHT>
 __device__ void hook_rest(const CcArgs &a, int32_t giant, unsigned long long &linked) {
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < a.n_active;
-         i += (int64_t)gridDim.x * blockDim.x) {
-        const int32_t v = __ldg(a.active + i);
-        // Membership in the largest component through L1: a stale view only
-        // shows an earlier ancestor chain, and trees only merge, so a vertex
-        // seen under the giant root is in its component (its edges to other
-        // components are hooked from their side); a stale view that misses
-        // the root only costs this vertex's own hooks.
-        if (find_root_ca(a.label, v) == giant) continue;
-        const uint32_t b = __ldg(a.aoff + i), e = __ldg(a.aoff + i + 1);
-        for (uint32_t k = b + 2; k < e; ++k) hook(a.label, v, __ldg(a.col + k), a.ctl);
-        linked += e > b + 2 ? e - b - 2 : 0u;
+    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+    for (int64_t i0 = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i0 < a.n_active; i0 += CC_FLIGHT * stride) {
+        int32_t v[CC_FLIGHT], p[CC_FLIGHT];
+#pragma unroll
+        for (int j = 0; j < CC_FLIGHT; ++j) v[j] = i0 + j * stride < a.n_active ? __ldg(a.active + i0 + j * stride) : -1;
+#pragma unroll
+        for (int j = 0; j < CC_FLIGHT; ++j) p[j] = v[j] >= 0 ? __ldca(a.label + v[j]) : giant;
+#pragma unroll
+        for (int j = 0; j < CC_FLIGHT; ++j) {
+            // Membership in the largest component through L1: a stale view only
+            // shows an earlier ancestor chain, and trees only merge, so a vertex
+            // seen under the giant root is in its component (its edges to other
+            // components are hooked from their side); a stale view that misses
+            // the root only costs this vertex's own hooks.
+            if (p[j] == giant || find_root_ca(a.label, p[j]) == giant) continue;
+            const int64_t i = i0 + j * stride;
+            const uint32_t b = __ldg(a.aoff + i), e = __ldg(a.aoff + i + 1);
+            for (uint32_t k = b + 2; k < e; ++k)
+                hook(a.label, __ldca(a.label + v[j]), __ldca(a.label + __ldg(a.col + k)), a.ctl);
+            linked += e > b + 2 ? e - b - 2 : 0u;
+        }
     }
 }
 
+// FLIGHT: vertices a thread has in flight.  Two where vertices have many edges
+// (R-MAT 22 / 24: 114 -> 108, 327 -> 271 us; four 113, 270); one on grids and
+// paths, where labels read ahead are older and more hooks are tried again (grid
+// of 1000 x 1000: 172 us, with two 183).
+template <int FLIGHT>
 __global__ void __launch_bounds__(CC_BLOCK) k_cc_persistent(CcArgs a) {
     FlagBarrier bar{a.bar_flags, &a.ctl->bar_release, a.ctl, a.timeout_ns, 0u};
     for (int64_t v = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; v < a.nv;
@@ -155,24 +193,44 @@ __global__ void __launch_bounds__(CC_BLOCK) k_cc_persistent(CcArgs a) {
         a.label[v] = (int32_t)v;
     if (!flag_barrier(bar)) return;
     for (uint32_t k = 0; k < 2; ++k) {
-        hook_kth(a, k);
+        hook_kth<FLIGHT>(a, k);
         if (!flag_barrier(bar)) return;
-        compress(a);
+        compress<FLIGHT>(a);
         if (!flag_barrier(bar)) return;
     }
     if (blockIdx.x == 0) find_giant(a);
     if (!flag_barrier(bar)) return;
     const int32_t giant = ld_relaxed_u32((const unsigned int *)&a.ctl->cc_giant);
     unsigned long long linked = 0;
-    hook_rest(a, giant, linked);
+    hook_rest<FLIGHT>(a, giant, linked);
     if (!flag_barrier(bar)) return;
-    compress(a);
+    compress<FLIGHT>(a);
     linked = warp_sum(linked);
     if ((threadIdx.x & 31) == 0 && linked) atomicAdd(&a.stats->edges_examined[0], linked);
     if (blockIdx.x == 0 && threadIdx.x == 0) {
         a.ctl->levels_run = 1;
         a.stats->levels = 1;
     }
+}
+
+template <int FLIGHT>
+grx_status cc_launch(grx_graph *g, const CcArgs &a, const grx_opts *o, cudaStream_t s) {
+    static int per_sm = -1;
+    if (per_sm < 0) {
+        GRX_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_cc_persistent<FLIGHT>, CC_BLOCK, 0));
+        if (per_sm < 1) return grx_fail(GRX_ECUDA, "cc: persistent kernel does not fit on an SM");
+    }
+    int max_grid = per_sm * g->ctx->num_sms;
+    if (max_grid > GRX_MAX_GRID) max_grid = GRX_MAX_GRID;
+    const int blocks = grx_grid(o, CC_BLOCK, max_grid);
+    GRX_CUDA(cudaMemsetAsync(g->bar_flags, 0, sizeof(unsigned int) * (size_t)blocks, s));
+    GRX_CUDA(cudaMemsetAsync(&g->ctl->bar_release, 0, sizeof(unsigned int), s));
+    GRX_CUDA(cudaMemsetAsync(&g->stats->levels, 0, sizeof(int32_t), s));
+    GRX_CUDA(cudaMemsetAsync(&g->stats->edges_examined[0], 0, sizeof(unsigned long long), s));
+    void *args[] = {(void *)&a};
+    GRX_CUDA(cudaLaunchCooperativeKernel((const void *)k_cc_persistent<FLIGHT>, dim3(blocks), dim3(CC_BLOCK),
+                                         args, 0, s));
+    return GRX_OK;
 }
 
 }  // namespace
@@ -190,20 +248,5 @@ grx_status grx_cc_launch(grx_graph *g, int32_t *label, const grx_opts *o, cudaSt
     a.stats = g->stats;
     a.bar_flags = g->bar_flags;
     a.timeout_ns = grx_timeout_ns(o);
-    static int per_sm = -1;
-    if (per_sm < 0) {
-        GRX_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_cc_persistent, CC_BLOCK, 0));
-        if (per_sm < 1) return grx_fail(GRX_ECUDA, "cc: persistent kernel does not fit on an SM");
-    }
-    int max_grid = per_sm * g->ctx->num_sms;
-    if (max_grid > GRX_MAX_GRID) max_grid = GRX_MAX_GRID;
-    int blocks = o->grid_blocks > 0 && o->grid_blocks < max_grid ? o->grid_blocks : max_grid;
-    GRX_CUDA(cudaMemsetAsync(g->bar_flags, 0, sizeof(unsigned int) * (size_t)blocks, s));
-    GRX_CUDA(cudaMemsetAsync(&g->ctl->bar_release, 0, sizeof(unsigned int), s));
-    GRX_CUDA(cudaMemsetAsync(&g->stats->levels, 0, sizeof(int32_t), s));
-    GRX_CUDA(cudaMemsetAsync(&g->stats->edges_examined[0], 0, sizeof(unsigned long long), s));
-    void *args[] = {(void *)&a};
-    GRX_CUDA(cudaLaunchCooperativeKernel((const void *)k_cc_persistent, dim3(blocks), dim3(CC_BLOCK),
-                                         args, 0, s));
-    return GRX_OK;
+    return g->ne >= 8ll * g->nv ? cc_launch<2>(g, a, o, s) : cc_launch<1>(g, a, o, s);
 }
