@@ -49,10 +49,9 @@
 
 namespace {
 
-#ifndef GRX_BC_MIN_BLOCKS
-#define GRX_BC_MIN_BLOCKS 3                 // resident blocks per SM (register cap)
-#endif
-constexpr int BC_BLOCK = 256;
+// Two blocks of 384 threads an SM, as in bfs.cu (R-MAT 22 / 18: 1 / 2 %).
+constexpr int BC_BLOCK = 384;
+constexpr int BC_MIN_BLOCKS = 2;            // resident blocks per SM (register cap)
 constexpr int BC_WARPS = BC_BLOCK / 32;
 constexpr int BC_ITEMS = 8;
 constexpr int BC_WTILE = 32 * BC_ITEMS;
@@ -707,7 +706,7 @@ __device__ BcState bc_next(const BcArgs<OffT> &a, const BcState &st) {
 }
 
 template <typename OffT>
-__global__ void __launch_bounds__(BC_BLOCK, GRX_BC_MIN_BLOCKS) k_bc_persistent(BcArgs<OffT> a) {
+__global__ void __launch_bounds__(BC_BLOCK, BC_MIN_BLOCKS) k_bc_persistent(BcArgs<OffT> a) {
     __shared__ BcState s_st;
     __shared__ BcWarpSmem<OffT> wsm[BC_WARPS];
     BcWarpSmem<OffT> &w = wsm[threadIdx.x >> 5];
