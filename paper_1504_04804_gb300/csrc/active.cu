@@ -114,6 +114,7 @@ grx_status grx_build_active(grx_graph *g, cudaStream_t s) {
     k_block_popcounts<<<(unsigned)nblocks, ACT_BLOCK, 0, s>>>(g->nz_bits, g->words, bsum);
     std::vector<uint32_t> h((size_t)nblocks);
     cudaError_t e = cudaMemcpyAsync(h.data(), bsum, (size_t)nblocks * 4, cudaMemcpyDeviceToHost, s);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(&g->max_deg, g->nz_bits + g->words, 4, cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     if (e != cudaSuccess) {
         grx_ctx_free(g->ctx, bsum, (size_t)nblocks * 4, s);

@@ -147,19 +147,27 @@ __global__ void k_offsets_32_to_64(const int32_t *in, int64_t *out, int64_t n) {
         out[i] = (int64_t)in[i];
 }
 
-// Bitmap of vertices with at least one edge.  One thread per 32-vertex word.
+// Bitmap of vertices with at least one edge, and the largest degree in the word
+// after it.  One thread per 32-vertex word.
 template <typename OffT>
 __global__ void k_nonzero_bits(const OffT *ro, int32_t nv, uint32_t *bits, int64_t words) {
+    uint32_t most = 0;
     for (int64_t w = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; w < words;
          w += (int64_t)gridDim.x * blockDim.x) {
         uint32_t b = 0;
         int64_t v0 = w * 32;
         for (int k = 0; k < 32; ++k) {
             int64_t v = v0 + k;
-            if (v < nv && ro[v + 1] > ro[v]) b |= 1u << k;
+            if (v < nv && ro[v + 1] > ro[v]) {
+                b |= 1u << k;
+                most = max(most, (uint32_t)(ro[v + 1] - ro[v]));
+            }
         }
         bits[w] = b;
     }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) most = max(most, __shfl_xor_sync(GRX_FULL_MASK, most, o));
+    if ((threadIdx.x & 31) == 0 && most) atomicMax(bits + words, most);
 }
 
 // Validation of a CSR on the device: offsets monotone with ro[0] == 0 and
@@ -242,7 +250,7 @@ extern "C" grx_status graph_load_csr(grx_ctx *ctx, int64_t nv, int64_t ne, const
 
     g->ro = grx_alloc(g, ro_bytes, s);
     g->col = (int32_t *)grx_alloc(g, (size_t)ne * 4, s);
-    g->nz_bits = (uint32_t *)grx_alloc(g, (size_t)g->words * 4, s);
+    g->nz_bits = (uint32_t *)grx_alloc(g, (size_t)g->words * 4 + 16, s);
     if (weights) g->w = (uint32_t *)grx_alloc(g, (size_t)ne * 4, s);
     if (!g->ro || !g->col || !g->nz_bits || (weights && !g->w))
         LOAD_FAIL(GRX_ENOMEM, "graph_load_csr: device allocation of %zu bytes failed",
@@ -272,7 +280,7 @@ extern "C" grx_status graph_load_csr(grx_ctx *ctx, int64_t nv, int64_t ne, const
         if (weights && ne > 0 &&
             cudaMemcpyAsync(g->w, weights, (size_t)ne * 4, kind, s) != cudaSuccess)
             LOAD_FAIL(GRX_ECUDA, "graph_load_csr: copy of weights failed");
-        cudaMemsetAsync(g->nz_bits, 0, (size_t)g->words * 4, s);
+        cudaMemsetAsync(g->nz_bits, 0, (size_t)g->words * 4 + 16, s);
         int blocks = (int)((g->words + 255) / 256);
         if (blocks > 4096) blocks = 4096;
         if (g->off64) k_nonzero_bits<<<blocks, 256, 0, s>>>((const int64_t *)g->ro, g->nv, g->nz_bits, g->words);

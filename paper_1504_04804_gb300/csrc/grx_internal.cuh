@@ -78,6 +78,7 @@ struct grx_graph {
     int32_t *col;                    // [ne]
     uint32_t *w;                     // [ne] or NULL
     uint32_t *nz_bits;               // non-isolated vertex bitmap [words]
+    uint32_t max_deg;                // largest degree
     int64_t words;                   // (nv + 31) / 32 rounded up to 32
     // non-isolated vertices in increasing id order and their row starts:
     // active[i] = v, aoff[i] = ro[v], aoff[n_active] = ne.  With isolated

@@ -768,6 +768,8 @@ grx_status launch_persistent(grx_graph *g, SsspArgs<OffT> &a, int32_t src, uint3
             a.pieces = a.lines + 2 * SS_LIST_BLOCKS;
             a.verts = (int32_t *)(a.pieces + 2 * (size_t)g->ss_list_blocks * ss_list_pieces(t));
             a.list_T = t;
+            // lists are the better form of a large round too, up to their limit,
+            // unless the caller set the line for the changed bitmap
             if (o->push_bitmap == 0.f && a.bmp_min_T <= t * (uint32_t)blocks) a.bmp_min_T = t * (uint32_t)blocks + 1;
         }
     }
@@ -815,10 +817,10 @@ grx_status launch_typed(grx_graph *g, int32_t src, uint32_t *dist, const grx_opt
         const double t = pb * (double)g->nv;
         a.bmp_min_T = pb < 0 ? 0xffffffffu : (t < 1.0 ? 1u : (t > 4294967295.0 ? 0xffffffffu : (uint32_t)t));
     }
-    // List rounds on graphs of few edges a vertex (see narrow levels of bfs.cu);
-    // only where they are the better form of a large round too: lists up to the
-    // limit, the changed bitmap past it, unless the caller set the line.
-    return g->ne < 8ll * g->nv ? launch_persistent<OffT, STATS, true>(g, a, src, dist, o, s)
+    // List rounds on graphs of few edges a vertex and no hubs: thousands of rounds
+    // of small rows (with hubs, R-MAT of edge factor 4, a handful of rounds, most of
+    // the work in two or three of them).
+    return g->ne < 8ll * g->nv && g->max_deg <= 64 ? launch_persistent<OffT, STATS, true>(g, a, src, dist, o, s)
                                : launch_persistent<OffT, STATS, false>(g, a, src, dist, o, s);
 }
 
