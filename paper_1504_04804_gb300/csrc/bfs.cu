@@ -1405,11 +1405,12 @@ __global__ void k_bfs_gtick(const BfsArgs<OffT> *ap, cudaGraphConditionalHandle 
 }
 
 // Opt every kernel of an instantiation in to its dynamic shared memory size
-// (once per process).
+// (once per device).
 template <typename OffT, bool PARENT, bool STATS>
-grx_status prepare_kernels() {
-    static bool done = false;
-    if (done) return GRX_OK;
+grx_status prepare_kernels(int device) {
+    static unsigned long long done = 0;
+    const unsigned long long bit = 1ull << (device & 63);
+    if ((done & bit) && device < 64) return GRX_OK;
     const int bytes = (int)bfs_smem_bytes<OffT>();
     GRX_CUDA(cudaFuncSetAttribute((const void *)k_bfs_persistent<OffT, PARENT, STATS, false>,
                                   cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
@@ -1421,7 +1422,7 @@ grx_status prepare_kernels() {
                                   cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
     GRX_CUDA(cudaFuncSetAttribute((const void *)k_bfs_glevel<OffT, PARENT>,
                                   cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
-    done = true;
+    done |= bit;
     return GRX_OK;
 }
 
@@ -1552,7 +1553,7 @@ template <typename OffT, bool PARENT, bool STATS>
 grx_status launch_typed(grx_graph *g, int32_t src, int32_t *depth, int32_t *parent,
                         const grx_opts *o, cudaStream_t s) {
     BfsArgs<OffT> a = make_args<OffT>(g, src, depth, parent, o);
-    grx_status pst = prepare_kernels<OffT, PARENT, STATS>();
+    grx_status pst = prepare_kernels<OffT, PARENT, STATS>(g->ctx->device);
     if (pst != GRX_OK) return pst;
     const size_t smem = bfs_smem_bytes<OffT>();
     if (o->loop == GRX_LOOP_GRAPH) {

@@ -739,10 +739,15 @@ grx_status launch_persistent(grx_graph *g, SsspArgs<OffT> &a, int32_t src, uint3
                                       o->collect_stats);
     GRX_CUDA(cudaGetLastError());
     constexpr int smem = (int)sizeof(SsSmem<OffT>);
-    static int per_sm = -1;
-    if (per_sm < 0) {
+    static unsigned long long ready = 0;         // devices whose kernel may use this much shared memory
+    const unsigned long long bit = 1ull << (g->ctx->device & 63);
+    if (!(ready & bit) || g->ctx->device > 63) {
         GRX_CUDA(cudaFuncSetAttribute((const void *)k_sssp_persistent<OffT, STATS, LIST>,
                                       cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+        ready |= bit;
+    }
+    static int per_sm = -1;
+    if (per_sm < 0) {
         GRX_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_sssp_persistent<OffT, STATS, LIST>,
                                                                SS_BLOCK, smem));
         if (per_sm < 1) return grx_fail(GRX_ECUDA, "sssp: persistent kernel does not fit on an SM");
