@@ -54,6 +54,7 @@ constexpr int BC_BLOCK = 384;
 constexpr int BC_MIN_BLOCKS = 2;            // resident blocks per SM (register cap)
 constexpr int BC_WARPS = BC_BLOCK / 32;
 constexpr int BC_ITEMS = 8;
+constexpr int BC_BATCH = 4;                 // tiles a warp takes at a time
 constexpr int BC_WTILE = 32 * BC_ITEMS;
 constexpr int BC_RPL = 4;                  // finalize: vertices per lane per round
 // A forward pull reads every edge of every unreached vertex (no early exit)
@@ -185,19 +186,30 @@ __device__ __forceinline__ void finish_vertex(const BcArgs<OffT> &a, int32_t v, 
     a.acc[v] = 1.0 / sg + s;
 }
 
-// Warp-tile range [tb0, tb1) of this warp over a level with T edges; false if empty.
-__device__ __forceinline__ bool warp_tiles(uint64_t T, uint64_t &tb0, uint64_t &tb1) {
+// Runs body(first tile, end) for the calling warp's batches of the level's
+// tiles: the first by the warp's number, the others from the phase's counter
+// (what a tile costs varies along the queue; four sources on R-MAT 22: one equal
+// share a warp 3.61 ms, batches of 8 / 4 / 2 tiles 3.51 / 3.45 / 3.55).
+template <typename Body>
+__device__ __forceinline__ void warp_batches(TravCtl *ctl, int phase, uint64_t T, Body &&body) {
     const uint64_t ntiles = (T + BC_WTILE - 1) / BC_WTILE;
     const uint64_t nwarps = (uint64_t)gridDim.x * BC_WARPS;
-    const uint64_t gw = (uint64_t)blockIdx.x * BC_WARPS + (threadIdx.x >> 5);
-    const uint64_t per = (ntiles + nwarps - 1) / nwarps;
-    tb0 = gw * per;
-    tb1 = min(ntiles, tb0 + per);
-    return tb0 < tb1;
+    const uint64_t batch = min((uint64_t)BC_BATCH, (ntiles + nwarps - 1) / nwarps);
+    if (batch == 0) return;
+    const uint64_t nbatch = (ntiles + batch - 1) / batch;
+    unsigned int *wq = &ctl->wq[phase & 3];
+    for (uint64_t bt = (uint64_t)blockIdx.x * BC_WARPS + (threadIdx.x >> 5); bt < nbatch;) {
+        unsigned int nn = 0;
+        if ((threadIdx.x & 31) == 0) nn = atomicAdd(wq, 1u);
+        body(bt * batch, min(ntiles, (bt + 1) * batch));
+        bt = nwarps + __shfl_sync(GRX_FULL_MASK, nn, 0);
+    }
 }
 
 // Forward step of level d: shortest-path edges add sigma; unreached vertices
-// are claimed for level d + 1 (claim mode) or marked in F (bitmap mode).
+// are claimed for level d + 1 (claim mode) or marked in F (bitmap mode).  Tile
+// positions are interleaved across the lanes, here and in the backward push, so that
+// a column load is one run (four sources on R-MAT 22: 3.87 -> 3.61 ms).
 template <typename OffT, bool BMP>
 __device__ void forward_level(const BcArgs<OffT> &a, const BcState &st, BcWarpSmem<OffT> &w) {
     const int d = st.d;
@@ -211,71 +223,70 @@ __device__ void forward_level(const BcArgs<OffT> &a, const BcState &st, BcWarpSm
     OffT *Qr_out = a.R + st.start + st.q;
     unsigned long long *ctr = &a.ctl->qpack[(d + 1) & 3];
     const uint64_t T = st.T;
-    uint64_t tb0, tb1;
-    if (!warp_tiles(T, tb0, tb1)) return;
-    int64_t i0 = warp_upper_index_cg(Qe, st.q, (uint32_t)(tb0 * BC_WTILE));
-    for (uint64_t tile = tb0; tile < tb1; ++tile) {
-        const uint64_t e0 = tile * BC_WTILE;
-        const uint32_t e1 = (uint32_t)min(T, e0 + BC_WTILE);
-        const int n = stage_elements<OffT, STAGE_SIGMA>(a, Qv, Qe, Qr, st.q, i0, e1, w);
-        const uint32_t next_start = w.qe[n];
-        int row[BC_ITEMS];
-        warp_tile_rows8(w.rid, w.qe, (uint32_t)e0, n, row);
-        const uint32_t t0 = (uint32_t)e0 + lane * BC_ITEMS;
-        int32_t v[BC_ITEMS];
-        double su[BC_ITEMS];
-#pragma unroll
-        for (int k = 0; k < BC_ITEMS; ++k) {
-            const uint32_t e = t0 + k;
-            const int j = row[k];
-            const bool ok = e < e1;
-            const OffT idx = ok ? w.rs[j] + (OffT)(e - w.qe[j]) : (OffT)0;
-            v[k] = ok ? __ldg(a.col + idx) : -1;
-            su[k] = ok ? w.val[j] : 0.0;
-        }
-        __syncwarp();
-        uint32_t c[BC_ITEMS];
-#pragma unroll
-        for (int k = 0; k < BC_ITEMS; ++k) c[k] = v[k] >= 0 ? level_code(a.code, v[k]) : 0xffu;
-        if (BMP) {
+    warp_batches(a.ctl, st.phase, T, [&](uint64_t tb0, uint64_t tb1) {
+        int64_t i0 = warp_upper_index_cg(Qe, st.q, (uint32_t)(tb0 * BC_WTILE));
+        for (uint64_t tile = tb0; tile < tb1; ++tile) {
+            const uint64_t e0 = tile * BC_WTILE;
+            const uint32_t e1 = (uint32_t)min(T, e0 + BC_WTILE);
+            const int n = stage_elements<OffT, STAGE_SIGMA>(a, Qv, Qe, Qr, st.q, i0, e1, w);
+            const uint32_t next_start = w.qe[n];
+            int row[BC_ITEMS];
+            warp_tile_rows8_strided(w.rid, w.qe, (uint32_t)e0, n, row);   // item k at position k*32 + lane
+            int32_t v[BC_ITEMS];
+            double su[BC_ITEMS];
 #pragma unroll
             for (int k = 0; k < BC_ITEMS; ++k) {
-                if (c[k] == 3u) atomicAdd(a.sigma + v[k], su[k]);   // codes fixed in this phase; reduction
+                const uint32_t e = (uint32_t)e0 + (uint32_t)k * 32 + lane;
+                const int j = row[k];
+                const bool ok = e < e1;
+                const OffT idx = ok ? w.rs[j] + (OffT)(e - w.qe[j]) : (OffT)0;
+                v[k] = ok ? __ldg(a.col + idx) : -1;
+                su[k] = ok ? w.val[j] : 0.0;
             }
-        } else {
-            uint32_t claimed = 0, dag = 0;
+            __syncwarp();
+            uint32_t c[BC_ITEMS];
 #pragma unroll
-            for (int k = 0; k < BC_ITEMS; ++k) {
-                if (c[k] == 3u) {
-                    const uint32_t sh = (uint32_t)(v[k] & 15) * 2u;
-                    const uint32_t old = atomicAnd(a.code + (v[k] >> 4), ~((3u ^ cn) << sh));
-                    if (((old >> sh) & 3u) == 3u) claimed |= 1u << k;
-                    dag |= 1u << k;
-                } else if (c[k] == cn) {
-                    dag |= 1u << k;
+            for (int k = 0; k < BC_ITEMS; ++k) c[k] = v[k] >= 0 ? level_code(a.code, v[k]) : 0xffu;
+            if (BMP) {
+#pragma unroll
+                for (int k = 0; k < BC_ITEMS; ++k) {
+                    if (c[k] == 3u) atomicAdd(a.sigma + v[k], su[k]);   // codes fixed in this phase; reduction
                 }
-            }
+            } else {
+                uint32_t claimed = 0, dag = 0;
 #pragma unroll
-            for (int k = 0; k < BC_ITEMS; ++k)
-                if (dag >> k & 1u) atomicAdd(a.sigma + v[k], su[k]);
-            uint32_t deg[BC_ITEMS];
-            OffT rb[BC_ITEMS];
-            uint32_t app = 0;
-#pragma unroll
-            for (int k = 0; k < BC_ITEMS; ++k) {
-                rb[k] = 0;
-                deg[k] = 0;
-                if (claimed >> k & 1u) {
-                    rb[k] = __ldg(a.ro + v[k]);
-                    deg[k] = (uint32_t)(__ldg(a.ro + v[k] + 1) - rb[k]);
-                    if (deg[k]) app |= 1u << k;
+                for (int k = 0; k < BC_ITEMS; ++k) {
+                    if (c[k] == 3u) {
+                        const uint32_t sh = (uint32_t)(v[k] & 15) * 2u;
+                        const uint32_t old = atomicAnd(a.code + (v[k] >> 4), ~((3u ^ cn) << sh));
+                        if (((old >> sh) & 3u) == 3u) claimed |= 1u << k;
+                        dag |= 1u << k;
+                    } else if (c[k] == cn) {
+                        dag |= 1u << k;
+                    }
                 }
+#pragma unroll
+                for (int k = 0; k < BC_ITEMS; ++k)
+                    if (dag >> k & 1u) atomicAdd(a.sigma + v[k], su[k]);
+                uint32_t deg[BC_ITEMS];
+                OffT rb[BC_ITEMS];
+                uint32_t app = 0;
+#pragma unroll
+                for (int k = 0; k < BC_ITEMS; ++k) {
+                    rb[k] = 0;
+                    deg[k] = 0;
+                    if (claimed >> k & 1u) {
+                        rb[k] = __ldg(a.ro + v[k]);
+                        deg[k] = (uint32_t)(__ldg(a.ro + v[k] + 1) - rb[k]);
+                        if (deg[k]) app |= 1u << k;
+                    }
+                }
+                warp_append_items<BC_ITEMS, OffT>(v, deg, rb, app, Qv_out, Qe_out, Qr_out, ctr);
             }
-            warp_append_items<BC_ITEMS, OffT>(v, deg, rb, app, Qv_out, Qe_out, Qr_out, ctr);
+            i0 = (next_start == e1) ? i0 + n : i0 + n - 1;
+            __syncwarp();
         }
-        i0 = (next_start == e1) ? i0 + n : i0 + n - 1;
-        __syncwarp();
-    }
+    });
 }
 
 // Second phase of a bitmap level: per 32-word chunk of vertices, the
@@ -353,106 +364,106 @@ __device__ void backward_level(const BcArgs<OffT> &a, const BcState &st, BcWarpS
     const uint32_t *Qe = a.E + st.start;
     const OffT *Qr = a.R + st.start;
     const uint64_t T = st.T;
-    uint64_t tb0, tb1;
-    if (!warp_tiles(T, tb0, tb1)) return;
-    int64_t i0 = warp_upper_index_cg(Qe, st.q, (uint32_t)(tb0 * BC_WTILE));
-    for (uint64_t tile = tb0; tile < tb1; ++tile) {
-        const uint64_t e0 = tile * BC_WTILE;
-        const uint32_t e1 = (uint32_t)min(T, e0 + BC_WTILE);
-        const int n = stage_elements<OffT, STAGE_NONE>(a, Qv, Qe, Qr, st.q, i0, e1, w);
-        const uint32_t next_start = w.qe[n];
-        int row[BC_ITEMS];
-        warp_tile_rows8(w.rid, w.qe, (uint32_t)e0, n, row);
-        const uint32_t t0 = (uint32_t)e0 + lane * BC_ITEMS;
-        int32_t u[BC_ITEMS];
-#pragma unroll
-        for (int k = 0; k < BC_ITEMS; ++k) {
-            const uint32_t e = t0 + k;
-            const int j = row[k];
-            const OffT idx = e < e1 ? w.rs[j] + (OffT)(e - w.qe[j]) : (OffT)0;
-            u[k] = e < e1 ? __ldg(a.col + idx) : -1;
-        }
-        uint32_t cu[BC_ITEMS];
-#pragma unroll
-        for (int k = 0; k < BC_ITEMS; ++k) cu[k] = u[k] >= 0 ? level_code(a.code, u[k]) : 0xffu;
-        double c[BC_ITEMS];
-#pragma unroll
-        for (int k = 0; k < BC_ITEMS; ++k) c[k] = cu[k] == ck ? __ldcg(a.acc + u[k]) : 0.0;
-        // Runs of equal rows in the lane.  Runs between the lane's first and
-        // last one are whole rows of the tile; the first (hr, hs) and last
-        // (tr, ts) may continue in the neighbouring lanes.
-        int hr = -1, tr = -1;
-        double hs = 0.0, ts = 0.0;
-        {
-            int cur = -1;
-            double part = 0.0;
+    warp_batches(a.ctl, st.phase, T, [&](uint64_t tb0, uint64_t tb1) {
+        int64_t i0 = warp_upper_index_cg(Qe, st.q, (uint32_t)(tb0 * BC_WTILE));
+        for (uint64_t tile = tb0; tile < tb1; ++tile) {
+            const uint64_t e0 = tile * BC_WTILE;
+            const uint32_t e1 = (uint32_t)min(T, e0 + BC_WTILE);
+            const int n = stage_elements<OffT, STAGE_NONE>(a, Qv, Qe, Qr, st.q, i0, e1, w);
+            const uint32_t next_start = w.qe[n];
+            int row[BC_ITEMS];
+            warp_tile_rows8(w.rid, w.qe, (uint32_t)e0, n, row);
+            const uint32_t t0 = (uint32_t)e0 + lane * BC_ITEMS;
+            int32_t u[BC_ITEMS];
 #pragma unroll
             for (int k = 0; k < BC_ITEMS; ++k) {
-                if (t0 + k < e1) {
-                    if (row[k] != cur) {
-                        if (cur >= 0) {
-                            if (hr < 0) {
-                                hr = cur;
-                                hs = part;
-                            } else {
-                                w.val[cur] = part;
-                            }
-                        }
-                        cur = row[k];
-                        part = 0.0;
-                    }
-                    part += c[k];
-                }
+                const uint32_t e = t0 + k;
+                const int j = row[k];
+                const OffT idx = e < e1 ? w.rs[j] + (OffT)(e - w.qe[j]) : (OffT)0;
+                u[k] = e < e1 ? __ldg(a.col + idx) : -1;
             }
-            if (cur >= 0) {
-                if (hr < 0) {
-                    hr = cur;
-                    hs = part;
-                }
-                tr = cur;
-                ts = part;
-            }
-        }
-        // Segmented inclusive scan of the lanes' last runs: a lane continues
-        // the previous lane's segment when its items all belong to that row.
-        const int prev_tr = __shfl_up_sync(GRX_FULL_MASK, tr, 1);
-        const bool single = hr == tr;
-        int f = (lane > 0 && single && tr >= 0 && prev_tr == tr) ? 0 : 1;
-        double sv = ts;
+            uint32_t cu[BC_ITEMS];
 #pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const double pv = __shfl_up_sync(GRX_FULL_MASK, sv, o);
-            const int pf = __shfl_up_sync(GRX_FULL_MASK, f, o);
-            if (lane >= (unsigned)o) {
-                if (!f) sv += pv;
-                f |= pf;
+            for (int k = 0; k < BC_ITEMS; ++k) cu[k] = u[k] >= 0 ? level_code(a.code, u[k]) : 0xffu;
+            double c[BC_ITEMS];
+#pragma unroll
+            for (int k = 0; k < BC_ITEMS; ++k) c[k] = cu[k] == ck ? __ldcg(a.acc + u[k]) : 0.0;
+            // Runs of equal rows in the lane.  Runs between the lane's first and
+            // last one are whole rows of the tile; the first (hr, hs) and last
+            // (tr, ts) may continue in the neighbouring lanes.
+            int hr = -1, tr = -1;
+            double hs = 0.0, ts = 0.0;
+            {
+                int cur = -1;
+                double part = 0.0;
+#pragma unroll
+                for (int k = 0; k < BC_ITEMS; ++k) {
+                    if (t0 + k < e1) {
+                        if (row[k] != cur) {
+                            if (cur >= 0) {
+                                if (hr < 0) {
+                                    hr = cur;
+                                    hs = part;
+                                } else {
+                                    w.val[cur] = part;
+                                }
+                            }
+                            cur = row[k];
+                            part = 0.0;
+                        }
+                        part += c[k];
+                    }
+                }
+                if (cur >= 0) {
+                    if (hr < 0) {
+                        hr = cur;
+                        hs = part;
+                    }
+                    tr = cur;
+                    ts = part;
+                }
             }
-        }
-        const double prev_sv = __shfl_up_sync(GRX_FULL_MASK, sv, 1);
-        const int next_hr = __shfl_down_sync(GRX_FULL_MASK, hr, 1);
-        if (!single && hr >= 0) w.val[hr] = (lane > 0 && prev_tr == hr ? prev_sv : 0.0) + hs;
-        if (tr >= 0 && (lane == 31 || next_hr != tr)) w.val[tr] = sv;
-        __syncwarp();
-        // rows inside the tile finish here; rows crossing it add to acc, and
-        // the tile with the row's last edge lists the vertex for the fix-up
-        for (int j = (int)lane; j < n; j += 32) {
-            const uint32_t rb = w.qe[j];
-            const uint32_t re = i0 + j + 1 < (int64_t)st.q ? w.qe[j + 1] : (uint32_t)T;   // row end
-            const uint32_t lo = rb > (uint32_t)e0 ? rb : (uint32_t)e0;
-            const uint32_t hi = re < e1 ? re : e1;
-            if (hi <= lo) continue;                          // empty row
-            const int32_t v = __ldcg(Qv + i0 + j);
-            const double s = w.val[j];
-            if (rb >= (uint32_t)e0 && re <= e1) {
-                finish_vertex(a, v, s);
-            } else {
-                if (s != 0.0) atomicAdd(a.acc + v, s);       // result unused: reduction
-                if (re <= e1) a.fix[atomicAdd(&a.ctl->bcfix[st.d % 3], 1u)] = v;
+            // Segmented inclusive scan of the lanes' last runs: a lane continues
+            // the previous lane's segment when its items all belong to that row.
+            const int prev_tr = __shfl_up_sync(GRX_FULL_MASK, tr, 1);
+            const bool single = hr == tr;
+            int f = (lane > 0 && single && tr >= 0 && prev_tr == tr) ? 0 : 1;
+            double sv = ts;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const double pv = __shfl_up_sync(GRX_FULL_MASK, sv, o);
+                const int pf = __shfl_up_sync(GRX_FULL_MASK, f, o);
+                if (lane >= (unsigned)o) {
+                    if (!f) sv += pv;
+                    f |= pf;
+                }
             }
+            const double prev_sv = __shfl_up_sync(GRX_FULL_MASK, sv, 1);
+            const int next_hr = __shfl_down_sync(GRX_FULL_MASK, hr, 1);
+            if (!single && hr >= 0) w.val[hr] = (lane > 0 && prev_tr == hr ? prev_sv : 0.0) + hs;
+            if (tr >= 0 && (lane == 31 || next_hr != tr)) w.val[tr] = sv;
+            __syncwarp();
+            // rows inside the tile finish here; rows crossing it add to acc, and
+            // the tile with the row's last edge lists the vertex for the fix-up
+            for (int j = (int)lane; j < n; j += 32) {
+                const uint32_t rb = w.qe[j];
+                const uint32_t re = i0 + j + 1 < (int64_t)st.q ? w.qe[j + 1] : (uint32_t)T;   // row end
+                const uint32_t lo = rb > (uint32_t)e0 ? rb : (uint32_t)e0;
+                const uint32_t hi = re < e1 ? re : e1;
+                if (hi <= lo) continue;                          // empty row
+                const int32_t v = __ldcg(Qv + i0 + j);
+                const double s = w.val[j];
+                if (rb >= (uint32_t)e0 && re <= e1) {
+                    finish_vertex(a, v, s);
+                } else {
+                    if (s != 0.0) atomicAdd(a.acc + v, s);       // result unused: reduction
+                    if (re <= e1) a.fix[atomicAdd(&a.ctl->bcfix[st.d % 3], 1u)] = v;
+                }
+            }
+            i0 = (next_start == e1) ? i0 + n : i0 + n - 1;
+            __syncwarp();
         }
-        i0 = (next_start == e1) ? i0 + n : i0 + n - 1;
-        __syncwarp();
-    }
+    });
 }
 
 
@@ -573,38 +584,37 @@ __device__ void backward_push(const BcArgs<OffT> &a, const BcState &st, BcWarpSm
     const uint32_t *Qe = a.E + st.ps;
     const OffT *Qr = a.R + st.ps;
     const uint64_t T = st.pT;
-    uint64_t tb0, tb1;
-    if (!warp_tiles(T, tb0, tb1)) return;
-    int64_t i0 = warp_upper_index_cg(Qe, st.pq, (uint32_t)(tb0 * BC_WTILE));
-    for (uint64_t tile = tb0; tile < tb1; ++tile) {
-        const uint64_t e0 = tile * BC_WTILE;
-        const uint32_t e1 = (uint32_t)min(T, e0 + BC_WTILE);
-        const int n = stage_elements<OffT, STAGE_ACC>(a, Qv, Qe, Qr, st.pq, i0, e1, w);
-        const uint32_t next_start = w.qe[n];
-        int row[BC_ITEMS];
-        warp_tile_rows8(w.rid, w.qe, (uint32_t)e0, n, row);
-        const uint32_t t0 = (uint32_t)e0 + lane * BC_ITEMS;
-        int32_t v[BC_ITEMS];
-        double x[BC_ITEMS];
+    warp_batches(a.ctl, st.phase, T, [&](uint64_t tb0, uint64_t tb1) {
+        int64_t i0 = warp_upper_index_cg(Qe, st.pq, (uint32_t)(tb0 * BC_WTILE));
+        for (uint64_t tile = tb0; tile < tb1; ++tile) {
+            const uint64_t e0 = tile * BC_WTILE;
+            const uint32_t e1 = (uint32_t)min(T, e0 + BC_WTILE);
+            const int n = stage_elements<OffT, STAGE_ACC>(a, Qv, Qe, Qr, st.pq, i0, e1, w);
+            const uint32_t next_start = w.qe[n];
+            int row[BC_ITEMS];
+            warp_tile_rows8_strided(w.rid, w.qe, (uint32_t)e0, n, row);   // item k at position k*32 + lane
+            int32_t v[BC_ITEMS];
+            double x[BC_ITEMS];
 #pragma unroll
-        for (int k = 0; k < BC_ITEMS; ++k) {
-            const uint32_t e = t0 + k;
-            const int j = row[k];
-            const bool ok = e < e1;
-            const OffT idx = ok ? w.rs[j] + (OffT)(e - w.qe[j]) : (OffT)0;
-            v[k] = ok ? __ldg(a.col + idx) : -1;
-            x[k] = ok ? w.val[j] : 0.0;
+            for (int k = 0; k < BC_ITEMS; ++k) {
+                const uint32_t e = (uint32_t)e0 + (uint32_t)k * 32 + lane;
+                const int j = row[k];
+                const bool ok = e < e1;
+                const OffT idx = ok ? w.rs[j] + (OffT)(e - w.qe[j]) : (OffT)0;
+                v[k] = ok ? __ldg(a.col + idx) : -1;
+                x[k] = ok ? w.val[j] : 0.0;
+            }
+            __syncwarp();
+            uint32_t cv[BC_ITEMS];
+#pragma unroll
+            for (int k = 0; k < BC_ITEMS; ++k) cv[k] = v[k] >= 0 ? level_code(a.code, v[k]) : 0xffu;
+#pragma unroll
+            for (int k = 0; k < BC_ITEMS; ++k)
+                if (cv[k] == cd) atomicAdd(a.acc + v[k], x[k]);              // result unused: reduction
+            i0 = (next_start == e1) ? i0 + n : i0 + n - 1;
+            __syncwarp();
         }
-        __syncwarp();
-        uint32_t cv[BC_ITEMS];
-#pragma unroll
-        for (int k = 0; k < BC_ITEMS; ++k) cv[k] = v[k] >= 0 ? level_code(a.code, v[k]) : 0xffu;
-#pragma unroll
-        for (int k = 0; k < BC_ITEMS; ++k)
-            if (cv[k] == cd) atomicAdd(a.acc + v[k], x[k]);              // result unused: reduction
-        i0 = (next_start == e1) ? i0 + n : i0 + n - 1;
-        __syncwarp();
-    }
+    });
 }
 
 // After a backward push: every vertex of level d finishes from acc.
@@ -725,9 +735,10 @@ __global__ void __launch_bounds__(BC_BLOCK, BC_MIN_BLOCKS) k_bc_persistent(BcArg
     }
     __syncthreads();
     for (;;) {
-        const BcState st = s_st;
+        const BcState &st = s_st;
         if (st.done) break;
         if (blockIdx.x == 0 && threadIdx.x == 0) {
+            a.ctl->wq[(st.phase + 2) & 3] = 0u;
             if (st.op == BOP_FWD || st.op == BOP_FWD_BMP || st.op == BOP_FWD_PULL) {
                 a.ctl->qpack[(st.d + 2) & 3] = 0ull;
                 a.lstart[st.d] = st.start;
@@ -785,6 +796,7 @@ __global__ void k_bc_init(int32_t src, const OffT *ro, uint32_t *code, double *s
     E[0] = 0;
     R[0] = ro[src];
     for (int i = 0; i < 4; ++i) ctl->qpack[i] = 0ull;
+    for (int i = 0; i < 4; ++i) ctl->wq[i] = 0u;
     for (int i = 0; i < 3; ++i) ctl->bcfix[i] = 0u;
 }
 
