@@ -158,8 +158,10 @@ __device__ __forceinline__ bool narrow_exchange(NarrowWord *lines, NarrowShared<
 }
 
 // The same for a group of up to NT = blockDim.x blocks: every thread waits for a
-// line.  No fence: what the blocks leave for each other beside the pieces has
-// to have reached L2 (atomics whose results were used).
+// line.  What the blocks wrote before (distances: reductions, which nobody waits
+// for) is visible to all of them after it: each block's writes come before thread
+// 0's fence through the __syncthreads, the line after it, and a thread's fence
+// after the line it read and before the block's next __syncthreads.
 template <int NT, int NB>
 __device__ __forceinline__ bool narrow_exchange_wide(NarrowWord *lines, NarrowShared<NB> &sh, int group,
                                                      unsigned long long tag, TravCtl *ctl,
@@ -167,11 +169,14 @@ __device__ __forceinline__ bool narrow_exchange_wide(NarrowWord *lines, NarrowSh
     static_assert(NT <= NB, "a line a thread");
     __shared__ uint32_t ws[4][NT / 32];              // per warp: pieces, vertices, edges, largest segment
     __syncthreads();
-    if (threadIdx.x == 0) narrow_publish(lines, sh, tag, false);
+    if (threadIdx.x == 0) narrow_publish(lines, sh, tag, true);
     const unsigned int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     uint32_t q = 0u, p = 0u, e = 0u;
     bool ok = true;
-    if ((int)threadIdx.x < group) ok = narrow_collect(lines + threadIdx.x, tag, q, p, e, timeout_ns);
+    if ((int)threadIdx.x < group) {
+        ok = narrow_collect(lines + threadIdx.x, tag, q, p, e, timeout_ns);
+        __threadfence();
+    }
     uint32_t cp = p;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {

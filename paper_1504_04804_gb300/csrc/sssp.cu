@@ -358,18 +358,12 @@ __device__ void far_split(const SsspArgs<OffT> &a, const SsState &st) {
 // and the source's distance; the target's distance and row bounds) and one for
 // the claim: the minimum and the round stamp are taken at once.  A proposal that
 // beats the distance read means that the target improves in this round, by it or
-// by a smaller one, so whoever sets the stamp may queue the target.  On a weighted
-// 4096 x 4096 grid (rounds of 170,000 edges on average) a round took 22.5 us on the
-// queue (search in the degree prefix, row lookup, global append counter, barrier)
-// and takes 11.6, rounds of 100 edges 13 and 7; the traversal 131 -> 78 ms.
+// by a smaller one, so whoever sets the stamp may queue the target.  The minima
+// are visible to the next round's reads through the exchange's fences.  A weighted
+// 4096 x 4096 grid (rounds of 170,000 edges on average) takes 87 ms, and 158 ms with
+// every round on the queue (search in the degree prefix, row lookup, global append
+// counter, barrier).
 // ---------------------------------------------------------------------------
-// atomicMin that has taken effect when it returns (the result is waited for).
-__device__ __forceinline__ void ss_min_done(uint32_t *p, uint32_t x) {
-    uint32_t old;
-    asm volatile("atom.relaxed.gpu.global.min.u32 %0, [%1], %2;" : "=r"(old) : "l"(p), "r"(x) : "memory");
-    asm volatile("{\n\t.reg .u32 sink;\n\tmov.u32 sink, %0;\n\t}" ::"r"(old));
-}
-
 template <typename OffT>
 __device__ __forceinline__ void ss_list_append(const SsspArgs<OffT> &a, NarrowShared<SS_LIST_BLOCKS> &sh, int L,
                                                unsigned long long tag, bool has, int32_t v, uint32_t row,
@@ -442,7 +436,7 @@ __device__ __forceinline__ void list_round(const SsspArgs<OffT> &a, const SsStat
             if (nd[k] < cur[k]) {
                 if (nd[k] < st.thr) stamp[k] = atomicExch(a.stamp + v[k], L + 1);
                 else far_push(a, st, v[k]);
-                ss_min_done(a.dist + v[k], nd[k]);
+                atomicMin(a.dist + v[k], nd[k]);   // result unused: a reduction, ordered by the exchange
             }
         }
 #pragma unroll
