@@ -382,17 +382,11 @@ __global__ void k_validate64(const int64_t *ro, const int64_t *col, int64_t nv, 
 grx_status ensure_ws64(grx_graph *g, cudaStream_t s) {
     if (g->ws64_ready) return GRX_OK;
     const size_t nv = (size_t)g->nv64, wb = (size_t)g->words * 4;
-    g->visited = (uint32_t *)grx_alloc(g, wb, s);
-    for (int i = 0; i < 3; ++i) g->fbits[i] = (uint32_t *)grx_alloc(g, wb, s);
-    for (int i = 0; i < 2; ++i) g->q64[i] = (int64_t *)grx_alloc(g, nv * 8, s);
-    for (int i = 0; i < 3; ++i) g->lr64[i] = (int64_t *)grx_alloc(g, nv * 8, s);
-    g->ctl = (TravCtl *)grx_alloc(g, sizeof(TravCtl), s);
-    g->bar_flags = (unsigned int *)grx_alloc(g, sizeof(unsigned int) * GRX_MAX_GRID, s);
-    bool ok = g->visited && g->ctl && g->bar_flags;
-    for (int i = 0; i < 3; ++i) ok = ok && g->fbits[i] && g->lr64[i];
-    for (int i = 0; i < 2; ++i) ok = ok && g->q64[i];
+    bool ok = grx_have(g, g->visited, wb, s) && grx_have(g, g->ctl, sizeof(TravCtl), s, true) &&
+              grx_have(g, g->bar_flags, sizeof(unsigned int) * GRX_MAX_GRID, s);
+    for (int i = 0; i < 3; ++i) ok = ok && grx_have(g, g->fbits[i], wb, s) && grx_have(g, g->lr64[i], nv * 8, s);
+    for (int i = 0; i < 2; ++i) ok = ok && grx_have(g, g->q64[i], nv * 8, s);
     if (!ok) return grx_fail(GRX_ENOMEM, "bfs64: workspace allocation failed (nv=%lld)", (long long)g->nv64);
-    GRX_CUDA(cudaMemsetAsync(g->ctl, 0, sizeof(TravCtl), s));
     g->ws64_ready = 1;
     return GRX_OK;
 }

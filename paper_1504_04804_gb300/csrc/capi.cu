@@ -340,25 +340,15 @@ grx_status grx_ensure_workspace(grx_graph *g, cudaStream_t s) {
     if (g->ws_ready) return GRX_OK;
     const size_t nv = (size_t)g->nv;
     const size_t wb = (size_t)g->words * 4;
-    g->visited = (uint32_t *)grx_alloc(g, wb, s);
-    for (int i = 0; i < 3; ++i) {
-        g->fbits[i] = (uint32_t *)grx_alloc(g, wb, s);
-        g->qv[i] = (int32_t *)grx_alloc(g, nv * 4, s);
-        g->qe[i] = (uint32_t *)grx_alloc(g, nv * 4, s);
-        g->qr[i] = grx_alloc(g, nv * (g->off64 ? 8 : 4), s);
-    }
-    for (int i = 0; i < 2; ++i) g->ulist[i] = (int32_t *)grx_alloc(g, nv * 4, s);
-    g->first2 = (int2 *)grx_alloc(g, nv * sizeof(int2), s);
-    g->ctl = (TravCtl *)grx_alloc(g, sizeof(TravCtl), s);
-    g->bar_flags = (unsigned int *)grx_alloc(g, sizeof(unsigned int) * GRX_MAX_GRID, s);
-    g->stats = (DevStats *)grx_alloc(g, sizeof(DevStats), s);
-    g->stamp = (int32_t *)grx_alloc(g, nv * 4, s);
-    bool ok = g->visited && g->ctl && g->bar_flags && g->stats && g->stamp && g->first2;
-    for (int i = 0; i < 3; ++i) ok = ok && g->fbits[i] && g->qv[i] && g->qe[i] && g->qr[i];
-    for (int i = 0; i < 2; ++i) ok = ok && g->ulist[i];
+    bool ok = grx_have(g, g->visited, wb, s);
+    for (int i = 0; i < 3; ++i)
+        ok = grx_have(g, g->fbits[i], wb, s) && grx_have(g, g->qv[i], nv * 4, s) && grx_have(g, g->qe[i], nv * 4, s) &&
+             grx_have(g, g->qr[i], nv * (g->off64 ? 8 : 4), s) && ok;
+    for (int i = 0; i < 2; ++i) ok = grx_have(g, g->ulist[i], nv * 4, s) && ok;
+    ok = grx_have(g, g->first2, nv * sizeof(int2), s) && grx_have(g, g->ctl, sizeof(TravCtl), s, true) &&
+         grx_have(g, g->bar_flags, sizeof(unsigned int) * GRX_MAX_GRID, s) &&
+         grx_have(g, g->stats, sizeof(DevStats), s, true) && grx_have(g, g->stamp, nv * 4, s) && ok;
     if (!ok) return grx_fail(GRX_ENOMEM, "traversal workspace allocation failed (nv=%d)", g->nv);
-    GRX_CUDA(cudaMemsetAsync(g->ctl, 0, sizeof(TravCtl), s));
-    GRX_CUDA(cudaMemsetAsync(g->stats, 0, sizeof(DevStats), s));
     grx_status st = grx_build_first2(g, s);
     if (st != GRX_OK) return st;
     g->ws_ready = 1;
@@ -370,10 +360,9 @@ grx_status grx_ensure_ms_workspace(grx_graph *g, cudaStream_t s) {
     if (st != GRX_OK) return st;
     if (g->ms_ready) return GRX_OK;
     const size_t b = (size_t)g->nv * 8;
-    for (int i = 0; i < 3; ++i) g->ms_cur[i] = (unsigned long long *)grx_alloc(g, b, s);
-    g->ms_next = (unsigned long long *)grx_alloc(g, b, s);
-    g->ms_seen = (unsigned long long *)grx_alloc(g, b, s);
-    if (!g->ms_cur[0] || !g->ms_cur[1] || !g->ms_cur[2] || !g->ms_next || !g->ms_seen)
+    bool ok = grx_have(g, g->ms_next, b, s) && grx_have(g, g->ms_seen, b, s);
+    for (int i = 0; i < 3; ++i) ok = ok && grx_have(g, g->ms_cur[i], b, s);
+    if (!ok)
         return grx_fail(GRX_ENOMEM, "multi-source workspace allocation failed (nv=%d)", g->nv);
     g->ms_ready = 1;
     return GRX_OK;
@@ -383,10 +372,25 @@ grx_status grx_ensure_ms_workspace(grx_graph *g, cudaStream_t s) {
 static size_t workspace_new_bytes(const grx_graph *g, bool multi) {
     const size_t nv = (size_t)g->nv, wb = (size_t)g->words * 4;
     size_t b = 0;
-    if (!g->ws_ready)
-        b += wb + 3 * (wb + nv * 8 + nv * (g->off64 ? 8 : 4)) + 2 * nv * 4 + nv * sizeof(int2) +
-             sizeof(TravCtl) + sizeof(unsigned int) * GRX_MAX_GRID + sizeof(DevStats) + nv * 4;
-    if (multi && !g->ms_ready) b += 5 * nv * 8;
+    auto need = [&](const void *p, size_t bytes) { b += p ? 0 : bytes; };
+    need(g->visited, wb);
+    for (int i = 0; i < 3; ++i) {
+        need(g->fbits[i], wb);
+        need(g->qv[i], nv * 4);
+        need(g->qe[i], nv * 4);
+        need(g->qr[i], nv * (g->off64 ? 8 : 4));
+    }
+    for (int i = 0; i < 2; ++i) need(g->ulist[i], nv * 4);
+    need(g->first2, nv * sizeof(int2));
+    need(g->ctl, sizeof(TravCtl));
+    need(g->bar_flags, sizeof(unsigned int) * GRX_MAX_GRID);
+    need(g->stats, sizeof(DevStats));
+    need(g->stamp, nv * 4);
+    if (multi) {
+        need(g->ms_next, nv * 8);
+        need(g->ms_seen, nv * 8);
+        for (int i = 0; i < 3; ++i) need(g->ms_cur[i], nv * 8);
+    }
     return b;
 }
 
@@ -508,13 +512,9 @@ extern "C" grx_status bc(grx_graph *g, const int32_t *srcs_host, int n, double *
     g->last_stream = stream;
     cudaStream_t s = (cudaStream_t)stream;
     if ((st = grx_ensure_workspace(g, s))) return st;
-    if (!g->bc_sigma) {
-        g->bc_sigma = (double *)grx_alloc(g, (size_t)g->nv * 8, s);
-        g->bc_acc = (double *)grx_alloc(g, (size_t)g->nv * 8, s);
-        g->bc_code = (uint32_t *)grx_alloc(g, (size_t)g->words * 8, s);
-        if (!g->bc_sigma || !g->bc_acc || !g->bc_code)
-            return grx_fail(GRX_ENOMEM, "bc: workspace allocation failed (nv=%d)", g->nv);
-    }
+    if (!grx_have(g, g->bc_sigma, (size_t)g->nv * 8, s) || !grx_have(g, g->bc_acc, (size_t)g->nv * 8, s) ||
+        !grx_have(g, g->bc_code, (size_t)g->words * 8, s))
+        return grx_fail(GRX_ENOMEM, "bc: workspace allocation failed (nv=%d)", g->nv);
     return grx_bc_launch(g, srcs_host, n, bc_out, sigma_out, &o, s);
 }
 
@@ -562,17 +562,11 @@ extern "C" grx_status bc_multi(grx_graph *g, const int32_t *srcs_host, int n, do
     g->last_stream = stream;
     cudaStream_t s = (cudaStream_t)stream;
     if ((st = grx_ensure_workspace(g, s))) return st;
-    if (!g->bcm_sig) {
-        const size_t nv = (size_t)g->nv;
-        g->bcm_seen = (unsigned long long *)grx_alloc(g, nv * 8, s);
-        g->bcm_next = (unsigned long long *)grx_alloc(g, nv * 8, s);
-        g->bcm_hist = (unsigned long long *)grx_alloc(g, nv * 8 * GRX_BCM_MAX_LEVELS, s);
-        g->bcm_sig = (double *)grx_alloc(g, nv * 64 * 8, s);
-        g->bcm_acc = (double *)grx_alloc(g, nv * 64 * 8, s);
-        g->bcm_srcs = (int32_t *)grx_alloc(g, 64 * 4, s);
-        if (!g->bcm_seen || !g->bcm_next || !g->bcm_hist || !g->bcm_sig || !g->bcm_acc || !g->bcm_srcs)
-            return grx_fail(GRX_ENOMEM, "bc_multi: workspace allocation failed (nv=%d)", g->nv);
-    }
+    const size_t nv = (size_t)g->nv;
+    if (!grx_have(g, g->bcm_seen, nv * 8, s) || !grx_have(g, g->bcm_next, nv * 8, s) ||
+        !grx_have(g, g->bcm_hist, nv * 8 * GRX_BCM_MAX_LEVELS, s) || !grx_have(g, g->bcm_sig, nv * 64 * 8, s) ||
+        !grx_have(g, g->bcm_acc, nv * 64 * 8, s) || !grx_have(g, g->bcm_srcs, 64 * 4, s))
+        return grx_fail(GRX_ENOMEM, "bc_multi: workspace allocation failed (nv=%d)", g->nv);
     return grx_bcm_launch(g, srcs_host, n, bc_out, &o, s);
 }
 

@@ -171,6 +171,17 @@ struct grx_graph {
 bool grx_capturing(cudaStream_t s);
 // Allocation through the context allocator (or cudaMallocAsync).
 void *grx_alloc(grx_graph *g, size_t bytes, cudaStream_t s);
+// A workspace buffer: allocated (and zeroed, where asked) unless it is there.  Every
+// buffer stands for itself alone, so that a call that was refused memory can be made
+// again and asks for what it still lacks.
+template <typename T>
+bool grx_have(grx_graph *g, T *&p, size_t bytes, cudaStream_t s, bool zero = false) {
+    if (p) return true;
+    void *q = grx_alloc(g, bytes, s);
+    if (q && zero && cudaMemsetAsync(q, 0, bytes, s) != cudaSuccess) return false;
+    p = (T *)q;
+    return q != nullptr;
+}
 void *grx_ctx_alloc(grx_ctx *c, size_t bytes, cudaStream_t s);
 void grx_ctx_free(grx_ctx *c, void *p, size_t bytes, cudaStream_t s);
 grx_status grx_ensure_workspace(grx_graph *g, cudaStream_t s);

@@ -873,6 +873,8 @@ size_t ms_rest_bytes(const grx_graph *g) {
     return (size_t)(g->ne / (MS_HEAD + 3) + g->ne / MS_PIECE + 1) * sizeof(int2);
 }
 
+size_t ms_tbits_bytes(const grx_graph *g) { return (size_t)g->words * 4 + 16; }
+
 template <typename OffT, bool STATS>
 grx_status ms_launch_typed(grx_graph *g, const int32_t *srcs, int n, int32_t *depth,
                            const grx_opts *o, cudaStream_t s) {
@@ -885,15 +887,10 @@ grx_status ms_launch_typed(grx_graph *g, const int32_t *srcs, int n, int32_t *de
     a.aoff = g->aoff;
     a.first2 = g->first2;
     a.n_active = g->n_active;
-    if (!g->ms_rest) {
-        g->ms_sat = (uint8_t *)grx_alloc(g, ms_sat_bytes(g), s);
-        g->ms_rest = g->ms_sat ? (int2 *)grx_alloc(g, ms_rest_bytes(g), s) : nullptr;
-        for (int i = 0; i < MS_HSLOTS && g->ms_rest; ++i) {
-            g->ms_hist[i] = (unsigned long long *)grx_alloc(g, (size_t)g->nv * 8, s);
-            if (!g->ms_hist[i]) return grx_fail(GRX_ENOMEM, "bfs_multi: history slot allocation failed");
-        }
-        if (!g->ms_rest) return grx_fail(GRX_ENOMEM, "bfs_multi: workspace allocation failed");
-    }
+    bool ok = grx_have(g, g->ms_sat, ms_sat_bytes(g), s) && grx_have(g, g->ms_rest, ms_rest_bytes(g), s) &&
+              grx_have(g, g->ms_tbits, ms_tbits_bytes(g), s, true);
+    for (int i = 0; i < MS_HSLOTS; ++i) ok = ok && grx_have(g, g->ms_hist[i], (size_t)g->nv * 8, s);
+    if (!ok) return grx_fail(GRX_ENOMEM, "bfs_multi: workspace allocation failed (nv=%d)", g->nv);
     a.rest = g->ms_rest;
     a.sat = g->ms_sat;
     for (int i = 0; i < MS_HSLOTS; ++i) a.hist[i] = g->ms_hist[i];
@@ -909,11 +906,6 @@ grx_status ms_launch_typed(grx_graph *g, const int32_t *srcs, int n, int32_t *de
         a.R[i] = (OffT *)g->qr[i];
     }
     a.touched = g->ulist[0];
-    if (!g->ms_tbits) {
-        g->ms_tbits = (uint32_t *)grx_alloc(g, (size_t)g->words * 4 + 16, s);
-        if (!g->ms_tbits) return grx_fail(GRX_ENOMEM, "bfs_multi: touched bitmap allocation failed");
-        GRX_CUDA(cudaMemsetAsync(g->ms_tbits, 0, (size_t)g->words * 4 + 16, s));
-    }
     a.tbits = g->ms_tbits;
     a.words = g->words;
     {   // bitmap push when a level's edges reach push_bitmap * nv (0 = 1/8, < 0 = never)
@@ -954,8 +946,11 @@ grx_status ms_launch_typed(grx_graph *g, const int32_t *srcs, int n, int32_t *de
 
 size_t grx_msbfs_new_bytes(const grx_graph *g) {
     size_t b = 0;
-    if (!g->ms_rest) b += ms_sat_bytes(g) + ms_rest_bytes(g) + (size_t)MS_HSLOTS * (size_t)g->nv * 8;
-    if (!g->ms_tbits) b += (size_t)g->words * 4 + 16;
+    if (!g->ms_sat) b += ms_sat_bytes(g);
+    if (!g->ms_rest) b += ms_rest_bytes(g);
+    if (!g->ms_tbits) b += ms_tbits_bytes(g);
+    for (int i = 0; i < MS_HSLOTS; ++i)
+        if (!g->ms_hist[i]) b += (size_t)g->nv * 8;
     return b;
 }
 

@@ -473,15 +473,9 @@ size_t grx_mssp_new_bytes(const grx_graph *g) {
 
 grx_status grx_mssp_launch(grx_graph *g, const int32_t *srcs, int n, uint32_t *dist,
                            const grx_opts *o, cudaStream_t s) {
-    if (!g->ms_dist) {
-        g->ms_dist = (uint32_t *)grx_alloc(g, (size_t)g->nv * 64 * sizeof(uint32_t), s);
-        if (!g->ms_dist) return grx_fail(GRX_ENOMEM, "sssp_multi: distance workspace allocation failed");
-    }
-    if (!g->ms_tbits) {
-        g->ms_tbits = (uint32_t *)grx_alloc(g, (size_t)g->words * 4 + 16, s);
-        if (!g->ms_tbits) return grx_fail(GRX_ENOMEM, "sssp_multi: touched bitmap allocation failed");
-        GRX_CUDA(cudaMemsetAsync(g->ms_tbits, 0, (size_t)g->words * 4 + 16, s));
-    }
+    if (!grx_have(g, g->ms_dist, (size_t)g->nv * 64 * sizeof(uint32_t), s) ||
+        !grx_have(g, g->ms_tbits, (size_t)g->words * 4 + 16, s, true))
+        return grx_fail(GRX_ENOMEM, "sssp_multi: workspace allocation failed (nv=%d)", g->nv);
     return g->off64 ? mp_launch_typed<int64_t>(g, srcs, n, dist, o, s)
                     : mp_launch_typed<int32_t>(g, srcs, n, dist, o, s);
 }

@@ -502,15 +502,11 @@ grx_status prb_build(grx_graph *g, int shift, cudaStream_t s) {
 
 grx_status grx_pr_launch(grx_graph *g, float damping, int iters, float *rank, cudaStream_t s) {
     const int64_t ntiles = (g->ne + PR_TILE - 1) / PR_TILE;
-    if (!g->pr_c[0]) {
-        g->pr_c[0] = (float *)grx_alloc(g, (size_t)g->nv * 4 + 16, s);   // + the padding's entry
-        g->pr_c[1] = (float *)grx_alloc(g, (size_t)g->nv * 4 + 16, s);
-        g->pr_s = (float *)grx_alloc(g, (size_t)g->nv * 4, s);
-        g->pr_fix = (int32_t *)grx_alloc(g, (size_t)(ntiles > 0 ? ntiles : 1) * 4, s);
-        if (!g->pr_c[0] || !g->pr_c[1] || !g->pr_s || !g->pr_fix)
-            return grx_fail(GRX_ENOMEM, "pagerank: workspace allocation failed");
-        GRX_CUDA(cudaMemsetAsync(g->pr_s, 0, (size_t)g->nv * 4, s));
-    }
+    const size_t nv = (size_t)g->nv;
+    if (!grx_have(g, g->pr_c[0], nv * 4 + 16, s) || !grx_have(g, g->pr_c[1], nv * 4 + 16, s) ||   // + the padding's entry
+        !grx_have(g, g->pr_s, nv * 4, s, true) ||
+        !grx_have(g, g->pr_fix, (size_t)(ntiles > 0 ? ntiles : 1) * 4, s))
+        return grx_fail(GRX_ENOMEM, "pagerank: workspace allocation failed");
     // column blocks only when asked for: on GB300 at R-MAT scale 26 the
     // unblocked gathers (22.5 ms per iteration) beat 2^21..2^25-vertex
     // blocks (32..38 ms), the extra segment reads and reductions costing

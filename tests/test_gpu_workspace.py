@@ -1,0 +1,129 @@
+"""Device memory of the graphs, seen through the allocator: what a refused
+request leaves behind."""
+import ctypes
+
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+
+import oracle
+from paper_1504_04804_gb300 import build, inputs
+from recording_allocator import recorded
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def grx():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    build.build()
+    oracle.build()
+    from paper_1504_04804_gb300 import grx as g
+    return g
+
+
+# Each entry point on a graph (R-MAT or grid), and the oracle's result for it.
+def _bfs(grx, dg, g, srcs):
+    return grx.bfs(dg, srcs[0]).cpu().numpy(), oracle.bfs(g.row_offsets, g.col_indices, srcs[0])
+
+
+def _sssp(grx, dg, g, srcs):
+    return (grx.as_uint32(grx.sssp(dg, srcs[0], opts=grx.opts(sssp_delta=40))),
+            oracle.sssp(g.row_offsets, g.col_indices, g.weights, srcs[0]))
+
+
+def _pagerank(grx, dg, g, srcs):
+    return grx.pagerank(dg, 0.85, 20).cpu().numpy(), oracle.pagerank(g.row_offsets, g.col_indices, 0.85, 20)
+
+
+def _bc(grx, dg, g, srcs):
+    return grx.bc(dg, srcs[:2]).cpu().numpy(), oracle.bc(g.row_offsets, g.col_indices, srcs[:2])
+
+
+def _bc_multi(grx, dg, g, srcs):
+    return grx.bc_multi(dg, srcs).cpu().numpy(), oracle.bc(g.row_offsets, g.col_indices, srcs)
+
+
+def _bfs_multi(grx, dg, g, srcs):
+    return (grx.bfs_multi(dg, srcs).cpu().numpy(),
+            np.stack([oracle.bfs(g.row_offsets, g.col_indices, s) for s in srcs]))
+
+
+def _sssp_multi(grx, dg, g, srcs):
+    return (grx.as_uint32(grx.sssp_multi(dg, srcs)),
+            np.stack([oracle.sssp(g.row_offsets, g.col_indices, g.weights, s) for s in srcs]))
+
+
+def _bfs64(grx, dg, g, srcs):
+    return grx.bfs64(dg, srcs[0]).cpu().numpy(), oracle.bfs(g.row_offsets, g.col_indices, srcs[0])
+
+
+CALLS = {f.__name__[1:]: f for f in (_bfs, _sssp, _pagerank, _bc, _bc_multi, _bfs_multi, _sssp_multi, _bfs64)}
+
+
+@pytest.fixture(scope="module")
+def graphs():
+    r = inputs.rmat_graph(10, 16, seed=10, wmax=64, weight_seed=11)
+    t = inputs.grid_graph(61, 47, p_del=0.1, seed=4)
+    t = inputs.Graph(t.name, t.row_offsets, t.col_indices, inputs.edge_weights(t.row_offsets, t.col_indices, 50, 5))
+    return {"rmat": r, "grid": t}
+
+
+def _load(grx, call, g):
+    if call == "bfs64":
+        return grx.graph_load_csr64(g.row_offsets, g.col_indices)
+    return grx.load(g)
+
+
+def _check(grx, call, dg, g):
+    srcs = [int(s) for s in inputs.pick_sources(g.row_offsets, 5, seed=2)]
+    got, want = CALLS[call](grx, dg, g, srcs)
+    grx.graph_status(dg)
+    if want.dtype.kind == "f":
+        assert np.allclose(got, want, rtol=1e-5 if call == "pagerank" else 1e-9, atol=0)
+    else:
+        assert np.array_equal(got, want)
+
+
+def _footprint(grx, call, dg):
+    kind = {"bfs_multi": grx.GRX_KIND_BFS, "sssp_multi": grx.GRX_KIND_SSSP}.get(call)
+    return None if kind is None else grx.multi_footprint(dg, kind)
+
+
+@pytest.mark.parametrize("name", ["rmat", "grid"])
+@pytest.mark.parametrize("call", list(CALLS))
+def test_a_call_that_was_refused_memory_can_be_made_again(grx, graphs, call, name):
+    """Every request of the first call refused in turn: it says GRX_ENOMEM (or does without), the second call
+    gives the result, and both together hold what one call holds that was not refused."""
+    g = graphs[name]
+    if call == "bc_multi" and name == "grid":
+        pytest.skip("deeper than bc_multi's levels")
+    with recorded(grx) as mem:
+        dg = _load(grx, call, g)
+        first = mem.asked
+        _check(grx, call, dg, g)
+        requests, held = mem.asked - first, sorted(n for _, n in mem.live.values())
+        dg.free()
+        assert not mem.live
+    assert requests > 0
+    for k in range(requests):
+        with recorded(grx, refuse=[first + k]) as mem:
+            dg = _load(grx, call, g)
+            done = True
+            try:
+                _check(grx, call, dg, g)
+            except grx.GrxError as e:
+                assert e.status == grx.GRX_ENOMEM, k
+                done = False
+            assert mem.refused == 1
+            need, used = _footprint(grx, call, dg), mem.used()
+            _check(grx, call, dg, g)
+            assert need is None or mem.used() - used == need, k
+            now = [n for _, n in mem.live.values()]
+            for n in held:
+                now.remove(n)
+            assert done or not now, k                # a call that did without may keep what it used instead
+            dg.free()
+            assert not mem.live
