@@ -837,7 +837,7 @@ grx_status launch_typed(grx_graph *g, const int32_t *srcs, int n, double *bc_out
     }
     int max_grid = per_sm * g->ctx->num_sms;
     if (max_grid > GRX_MAX_GRID) max_grid = GRX_MAX_GRID;
-    const int blocks = o->grid_blocks > 0 && o->grid_blocks < max_grid ? o->grid_blocks : max_grid;
+    const int blocks = grx_grid(o, BC_BLOCK, max_grid);
     const size_t nv = (size_t)g->nv;
     GRX_CUDA(cudaMemsetAsync(bc_out, 0, nv * 8, s));
     if (o->ev_begin) GRX_CUDA(cudaEventRecord((cudaEvent_t)o->ev_begin, s));

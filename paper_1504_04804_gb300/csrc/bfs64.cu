@@ -507,7 +507,7 @@ extern "C" grx_status bfs64(grx_graph *g, int64_t src, int32_t *depth_out, int64
     }
     int max_grid = per_sm * g->ctx->num_sms;
     if (max_grid > GRX_MAX_GRID) max_grid = GRX_MAX_GRID;
-    const int blocks = o.grid_blocks > 0 && o.grid_blocks < max_grid ? o.grid_blocks : max_grid;
+    const int blocks = grx_grid(&o, B64_BLOCK, max_grid);
     GRX_CUDA(cudaMemsetAsync(g->bar_flags, 0, sizeof(unsigned int) * (size_t)blocks, s));
     GRX_CUDA(cudaMemsetAsync(&g->ctl->bar_release, 0, sizeof(unsigned int), s));
     void *args[] = {(void *)&a};

@@ -448,7 +448,7 @@ grx_status mp_launch_typed(grx_graph *g, const int32_t *srcs, int n, uint32_t *d
     }
     int max_grid = per_sm * g->ctx->num_sms;
     if (max_grid > GRX_MAX_GRID) max_grid = GRX_MAX_GRID;
-    int blocks = o->grid_blocks > 0 && o->grid_blocks < max_grid ? o->grid_blocks : max_grid;
+    const int blocks = grx_grid(o, MP_BLOCK, max_grid);
     GRX_CUDA(cudaMemsetAsync(g->bar_flags, 0, sizeof(unsigned int) * (size_t)blocks, s));
     GRX_CUDA(cudaMemsetAsync(&g->ctl->bar_release, 0, sizeof(unsigned int), s));
     void *args[] = {(void *)&a};

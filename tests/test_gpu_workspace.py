@@ -1,5 +1,5 @@
 """Device memory of the graphs, seen through the allocator: what a refused
-request leaves behind."""
+request leaves behind, and how many blocks a call ran on."""
 import ctypes
 
 import numpy as np
@@ -127,3 +127,24 @@ def test_a_call_that_was_refused_memory_can_be_made_again(grx, graphs, call, nam
             assert done or not now, k                # a call that did without may keep what it used instead
             dg.free()
             assert not mem.live
+
+
+FLAGS = 4096                             # entries of the grid barrier's flags: a block writes its own, block 0 none
+
+
+@pytest.mark.parametrize("call,threads", [("bfs", 384), ("sssp", 384), ("bfs_multi", 384), ("sssp_multi", 256),
+                                          ("bc", 384), ("bc_multi", 128), ("bfs64", 256)])
+@pytest.mark.parametrize("units", [1, 2, 6, 31])
+def test_grid_blocks_counts_units_of_256_threads(grx, graphs, call, threads, units):
+    """As many blocks as make up grid_blocks x 256 threads, whatever the kernel's block size."""
+    g = graphs["rmat"]
+    with recorded(grx) as mem:
+        dg = _load(grx, call, g)
+        before = set(mem.live)
+        srcs = [int(s) for s in inputs.pick_sources(g.row_offsets, 2, seed=2)]
+        arg = srcs if call in ("bfs_multi", "sssp_multi", "bc", "bc_multi") else srcs[0]
+        getattr(grx, call)(dg, arg, opts=grx.opts(grid_blocks=units))
+        grx.graph_status(dg)
+        (flags,) = [p for p in set(mem.live) - before if mem.live[p][1] == 4 * FLAGS]
+        assert int((mem.words(flags, FLAGS) != 0).sum()) + 1 == -(-units * 256 // threads)
+        dg.free()
