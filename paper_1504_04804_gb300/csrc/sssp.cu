@@ -31,8 +31,9 @@
 // Rounds and phases are separated by the bounded grid barrier.
 //
 // On graphs of few edges a vertex, whose shortest paths take thousands of small
-// rounds, rounds that fit run on lists instead (list_round): the whole grid
-// with the exchange and the pieces of the narrow levels (narrow.cuh).
+// rounds, rounds that fit run on lists instead (list_round): a group of blocks
+// with the exchange and the pieces of the narrow levels (narrow.cuh), while the
+// rest of the grid waits.
 #include "grx_internal.cuh"
 #include "narrow.cuh"
 
@@ -73,6 +74,8 @@ struct SsspArgs {
     NarrowWord *lines, *pieces;
     int32_t *verts;
     uint32_t list_T;                         // edges of a round, at most, per block
+    uint32_t group;                          // blocks that run them, and rounds between two
+    uint32_t list_rounds;                    // grid barriers, at which the others renew their wait
 };
 
 constexpr int SS_LIST_BLOCKS = 512;          // blocks of a list round: at most SS_BLOCK, searched as 512
@@ -83,13 +86,15 @@ __host__ __device__ inline uint32_t ss_list_pieces(uint32_t t) { return t; }
 __host__ __device__ inline uint32_t ss_list_verts(uint32_t t) { return 4 * (t + SS_WARPS * 8 * 2); }
 
 enum { SOP_RELAX, SOP_FINAL, SOP_FARMIN, SOP_FARSPLIT };
+enum { LIST_OFF = 1, LIST_ON = 2 };
 
 struct SsState {
     int L;
     int op;
     int bmp;
     int done;
-    int nolist;                              // run this round on the queue, whatever its size
+    int list;                                // LIST_OFF: the whole grid runs this round, whatever its size;
+                                             // LIST_ON: the group goes on (the other blocks wait again)
     int fsel;                                // current far pile
     uint32_t q, T;
     uint32_t thr;                            // near-far threshold (UINT32_MAX: no bands)
@@ -369,7 +374,7 @@ __device__ __forceinline__ void ss_list_append(const SsspArgs<OffT> &a, NarrowSh
                                                unsigned long long tag, bool has, int32_t v, uint32_t row,
                                                uint32_t deg) {
     const uint32_t cap = ss_list_pieces(a.list_T), vcap = ss_list_verts(a.list_T);
-    const size_t seg = (size_t)(L & 1) * gridDim.x + blockIdx.x;
+    const size_t seg = (size_t)(L & 1) * a.group + blockIdx.x;
     narrow_append(sh, a.pieces + seg * cap, cap, a.verts + seg * vcap, vcap, tag, has, v, row, deg, a.ctl);
 }
 
@@ -378,10 +383,10 @@ __device__ __forceinline__ void list_round(const SsspArgs<OffT> &a, const SsStat
                                            NarrowShared<SS_LIST_BLOCKS> &sh, unsigned long long tag) {
     const int L = st.L;
     const unsigned int lane = threadIdx.x & 31;
-    const uint32_t step = gridDim.x * SS_WARPS * 8;
-    const uint32_t mine = ((threadIdx.x >> 5) * gridDim.x + blockIdx.x) * 8 + (lane >> 2);
+    const uint32_t step = a.group * SS_WARPS * 8;
+    const uint32_t mine = ((threadIdx.x >> 5) * a.group + blockIdx.x) * 8 + (lane >> 2);
     const uint32_t total = sh.first[SS_LIST_BLOCKS], cap = ss_list_pieces(a.list_T);
-    const NarrowWord *segs = a.pieces + (size_t)(L & 1) * gridDim.x * cap;
+    const NarrowWord *segs = a.pieces + (size_t)(L & 1) * a.group * cap;
     for (uint32_t base = 0; base < total; base += 2 * step) {
         const NarrowWord *at[2];
         NarrowWord w[2];
@@ -454,15 +459,16 @@ __device__ __forceinline__ void list_round(const SsspArgs<OffT> &a, const SsStat
 // Whether round st goes on lists (half the limit to come in, the limit to stay).
 template <typename OffT>
 __device__ __forceinline__ bool list_may_start(const SsspArgs<OffT> &a, const SsState &st) {
-    return a.lines && st.op == SOP_RELAX && !st.bmp && !st.nolist && st.T <= a.list_T * gridDim.x / 2;
+    return a.lines && st.op == SOP_RELAX && !st.bmp && st.list != LIST_OFF && st.T <= a.list_T * a.group / 2;
 }
 
-// Runs rounds from s_st on lists while they fit; s_st is then the next phase of
-// the other kind, with its queue.  Every block calls.  false: a wait gave up.
+// Runs rounds from s_st on lists while they fit.  Called by the group's blocks;
+// leaves in ctl->hstate the phase that every block goes on from after the next
+// grid barrier, with its queue.  false: a wait gave up.
 template <typename OffT, bool STATS>
-__device__ __forceinline__ bool list_rounds(const SsspArgs<OffT> &a, SsState &s_st, NarrowShared<SS_LIST_BLOCKS> &sh,
+__device__ __forceinline__ bool list_run(const SsspArgs<OffT> &a, SsState &s_st, NarrowShared<SS_LIST_BLOCKS> &sh,
                                             FlagBarrier &bar) {
-    const int group = (int)gridDim.x;
+    const int group = (int)a.group;
     const unsigned int lane = threadIdx.x & 31;
     // no tag of this stretch was used before: every stretch counts up the epoch
     unsigned long long tag = (unsigned long long)(ld_relaxed_u32(&a.ctl->narrow_epoch) & 0x7fffffffu) << 32;
@@ -476,8 +482,8 @@ __device__ __forceinline__ bool list_rounds(const SsspArgs<OffT> &a, SsState &s_
         const uint32_t q = s_st.q;
         const int32_t *Q = pick3(a.Q[0], a.Q[1], a.Q[2], L % 3);
         const OffT *R = pick3(a.R[0], a.R[1], a.R[2], L % 3);
-        const uint32_t i0 = (uint32_t)((uint64_t)q * blockIdx.x / gridDim.x);
-        const uint32_t i1 = (uint32_t)((uint64_t)q * (blockIdx.x + 1) / gridDim.x);
+        const uint32_t i0 = (uint32_t)((uint64_t)q * blockIdx.x / a.group);
+        const uint32_t i1 = (uint32_t)((uint64_t)q * (blockIdx.x + 1) / a.group);
         for (uint32_t base = i0 + (threadIdx.x & ~31u); base < i1; base += SS_BLOCK) {
             const uint32_t i = base + lane;
             int32_t v = 0;
@@ -493,8 +499,19 @@ __device__ __forceinline__ bool list_rounds(const SsspArgs<OffT> &a, SsState &s_
     }
     ++tag;
     if (!narrow_exchange_wide<SS_BLOCK>(a.lines + (tag & 1) * SS_LIST_BLOCKS, sh, group, tag, a.ctl, a.timeout_ns)) return false;
+    uint32_t ran = 0;
     for (;;) {
-        if (s_st.q == 0 || s_st.T > a.list_T * gridDim.x || sh.most > ss_list_pieces(a.list_T)) break;
+        if (s_st.q == 0 || s_st.T > a.list_T * a.group || sh.most > ss_list_pieces(a.list_T)) break;
+        if (ran == a.list_rounds && a.group < gridDim.x) {   // the other blocks' wait is bounded: renew it
+            if (blockIdx.x == 0 && threadIdx.x == 0) {
+                SsState st = s_st;
+                st.list = LIST_ON;
+                memcpy((void *)a.ctl->hstate[(bar.gen + 1) & 1], &st, sizeof st);
+            }
+            if (!flag_barrier(bar)) return false;
+            ran = 0;
+        }
+        ++ran;
         const int L = s_st.L;
         if (STATS && blockIdx.x == 0 && threadIdx.x == 0 && L < GRX_MAX_LEVELS_STATS) {
             a.stats->level_t0[L] = grx_globaltimer();
@@ -531,7 +548,7 @@ __device__ __forceinline__ bool list_rounds(const SsspArgs<OffT> &a, SsState &s_
         int32_t *Q = pick3(a.Q[0], a.Q[1], a.Q[2], L % 3);
         uint32_t *E = pick3(a.E[0], a.E[1], a.E[2], L % 3);
         OffT *R = pick3(a.R[0], a.R[1], a.R[2], L % 3);
-        const int32_t *mine = a.verts + ((size_t)(L & 1) * gridDim.x + blockIdx.x) * ss_list_verts(a.list_T);
+        const int32_t *mine = a.verts + ((size_t)(L & 1) * a.group + blockIdx.x) * ss_list_verts(a.list_T);
         const uint32_t n = sh.own;
         for (uint32_t base = 0; base < n; base += SS_BLOCK) {
             const uint32_t i = base + threadIdx.x;
@@ -554,24 +571,43 @@ __device__ __forceinline__ bool list_rounds(const SsspArgs<OffT> &a, SsState &s_
         }
     }
     if (blockIdx.x == 0 && threadIdx.x == 0) {
-        a.ctl->narrow_epoch += 1;                // no block reads it before the barrier below
+        a.ctl->narrow_epoch += 1;                // no block reads it before the next grid barrier
         for (int i = 0; i < 4; ++i) {
             a.ctl->qpack[i] = 0ull;
             a.ctl->wq[i] = 0u;
         }
-    }
-    if (!flag_barrier(bar)) return false;
-    if (threadIdx.x == 0) {
-        if (s_st.q) {
-            s_st.nolist = 1;                     // the round it stopped at may look small (one long row)
-            ss_set_kind(a, s_st);
+        SsState st = s_st;
+        st.list = LIST_OFF;                      // a round that did not fit its segments may look small
+        if (st.q) {
+            ss_set_kind(a, st);
         } else {
-            s_st.nfar = ld_relaxed_u32(&a.ctl->farcnt[s_st.fsel]);
-            if (a.delta && s_st.nfar > 0) s_st.op = SOP_FARMIN;
-            else s_st.done = 1;
+            st.nfar = ld_relaxed_u32(&a.ctl->farcnt[st.fsel]);
+            if (a.delta && st.nfar > 0) st.op = SOP_FARMIN;
+            else st.done = 1;
         }
+        memcpy((void *)a.ctl->hstate[(bar.gen + 1) & 1], &st, sizeof st);
     }
-    __syncthreads();
+    return true;
+}
+
+// A stretch of list rounds, for every block of the grid: from s_st to the s_st
+// that all go on from.  false: a wait gave up.
+template <typename OffT, bool STATS>
+__device__ __forceinline__ bool list_rounds(const SsspArgs<OffT> &a, SsState &s_st, NarrowShared<SS_LIST_BLOCKS> &sh,
+                                            FlagBarrier &bar) {
+    const bool in = blockIdx.x < a.group;
+    if (in && !list_run<OffT, STATS>(a, s_st, sh, bar)) return false;
+    do {
+        if (!flag_barrier(bar, in ? 32 : 500)) return false;
+        if (threadIdx.x == 0) {
+            static_assert(sizeof(SsState) <= sizeof a.ctl->hstate[0] && sizeof(SsState) % 4 == 0, "handed over by words");
+            const uint32_t *h = (const uint32_t *)a.ctl->hstate[bar.gen & 1];
+            uint32_t words[sizeof(SsState) / 4];
+            for (int i = 0; i < (int)(sizeof(SsState) / 4); ++i) words[i] = __ldcg(h + i);
+            memcpy(&s_st, words, sizeof s_st);
+        }
+        __syncthreads();
+    } while (s_st.list == LIST_ON);
     return true;
 }
 
@@ -579,7 +615,7 @@ __device__ __forceinline__ bool list_rounds(const SsspArgs<OffT> &a, SsState &s_
 template <typename OffT>
 __device__ SsState ss_next(const SsspArgs<OffT> &a, const SsState &st, bool stats) {
     SsState ns = st;
-    ns.nolist = 0;
+    ns.list = 0;
     if (st.op == SOP_RELAX && st.bmp) {
         ns.op = SOP_FINAL;
         return ns;
@@ -748,28 +784,36 @@ grx_status launch_persistent(grx_graph *g, SsspArgs<OffT> &a, int32_t src, uint3
     }
     int max_grid = per_sm * g->ctx->num_sms;
     if (max_grid > GRX_MAX_GRID) max_grid = GRX_MAX_GRID;
-    // Deep graphs of less than 1M (4M) vertices have rounds of 20,000 edges or
-    // fewer (100,000): 64 blocks (one an SM) then lose less in a round's work than
-    // they save in its exchange.  Grids of 200^2 / 500^2 / 1,500^2 / 4,096^2, us per
-    // round on 64 / 152 / 304 blocks: 5.6 / 6.9 / 7.9, 6.0 / 7.4 / 8.2, 7.0 / 7.5 / 8.4,
-    // 23.4 / 15.2 / 12.8.
-    if (LIST && o->grid_blocks <= 0) {
-        const int few = g->nv < (1 << 20) ? 64 : (g->nv < (1 << 22) ? g->ctx->num_sms : max_grid);
-        if (few < max_grid) max_grid = few;
-    }
-    const int blocks = grx_grid(o, SS_BLOCK, max_grid);
+    int blocks = grx_grid(o, SS_BLOCK, max_grid);
     if (LIST) {
-        const grx_status st = ss_list_buffers(g, max_grid, s);
+        // The group: rounds of deep graphs of less than 1M (4M) vertices hold 20,000
+        // edges or fewer (100,000), and 64 blocks (one an SM) then lose less in a round's
+        // work than they save in its exchange.  Grids of 200^2 / 500^2 / 1,500^2 /
+        // 4,096^2, us per round with 64 / 152 / 304 blocks in the group: 6.0 / 7.2 / 9.0,
+        // 6.2 / 7.2 / 8.4, 10.9 / 9.2 / 9.1, 18.2 / 14.4 / 13.1.  Larger rounds run on
+        // the whole grid.
+        int few = g->nv < (1 << 20) ? 64 : (g->nv < (1 << 22) ? g->ctx->num_sms : max_grid);
+        if (few > max_grid) few = max_grid;
+        const grx_status st = ss_list_buffers(g, few, s);
         if (st != GRX_OK) return st;
-        if (g->ss_lines && blocks <= g->ss_list_blocks) {
+        if (g->ss_lines) {
             const uint32_t t = g->ss_list_T;
             a.lines = (NarrowWord *)g->ss_lines;
             a.pieces = a.lines + 2 * SS_LIST_BLOCKS;
             a.verts = (int32_t *)(a.pieces + 2 * (size_t)g->ss_list_blocks * ss_list_pieces(t));
             a.list_T = t;
+            a.group = (uint32_t)(blocks < g->ss_list_blocks ? blocks : g->ss_list_blocks);
+            // A grid of the group alone where every round is that small: uniform random
+            // graphs of 0.2M / 0.8M / 1.2M / 3.6M edges on 64 blocks 293 / 379 / 453 / 754 us,
+            // on the full grid 322 / 389 / 435 / 567; grids of 200^2 / 500^2 2.5 / 7.0 ms and
+            // 2.7 / 7.5.
+            if (o->grid_blocks <= 0 && g->nv < (1 << 20) && g->ne < (1 << 20)) blocks = g->ss_list_blocks;
+            // a list round takes some ten microseconds: far less than the bound on a wait
+            const unsigned long long n = a.timeout_ns >> 16;
+            a.list_rounds = n < 1 ? 1u : (n > 256 ? 256u : (uint32_t)n);
             // lists are the better form of a large round too, up to their limit,
             // unless the caller set the line for the changed bitmap
-            if (o->push_bitmap == 0.f && a.bmp_min_T <= t * (uint32_t)blocks) a.bmp_min_T = t * (uint32_t)blocks + 1;
+            if (o->push_bitmap == 0.f && a.bmp_min_T <= t * a.group) a.bmp_min_T = t * a.group + 1;
         }
     }
     GRX_CUDA(cudaMemsetAsync(g->bar_flags, 0, sizeof(unsigned int) * (size_t)blocks, s));
@@ -810,7 +854,7 @@ grx_status launch_typed(grx_graph *g, int32_t src, uint32_t *dist, const grx_opt
     a.src = src;
     a.lines = a.pieces = nullptr;
     a.verts = nullptr;
-    a.list_T = 0;
+    a.list_T = a.group = a.list_rounds = 0;
     {   // reduction rounds when a round's edges reach push_bitmap * nv (0 = 1/8, < 0 = never)
         const double pb = o->push_bitmap == 0.f ? 0.125 : (double)o->push_bitmap;
         const double t = pb * (double)g->nv;

@@ -115,3 +115,35 @@ def test_distances_lowered_by_other_blocks_are_seen_in_the_next_round(grx, block
         d = grx.sssp(dg, src, opts=grx.opts(grid_blocks=blocks))
         grx.graph_status(dg)
         assert np.array_equal(grx.as_uint32(d), want)
+
+
+FLAGS = 4096                             # entries of the grid barrier's flags: a block writes its own, block 0 none
+
+
+def _uniform(nv, ne, seed):
+    rng = np.random.default_rng(seed)
+    return nv, rng.integers(0, nv, (ne // 2, 2)).tolist()
+
+
+@pytest.mark.parametrize("nv,ne,full", [(30_000, 120_000, False), (300_000, 1_300_000, True)])
+def test_large_rounds_run_on_the_whole_grid(grx, nv, ne, full):
+    """A sparse graph that is not deep: ten-odd rounds of most of its edges.  The group that runs the small
+    rounds on lists is 64 blocks, the others run the large ones with it."""
+    g = _weighted(*_uniform(nv, ne, 7), wmax=40, seed=3)
+    assert np.diff(g.row_offsets).max() <= 64 and g.ne < 8 * g.nv and (g.ne > 1 << 20) == full
+    with recorded(grx) as mem:
+        dg = grx.load(g)
+        before = set(mem.live)
+        for delta in (0, 10):
+            d = grx.sssp(dg, 1, opts=grx.opts(sssp_delta=delta))
+            grx.graph_status(dg)
+            assert np.array_equal(grx.as_uint32(d), oracle.sssp(g.row_offsets, g.col_indices, g.weights, 1))
+        new = set(mem.live) - before
+        (flags,) = [p for p in new if mem.live[p][1] == 4 * FLAGS]
+        blocks = int((mem.words(flags, FLAGS) != 0).sum()) + 1
+        sms = torch.cuda.get_device_properties(0).multi_processor_count
+        assert blocks == 2 * sms if full else blocks == 64
+        lists = [mem.words(p, LINES).view(2, 512, 4) for p in new if mem.live[p][1] > 4 * LINES
+                 and mem.live[p][1] not in (4 * g.nv, 8 * g.nv)]
+        assert any(x[:, :64].any() and not x[:, 64:].any() for x in lists), "no list round of 64 blocks ran"
+        dg.free()
