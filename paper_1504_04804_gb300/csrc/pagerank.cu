@@ -31,12 +31,19 @@ constexpr int PR_BLOCK = 256;
 constexpr int PR_ITEMS = 9;                  // odd: conflict-free strided smem reads
 constexpr int PR_TILE = PR_BLOCK * PR_ITEMS;
 
-// Iterations a graph must be worth before its rows are sorted (pr_rows.cu);
-// those it ran in CSR order count.  On GB300 the sort takes 1.1 ms at R-MAT 22
-// and 18 ms at R-MAT 26, and every iteration after it is 0.39 and 10.9 ms
-// shorter: it is paid for by the fourth.  Below 16M edges it takes 0.2 ms,
-// mostly launches and allocation, against 0.02-0.04 ms an iteration.
-inline int64_t prs_min_iters(int64_t ne) { return ne >= (16ll << 20) ? 4 : 12; }
+// Iterations a graph must be worth before its rows are sorted (pr_rows.cu); those
+// it ran in CSR order count.  The line lies where a new graph's first pass is no
+// slower for the sort.  On GB300 the sort and what an iteration after it saves:
+// R-MAT 22 0.66 and 0.39 ms, R-MAT 24 2.4 and 1.86 ms, R-MAT 20 0.24 and 0.09 ms: paid
+// for by the third.  With few edges a vertex the saving is smaller: grid of
+// 4096 x 4096 0.52 and 0.08 ms, uniform random of 18M edges 0.25 and 0.04 ms: by the
+// seventh.  Below 16M edges it takes 0.05-0.2 ms, mostly launches and allocation,
+// and saves 0.003-0.023 ms: R-MAT 14 and 16 break even at 16 iterations, grids of
+// 300 and 2,000 squared earlier.
+inline int64_t prs_min_iters(const grx_graph *g) {
+    if (g->ne < (16ll << 20)) return 16;
+    return g->ne >= 8ll * g->nv ? 4 : 7;
+}
 
 struct PrSmem {
     union alignas(16) {
@@ -538,7 +545,7 @@ grx_status grx_pr_launch(grx_graph *g, float damping, int iters, float *rank, cu
         base[(size_t)i] = (float)b;
         riso = b;
     }
-    if (!blocked && ntiles > 0 && (g->prs_cols || g->pr_csr_iters + iters >= prs_min_iters(g->ne))) {
+    if (!blocked && ntiles > 0 && (g->prs_cols || g->pr_csr_iters + iters >= prs_min_iters(g))) {
         int ready = 0;
         grx_status st = grx_prs_build(g, s, &ready);
         if (st != GRX_OK) return st;
