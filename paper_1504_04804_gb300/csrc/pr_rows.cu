@@ -357,6 +357,7 @@ __global__ void __launch_bounds__(PRS_BLOCK, 1) k_prs_iter(PrsIter a) {
                 before = atomicAdd(a.done + r, 1u);
                 __threadfence();
             }
+            __syncwarp();                             // the other lanes read part after lane 0's fence (a shuffle orders no memory)
             if (__shfl_sync(GRX_FULL_MASK, before, 0) + 1 == nc) {
                 float t = 0.f;                        // the row's last chunk: add them up in order
                 for (uint32_t k = lane; k < nc; k += 32) t += __ldcg(a.part + c0 + k);
