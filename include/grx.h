@@ -23,6 +23,11 @@
  *  - One grx_ctx per host thread; a ctx and its graphs are not thread-safe.
  *    Calls on the same graph must be issued on one stream (or ordered by the
  *    caller), because a graph's traversal workspace is shared by its calls.
+ *  - bfs, sssp and pagerank may keep buffers that they can do without (sizes
+ *    below).  They are not allocated where the allocator refuses them or
+ *    while `stream` is captured, and go back when it refuses memory that
+ *    another call on the same graph needs (that call then waits for `stream`
+ *    once), unless a captured graph holds them.
  */
 #ifndef GRX_H
 #define GRX_H
@@ -151,7 +156,9 @@ void grx_opts_default(grx_opts *o);
  * Sec. 6.1).  depth_out: device int32[nv], hop distance from src, -1 if
  * unreached.  parent_out: NULL or device int32[nv]; parent_out[src] = src,
  * -1 if unreached, else a neighbour one level closer (any valid one).
- * opts NULL = defaults.  Invalid src -> GRX_EINVAL. */
+ * opts NULL = defaults.  Invalid src -> GRX_EINVAL.  Graphs of fewer than
+ * eight edges a vertex: 6.4 MB of optional buffers (small levels in a row
+ * are run by a group of blocks). */
 grx_status bfs(grx_graph *g, int32_t src, int32_t *depth_out, int32_t *parent_out,
                const grx_opts *opts, void *stream);
 
@@ -166,7 +173,9 @@ grx_status bfs_multi(grx_graph *g, const int32_t *srcs_host, int n, int32_t *dep
 /* sssp -- Table 1 SSSP: frontier label-correcting relaxation with atomicMin
  * (the paper's min combiner, Sec. 3) until no distance improves.
  * dist_out: device uint32[nv], UINT32_MAX if unreached.  Needs weights
- * (else GRX_EINVAL).  A distance >= UINT32_MAX sets GRX_ERANGE status. */
+ * (else GRX_EINVAL).  A distance >= UINT32_MAX sets GRX_ERANGE status.
+ * Graphs of fewer than eight edges a vertex and no row past 64: up to 62 MB
+ * of optional buffers (small rounds run on lists). */
 grx_status sssp(grx_graph *g, int32_t src, uint32_t *dist_out,
                 const grx_opts *opts, void *stream);
 
@@ -232,7 +241,9 @@ grx_status cc(grx_graph *g, int32_t *label_out, void *stream);
  * (Sec. 7): r0 = 1/N, then `iters` updates
  *   r'[v] = (1-d)/N + d * (sum_{u in N(v)} r[u]/deg(u) + D/N),
  *   D = sum of r over zero-degree vertices.
- * rank_out: device float[nv].  FP32 arithmetic. */
+ * rank_out: device float[nv].  FP32 arithmetic.  Graphs that are ranked for
+ * more than a few iterations keep an optional copy of their rows sorted by
+ * degree: 4 bytes per edge and about 20 per vertex. */
 grx_status pagerank(grx_graph *g, float damping, int iters, float *rank_out, void *stream);
 
 /* grx_pagerank_block -- column-block width of pagerank's gathers.  When the
@@ -295,7 +306,9 @@ grx_status bfs64(grx_graph *g, int64_t src, int32_t *depth_out, int64_t *parent_
  * The first call on a device looks up the array's device address (once per
  * device, with that device current); make that first call before any CUDA
  * stream capture.  Every call shares the array and clears what it needs;
- * calls whose GPU work overlaps race on it, so order them (one stream). */
+ * calls whose GPU work overlaps race on it, so order them (one stream).
+ * There is no room in it for the buffers that bfs() runs small levels with:
+ * on graphs of thousands of levels (grids) bfs() is several times faster. */
 #define GRX_NOALLOC_MAX_NV (1 << 19)
 #define GRX_NOALLOC_SCRATCH_BYTES 23413632
 grx_status bfs_noalloc(int64_t nv, int64_t ne, const int32_t *row_offsets,

@@ -1601,12 +1601,13 @@ grx_status launch_typed(grx_graph *g, int32_t src, int32_t *depth, int32_t *pare
     if (g->ne >= 8ll * g->nv || o->direction == GRX_DIR_PULL)
         return launch_persistent<OffT, PARENT, STATS, false>(g, a, o, s);
     if (!g->narrow && !g->fixed_scratch && !grx_capturing(s)) {
-        g->narrow = (NarrowBuffers *)grx_alloc(g, sizeof(NarrowBuffers), s);
+        g->narrow = (NarrowBuffers *)grx_alloc_optional(g, sizeof(NarrowBuffers), s);
         if (g->narrow) GRX_CUDA(cudaMemsetAsync(g->narrow, 0, sizeof(NarrowBuffers), s));
         a.narrow = g->narrow;
     }
-    return a.narrow ? launch_persistent<OffT, PARENT, STATS, true>(g, a, o, s)
-                    : launch_persistent<OffT, PARENT, STATS, false>(g, a, o, s);
+    if (!a.narrow) return launch_persistent<OffT, PARENT, STATS, false>(g, a, o, s);
+    grx_uses_optional(g, s);
+    return launch_persistent<OffT, PARENT, STATS, true>(g, a, o, s);
 }
 
 template <typename OffT>

@@ -56,7 +56,7 @@ bool grx_capturing(cudaStream_t s) {
     return true;
 }
 
-void *grx_alloc(grx_graph *g, size_t bytes, cudaStream_t s) {
+void *grx_alloc_optional(grx_graph *g, size_t bytes, cudaStream_t s) {
     if (g->nallocs >= (int)(sizeof g->allocs / sizeof g->allocs[0])) return nullptr;
     void *p = grx_ctx_alloc(g->ctx, bytes, s);
     if (p && ((uintptr_t)p & 15)) {              // 16-byte loads; CUDA's own allocators align to 256
@@ -66,6 +66,41 @@ void *grx_alloc(grx_graph *g, size_t bytes, cudaStream_t s) {
     }
     if (p) g->allocs[g->nallocs++] = {p, bytes};
     return p ? (void *)(((uintptr_t)p + 15) & ~(uintptr_t)15) : nullptr;
+}
+
+static void give_back(grx_graph *g, void *p, cudaStream_t s) {
+    for (int i = 0; p && i < g->nallocs; ++i) {
+        const grx_graph::Alloc x = g->allocs[i];
+        if ((char *)p < (char *)x.p || (char *)p >= (char *)x.p + x.n) continue;
+        g->allocs[i] = g->allocs[--g->nallocs];
+        grx_ctx_free(g->ctx, x.p, x.n, s);
+        return;
+    }
+}
+
+// Frees the optional buffers; false: there are none to free.  The calls that used
+// them are ordered before this one, but not necessarily on the stream the allocator
+// knows them by: they are waited for.
+static bool give_back_optional(grx_graph *g, cudaStream_t s) {
+    if (g->keep_optional || !(g->narrow || g->ss_lines || g->prs_cols) || grx_capturing(s)) return false;
+    if (cudaStreamSynchronize(s) != cudaSuccess) return false;
+    give_back(g, g->narrow, s);
+    give_back(g, g->ss_lines, s);
+    give_back(g, g->prs_cols, s);                // the head of the sorted rows' one block
+    g->narrow = nullptr;
+    g->ss_lines = nullptr;
+    g->prs_cols = nullptr;
+    return true;
+}
+
+void *grx_alloc(grx_graph *g, size_t bytes, cudaStream_t s) {
+    void *p = grx_alloc_optional(g, bytes, s);
+    if (!p && give_back_optional(g, s)) p = grx_alloc_optional(g, bytes, s);
+    return p;
+}
+
+void grx_uses_optional(grx_graph *g, cudaStream_t s) {
+    if (!g->keep_optional && grx_capturing(s)) g->keep_optional = 1;
 }
 
 // ---------------------------------------------------------------------------

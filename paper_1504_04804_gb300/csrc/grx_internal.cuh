@@ -151,6 +151,7 @@ struct grx_graph {
     int ss_list_blocks;              // ... blocks they are laid out for
     struct NarrowBuffers *narrow;    // narrow levels of bfs (narrow.cuh), first use
     int fixed_scratch;               // bfs_noalloc's view: nothing may be allocated
+    int keep_optional;               // optional buffers are part of a captured graph
     cudaGraphExec_t bfs_gexec[2];
     void *bfs_gargs;                 // device copy of the call's arguments
     // 64-bit vertex ids (graph_load_csr64): columns, frontier queues and
@@ -169,8 +170,15 @@ struct grx_graph {
 // Whether s is being captured (or may not be asked): no time to allocate what a
 // call can do without.
 bool grx_capturing(cudaStream_t s);
-// Allocation through the context allocator (or cudaMallocAsync).
+// Allocation through the context allocator (or cudaMallocAsync), kept until
+// graph_free.  Where it is refused, the graph's optional buffers (narrow levels, list
+// rounds, sorted PageRank rows) go back and it is asked again.
 void *grx_alloc(grx_graph *g, size_t bytes, cudaStream_t s);
+// The same for an optional buffer: a refusal stands, and the caller does without.
+void *grx_alloc_optional(grx_graph *g, size_t bytes, cudaStream_t s);
+// A call that uses optional buffers says so: while s is captured they are in the
+// captured graph for good, and are not given back any more.
+void grx_uses_optional(grx_graph *g, cudaStream_t s);
 // A workspace buffer: allocated (and zeroed, where asked) unless it is there.  Every
 // buffer stands for itself alone, so that a call that was refused memory can be made
 // again and asks for what it still lacks.

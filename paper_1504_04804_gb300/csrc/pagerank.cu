@@ -550,6 +550,7 @@ grx_status grx_pr_launch(grx_graph *g, float damping, int iters, float *rank, cu
         grx_status st = grx_prs_build(g, s, &ready);
         if (st != GRX_OK) return st;
         if (ready) {
+            grx_uses_optional(g, s);
             grx_prs_init(g, (float)(1.0 / N), g->pr_c[0], g->pr_c[1], s);
             for (int i = 0; i < iters; ++i)
                 grx_prs_iterate(g, g->pr_c[i & 1], g->pr_c[(i + 1) & 1], i == iters - 1 ? rank : nullptr,

@@ -462,7 +462,7 @@ grx_status grx_prs_build(grx_graph *g, cudaStream_t s, int *ready) {
     const size_t tmp_bytes = mat_bytes + label_bytes + src_bytes;
     char *tmp = (char *)grx_ctx_alloc(g->ctx, tmp_bytes, s);
     if (!tmp) return GRX_OK;
-    char *p = (char *)grx_alloc(g, keep, s);
+    char *p = (char *)grx_alloc_optional(g, keep, s);
     if (!p) {
         grx_ctx_free(g->ctx, tmp, tmp_bytes, s);
         return GRX_OK;

@@ -753,7 +753,7 @@ grx_status ss_list_buffers(grx_graph *g, int blocks, cudaStream_t s) {
     const size_t lines = 2 * SS_LIST_BLOCKS * sizeof(NarrowWord);
     const size_t pieces = 2 * (size_t)blocks * ss_list_pieces(t) * sizeof(NarrowWord);
     const size_t verts = 2 * (size_t)blocks * ss_list_verts(t) * sizeof(int32_t);
-    char *p = (char *)grx_alloc(g, lines + pieces + verts, s);
+    char *p = (char *)grx_alloc_optional(g, lines + pieces + verts, s);
     if (!p) return GRX_OK;
     GRX_CUDA(cudaMemsetAsync(p, 0, lines + pieces, s));           // tag 0 is never used
     g->ss_lines = p;
@@ -797,6 +797,7 @@ grx_status launch_persistent(grx_graph *g, SsspArgs<OffT> &a, int32_t src, uint3
         const grx_status st = ss_list_buffers(g, few, s);
         if (st != GRX_OK) return st;
         if (g->ss_lines) {
+            grx_uses_optional(g, s);
             const uint32_t t = g->ss_list_T;
             a.lines = (NarrowWord *)g->ss_lines;
             a.pieces = a.lines + 2 * SS_LIST_BLOCKS;

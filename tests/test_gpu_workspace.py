@@ -1,5 +1,6 @@
 """Device memory of the graphs, seen through the allocator: what a refused
-request leaves behind, and how many blocks a call ran on."""
+request leaves behind, what goes back to make room, captured calls, and how
+many blocks a call ran on."""
 import ctypes
 
 import numpy as np
@@ -147,4 +148,100 @@ def test_grid_blocks_counts_units_of_256_threads(grx, graphs, call, threads, uni
         grx.graph_status(dg)
         (flags,) = [p for p in set(mem.live) - before if mem.live[p][1] == 4 * FLAGS]
         assert int((mem.words(flags, FLAGS) != 0).sum()) + 1 == -(-units * 256 // threads)
+        dg.free()
+
+
+@pytest.fixture(scope="module")
+def long_grid():
+    g = inputs.grid_graph(200, 203, p_del=0.1, seed=4)
+    return inputs.Graph(g.name, g.row_offsets, g.col_indices,
+                        inputs.edge_weights(g.row_offsets, g.col_indices, 50, 5))
+
+
+def _required(grx, g):
+    """Bytes that a graph, pagerank in CSR order and both multi-source calls cannot do without."""
+    with recorded(grx) as mem:
+        dg = grx.load(g)
+        grx.pagerank(dg, 0.85, 1)
+        for call in ("bfs_multi", "sssp_multi"):
+            _check(grx, call, dg, g)
+        used = mem.used()
+        dg.free()
+    return used
+
+
+def test_optional_buffers_go_back_when_memory_is_refused(grx, long_grid):
+    """Calls that fit a budget fit it whatever ran before them: the buffers of narrow levels, of list rounds and of
+    the sorted rows make room, and those calls go on without them."""
+    need = _required(grx, long_grid)
+    with recorded(grx, budget=need) as mem:
+        dg = grx.load(long_grid)
+        grx.cc(dg)
+        before = set(mem.live)
+        for call in ("bfs", "sssp", "pagerank"):
+            _check(grx, call, dg, long_grid)
+        assert len(set(mem.live) - before) >= 3 and mem.refused == 0
+        for call in ("bfs_multi", "sssp_multi"):
+            _check(grx, call, dg, long_grid)
+        assert mem.refused > 0
+        for call in CALLS:
+            if call not in ("bfs64", "bc", "bc_multi"):
+                _check(grx, call, dg, long_grid)
+        dg.free()
+        assert not mem.live
+
+
+def _captured(run):
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        run()
+    return graph
+
+
+@pytest.mark.parametrize("warm", [False, True])
+def test_calls_in_a_captured_graph(grx, long_grid, warm):
+    """bfs, sssp and pagerank captured before the optional buffers are there (the capture allocates nothing and does
+    without) and after (they stay, whatever is refused later); each graph is replayed for the result."""
+    g = long_grid
+    src = int(inputs.pick_sources(g.row_offsets, 1, seed=2)[0])
+    want = {"bfs": oracle.bfs(g.row_offsets, g.col_indices, src),
+            "sssp": oracle.sssp(g.row_offsets, g.col_indices, g.weights, src),
+            "pagerank": oracle.pagerank(g.row_offsets, g.col_indices, 0.85, 20)}
+    need = _required(grx, g)
+    with recorded(grx, budget=need) as mem:
+        dg = grx.load(g)
+        out = {"bfs": torch.empty(g.nv, dtype=torch.int32, device="cuda"),
+               "sssp": torch.empty(g.nv, dtype=torch.int32, device="cuda"),
+               "pagerank": torch.empty(g.nv, dtype=torch.float32, device="cuda")}
+        o = grx.opts(sssp_delta=40)
+        run = {"bfs": lambda: grx.bfs(dg, src, depth_out=out["bfs"]),
+               "sssp": lambda: grx.sssp(dg, src, dist_out=out["sssp"], opts=o),
+               "pagerank": lambda: grx.pagerank(dg, 0.85, 20, rank_out=out["pagerank"])}
+        grx.cc(dg)
+        grx.pagerank(dg, 0.85, 1)
+        before = set(mem.live)
+        if warm:
+            for f in run.values():
+                f()
+            assert len(set(mem.live) - before) >= 3
+        live = set(mem.live)
+        torch.cuda.synchronize()
+        graphs = {k: _captured(f) for k, f in run.items()}
+        assert set(mem.live) == live
+        if warm:                                     # no room: what the graphs use is not given back
+            with pytest.raises(grx.GrxError) as e:
+                grx.bfs_multi(dg, [src] * 4)
+                grx.sssp_multi(dg, [src] * 4)
+            assert e.value.status == grx.GRX_ENOMEM and live <= set(mem.live)
+        for _ in range(3):
+            for k, graph in graphs.items():
+                out[k].fill_(77)
+                graph.replay()
+                grx.graph_status(dg)
+                got = out[k].cpu().numpy()
+                if k == "pagerank":
+                    assert np.max(np.abs(got - want[k]) / want[k]) <= 1e-5
+                else:
+                    assert np.array_equal(got.view(want[k].dtype), want[k]), k
+        del graphs
         dg.free()
