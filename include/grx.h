@@ -54,7 +54,9 @@ typedef struct grx_graph grx_graph;
 typedef struct grx_batch grx_batch;
 
 /* Device-memory allocator.  alloc must return a device pointer usable on
- * `stream` (or NULL on failure); free receives the same pointer and size.
+ * `stream` (or NULL on failure), aligned to 8 bytes at least (what needs
+ * more is aligned inside; below 128 that takes a second request, 128 bytes
+ * larger); free receives the same pointer and size.
  * The library keeps no pointer past the matching free. */
 typedef struct {
     void *(*alloc)(size_t bytes, void *stream, void *user);

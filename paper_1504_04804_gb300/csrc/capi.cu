@@ -59,13 +59,15 @@ bool grx_capturing(cudaStream_t s) {
 void *grx_alloc_optional(grx_graph *g, size_t bytes, cudaStream_t s) {
     if (g->nallocs >= (int)(sizeof g->allocs / sizeof g->allocs[0])) return nullptr;
     void *p = grx_ctx_alloc(g->ctx, bytes, s);
-    if (p && ((uintptr_t)p & 15)) {              // 16-byte loads; CUDA's own allocators align to 256
+    constexpr uintptr_t ALIGN = alignof(TravCtl);   // the widest of all: the compiler counts on it
+    static_assert(ALIGN >= 16, "16-byte loads of every buffer");
+    if (p && ((uintptr_t)p & (ALIGN - 1))) {     // CUDA's own allocators align to 256
         grx_ctx_free(g->ctx, p, bytes, s);
-        bytes += 16;
+        bytes += ALIGN;
         p = grx_ctx_alloc(g->ctx, bytes, s);
     }
     if (p) g->allocs[g->nallocs++] = {p, bytes};
-    return p ? (void *)(((uintptr_t)p + 15) & ~(uintptr_t)15) : nullptr;
+    return p ? (void *)(((uintptr_t)p + ALIGN - 1) & ~(ALIGN - 1)) : nullptr;
 }
 
 static void give_back(grx_graph *g, void *p, cudaStream_t s) {

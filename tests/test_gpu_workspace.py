@@ -245,3 +245,18 @@ def test_calls_in_a_captured_graph(grx, long_grid, warm):
                     assert np.array_equal(got.view(want[k].dtype), want[k]), k
         del graphs
         dg.free()
+
+
+@pytest.mark.parametrize("name", ["rmat", "grid"])
+@pytest.mark.parametrize("call", list(CALLS))
+def test_allocators_that_align_to_eight_bytes(grx, graphs, call, name):
+    """Buffers start where their types want them all the same (16-byte loads, control words on lines of 128 bytes),
+    and go back by the allocator's address."""
+    if call == "bc_multi" and name == "grid":
+        pytest.skip("deeper than bc_multi's levels")
+    with recorded(grx, skew=8) as mem:
+        dg = _load(grx, call, graphs[name])
+        _check(grx, call, dg, graphs[name])
+        _check(grx, call, dg, graphs[name])
+        dg.free()
+        assert not mem.live
