@@ -147,3 +147,17 @@ def test_large_rounds_run_on_the_whole_grid(grx, nv, ne, full):
                  and mem.live[p][1] not in (4 * g.nv, 8 * g.nv)]
         assert any(x[:, :64].any() and not x[:, 64:].any() for x in lists), "no list round of 64 blocks ran"
         dg.free()
+
+
+def test_narrow_levels_run_where_bfs_has_many_small_ones(grx):
+    """The counterpart for BFS (its results are tested with its limits elsewhere): the group's lines are used."""
+    g = inputs.grid_graph(301, 97, p_del=0.1, seed=5)
+    with recorded(grx) as mem:
+        dg = grx.load(g)
+        grx.cc(dg)
+        before = set(mem.live)
+        src = int(inputs.pick_sources(g.row_offsets, 1, seed=3)[0])
+        assert np.array_equal(grx.bfs(dg, src).cpu().numpy(), oracle.bfs(g.row_offsets, g.col_indices, src))
+        (narrow,) = set(mem.live) - before
+        assert int((mem.words(narrow, 2 * 64 * 4) != 0).sum()) > 0, "no narrow level ran"
+        dg.free()
