@@ -22,7 +22,6 @@
 
 namespace {
 
-constexpr int CC_BLOCK = 1024;                // (1,216 blocks of 256 in every grid barrier: R-MAT 22 138 -> 116 us)
 constexpr int CC_SAMPLES = 1024;              // vertices sampled for the largest component
 
 struct CcArgs {
@@ -185,8 +184,15 @@ __device__ void hook_rest(const CcArgs &a, int32_t giant, unsigned long long &li
 // (R-MAT 22 / 24: 114 -> 108, 327 -> 271 us; four 113, 270); one on grids and
 // paths, where labels read ahead are older and more hooks are tried again (grid
 // of 1000 x 1000: 172 us, with two 183).
-template <int FLIGHT>
-__global__ void __launch_bounds__(CC_BLOCK) k_cc_persistent(CcArgs a) {
+// BLOCK: 1,024 threads where the six grid barriers are the time (R-MAT 22 138 -> 116
+// us with a quarter of the blocks; a path of 100,000 217 -> 172).  256 where chains of
+// labels are: past 128K vertices without a vertex joined to a good part of them, the
+// smaller blocks' hooks leave shorter chains (us, 256 / 1,024 threads: ring of 1M
+// vertices with four neighbours and 5 % shortcuts 240 / 468, path of 1M 1,787 / 3,203,
+// grid of 4096 x 4096 1,363 / 1,664, uniform random 16M vertices 3,519 / 4,229, 2M of
+// degree 16 1,606 / 1,764; path of 300,000 337 / 719).
+template <int FLIGHT, int BLOCK>
+__global__ void __launch_bounds__(BLOCK) k_cc_persistent(CcArgs a) {
     FlagBarrier bar{a.bar_flags, &a.ctl->bar_release, a.ctl, a.timeout_ns, 0u};
     for (int64_t v = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; v < a.nv;
          v += (int64_t)gridDim.x * blockDim.x)
@@ -213,22 +219,22 @@ __global__ void __launch_bounds__(CC_BLOCK) k_cc_persistent(CcArgs a) {
     }
 }
 
-template <int FLIGHT>
+template <int FLIGHT, int BLOCK>
 grx_status cc_launch(grx_graph *g, const CcArgs &a, const grx_opts *o, cudaStream_t s) {
     static int per_sm = -1;
     if (per_sm < 0) {
-        GRX_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_cc_persistent<FLIGHT>, CC_BLOCK, 0));
+        GRX_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_cc_persistent<FLIGHT, BLOCK>, BLOCK, 0));
         if (per_sm < 1) return grx_fail(GRX_ECUDA, "cc: persistent kernel does not fit on an SM");
     }
     int max_grid = per_sm * g->ctx->num_sms;
     if (max_grid > GRX_MAX_GRID) max_grid = GRX_MAX_GRID;
-    const int blocks = grx_grid(o, CC_BLOCK, max_grid);
+    const int blocks = grx_grid(o, BLOCK, max_grid);
     GRX_CUDA(cudaMemsetAsync(g->bar_flags, 0, sizeof(unsigned int) * (size_t)blocks, s));
     GRX_CUDA(cudaMemsetAsync(&g->ctl->bar_release, 0, sizeof(unsigned int), s));
     GRX_CUDA(cudaMemsetAsync(&g->stats->levels, 0, sizeof(int32_t), s));
     GRX_CUDA(cudaMemsetAsync(&g->stats->edges_examined[0], 0, sizeof(unsigned long long), s));
     void *args[] = {(void *)&a};
-    GRX_CUDA(cudaLaunchCooperativeKernel((const void *)k_cc_persistent<FLIGHT>, dim3(blocks), dim3(CC_BLOCK),
+    GRX_CUDA(cudaLaunchCooperativeKernel((const void *)k_cc_persistent<FLIGHT, BLOCK>, dim3(blocks), dim3(BLOCK),
                                          args, 0, s));
     return GRX_OK;
 }
@@ -248,5 +254,8 @@ grx_status grx_cc_launch(grx_graph *g, int32_t *label, const grx_opts *o, cudaSt
     a.stats = g->stats;
     a.bar_flags = g->bar_flags;
     a.timeout_ns = grx_timeout_ns(o);
-    return g->ne >= 8ll * g->nv ? cc_launch<2>(g, a, o, s) : cc_launch<1>(g, a, o, s);
+    // paths, meshes, uniform random graphs: no vertex joined to a good part of the graph
+    if (g->nv > 1 << 17 && (g->max_deg <= 64 || g->max_deg <= (uint32_t)g->nv >> 10))
+        return cc_launch<1, 256>(g, a, o, s);
+    return g->ne >= 8ll * g->nv ? cc_launch<2, 1024>(g, a, o, s) : cc_launch<1, 1024>(g, a, o, s);
 }
