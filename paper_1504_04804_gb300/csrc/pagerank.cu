@@ -45,6 +45,12 @@ inline int64_t prs_min_iters(const grx_graph *g) {
     return g->ne >= 8ll * g->nv ? 4 : 7;
 }
 
+// A row with a sixteenth of a million edges or more (a star, or a few) is a critical
+// path of its own: its chunks, their sum.  Such graphs stay in CSR order (stars of 1M
+// leaves on 1 / 4 hubs 16.0 / 18.1 us an iteration, sorted 18.0 / 19.9; on 8 and more
+// sorting is the better form again, as it is for a star of 100,000: 13.6 and 9.4).
+inline bool prs_suits(const grx_graph *g) { return g->ne < (1 << 20) || (int64_t)g->max_deg < g->ne / 16; }
+
 struct PrSmem {
     union alignas(16) {
         float acc[PR_TILE + 2];
@@ -545,7 +551,7 @@ grx_status grx_pr_launch(grx_graph *g, float damping, int iters, float *rank, cu
         base[(size_t)i] = (float)b;
         riso = b;
     }
-    if (!blocked && ntiles > 0 && (g->prs_cols || g->pr_csr_iters + iters >= prs_min_iters(g))) {
+    if (!blocked && ntiles > 0 && prs_suits(g) && (g->prs_cols || g->pr_csr_iters + iters >= prs_min_iters(g))) {
         int ready = 0;
         grx_status st = grx_prs_build(g, s, &ready);
         if (st != GRX_OK) return st;

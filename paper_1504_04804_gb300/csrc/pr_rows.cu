@@ -353,14 +353,18 @@ __global__ void __launch_bounds__(PRS_BLOCK, 1) k_prs_iter(PrsIter a) {
             unsigned int before = 0;
             if (lane == 0) {
                 a.part[c] = s;
-                __threadfence();
-                before = atomicAdd(a.done + r, 1u);
-                __threadfence();
+                asm volatile("atom.acq_rel.gpu.global.add.u32 %0, [%1], 1;" : "=r"(before) : "l"(a.done + r) : "memory");
             }
-            __syncwarp();                             // the other lanes read part after lane 0's fence (a shuffle orders no memory)
+            __syncwarp();                             // the other lanes read part after it (a shuffle orders no memory)
             if (__shfl_sync(GRX_FULL_MASK, before, 0) + 1 == nc) {
                 float t = 0.f;                        // the row's last chunk: add them up in order
-                for (uint32_t k = lane; k < nc; k += 32) t += __ldcg(a.part + c0 + k);
+                for (uint32_t k = lane; k < nc; k += 32 * 8) {
+                    float x[8];
+#pragma unroll
+                    for (int j = 0; j < 8; ++j) x[j] = k + j * 32 < nc ? __ldcg(a.part + c0 + k + j * 32) : 0.f;
+#pragma unroll
+                    for (int j = 0; j < 8; ++j) t += x[j];
+                }
                 t = warp_sum(t);
                 if (lane == 0) {
                     a.done[r] = 0u;
@@ -438,10 +442,15 @@ grx_status grx_prs_build(grx_graph *g, cudaStream_t s, int *ready) {
     if (*ready || g->n_active == 0) return GRX_OK;
     if (grx_capturing(s)) return GRX_OK;
     const int64_t n = g->n_active, ne = g->ne;
-    // chunks of 1,024 edges on large graphs; smaller ones on small graphs, where
-    // a warp's whole share is a few hundred edges.  Rows past eight chunks are
-    // cut, so padding them to whole chunks costs an eighth at most.
-    const int chunk_shift = ne >= (64ll << 20) ? 10 : (ne >= (4ll << 20) ? 8 : 7);
+    // Chunks of 1,024 edges on large graphs, smaller ones on small graphs, where a
+    // warp's whole share is a few hundred edges (per iteration with chunks of 128 / 256 /
+    // 512 edges: R-MAT 16 13.5 / 11.5 / - us, 18 - / 19.8 / 18.0, 20 - / 64.6 / 57.1); but
+    // about a thousand of the longest row at most, which are counted by one word and
+    // added up by one warp (a star of 1M leaves: 7,813 chunks of 128 37 us, 977 of 1,024
+    // 18).  Rows past eight chunks are cut, so padding them to whole chunks costs an
+    // eighth at most.
+    int chunk_shift = ne >= (64ll << 20) ? 10 : (ne >= (4ll << 20) ? 9 : (ne >= (1ll << 20) ? 8 : 7));
+    while (chunk_shift < 12 && g->max_deg >> chunk_shift > 1024) ++chunk_shift;
     const uint32_t longest = 8u << chunk_shift;
     const int long_key = prs_key_log(chunk_shift + 3, 0);
     const int64_t max_long = ne / longest + 1;

@@ -8,6 +8,7 @@ torch = pytest.importorskip("torch")
 
 import oracle
 from paper_1504_04804_gb300 import build, inputs
+from recording_allocator import recorded
 
 pytestmark = pytest.mark.gpu
 
@@ -76,6 +77,35 @@ def _wide(grx, nv, neighbours, seed):
     pairs += [rows(torch.arange(1000, 21_000, device="cuda"), 150), rows(torch.arange(420, device="cuda") * 3, 20_000)]
     u, v = torch.cat([p[0] for p in pairs]), torch.cat([p[1] for p in pairs])
     return grx.build_csr_device(nv, u.to(torch.int32), v.to(torch.int32))
+
+
+def _starred(grx, nv, hub, edges, seed):
+    """A uniform random graph, vertex 3 joined to `hub` others."""
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(seed)
+    u, v = (torch.randint(0, nv, (edges,), device="cuda", generator=gen) for _ in range(2))
+    k = torch.arange(hub, device="cuda") + 10
+    return grx.build_csr_device(nv, torch.cat([u, torch.full_like(k, 3)]).to(torch.int32),
+                                torch.cat([v, k]).to(torch.int32))
+
+
+# chunks by the longest row: 600,000 edges in 587 chunks of 1,024 where others have 512
+# a row with a sixteenth of a million edges and more: CSR order, whatever the iterations
+@pytest.mark.parametrize("nv,hub,edges,is_sorted", [(1_000_000, 600_000, 5_000_000, True),
+                                                    (700_000, 600_000, 100_000, False),
+                                                    (90_000, 80_000, 100_000, True)])
+def test_graphs_with_one_long_row(grx, nv, hub, edges, is_sorted):
+    ro, col = _starred(grx, nv, hub, edges, 4)
+    with recorded(grx) as mem:
+        dg = grx.graph_load_csr(ro, col)
+        grx.pagerank(dg, 0.85, 1)
+        before = set(mem.live)
+        r = grx.pagerank(dg, 0.85, 20)
+        torch.cuda.synchronize()
+        assert bool(set(mem.live) - before) == is_sorted
+        want = oracle.pagerank(ro.cpu().numpy(), col.cpu().numpy(), 0.85, 20)
+        assert np.max(np.abs(r.cpu().numpy().astype(np.float64) - want) / want) <= PR_TOL
+        dg.free()
 
 
 # 64M edges: chunks of 1,024; 2^24 rows: the smaller shared table
