@@ -198,7 +198,7 @@ __device__ __forceinline__ void warp_batches(TravCtl *ctl, int phase, uint64_t T
     if (batch == 0) return;
     const uint64_t nbatch = (ntiles + batch - 1) / batch;
     unsigned int *wq = &ctl->wq[phase & 3];
-    for (uint64_t bt = (uint64_t)blockIdx.x * BC_WARPS + (threadIdx.x >> 5); bt < nbatch;) {
+    for (uint64_t bt = grx_warp(); bt < nbatch;) {
         unsigned int nn = 0;
         if ((threadIdx.x & 31) == 0) nn = atomicAdd(wq, 1u);
         body(bt * batch, min(ntiles, (bt + 1) * batch));
@@ -304,7 +304,7 @@ __device__ void forward_final(const BcArgs<OffT> &a, const BcState &st, uint16_t
     const unsigned int lane = threadIdx.x & 31;
     const int64_t nsc = (a.words + 31) / 32;
     const int64_t nwarps = (int64_t)gridDim.x * BC_WARPS;
-    for (int64_t sc = (int64_t)blockIdx.x * BC_WARPS + (threadIdx.x >> 5); sc < nsc; sc += nwarps) {
+    for (int64_t sc = grx_warp(); sc < nsc; sc += nwarps) {
         const int64_t wd = sc * 32 + lane;
         uint32_t cand = 0u;
         if (wd < a.words)
@@ -484,7 +484,7 @@ __device__ void forward_pull(const BcArgs<OffT> &a, const BcState &st, BcWarpSme
     const unsigned int lane = threadIdx.x & 31;
     const int64_t nsc = (a.words + 31) / 32;
     const int64_t nwarps = (int64_t)gridDim.x * BC_WARPS;
-    for (int64_t sc = (int64_t)blockIdx.x * BC_WARPS + (threadIdx.x >> 5); sc < nsc; sc += nwarps) {
+    for (int64_t sc = grx_warp(); sc < nsc; sc += nwarps) {
         const int64_t wd = sc * 32 + lane;
         uint32_t cand = 0u;
         if (wd < a.words)

@@ -379,6 +379,12 @@ __device__ __forceinline__ bool flag_barrier(FlagBarrier &b, unsigned int sleep_
     return s_ok != 0;
 }
 
+// Number of the calling warp in the grid, neighbours in different blocks: a phase
+// with fewer pieces of work than warps spreads over every SM.  (With neighbours in
+// one block, the 977 bitmap chunks of a million vertices kept 82 blocks of 12 warps
+// busy and 70 SMs idle.)
+__device__ __forceinline__ int64_t grx_warp() { return (int64_t)(threadIdx.x >> 5) * gridDim.x + blockIdx.x; }
+
 // Warp-aggregated append of up to N items per lane (bit k of mask = item k
 // present) to a frontier whose counter packs (count << 32 | edge total).  One
 // atomic per warp; the edge prefix stays monotone in position order.  Must be

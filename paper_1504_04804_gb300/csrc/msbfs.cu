@@ -286,7 +286,7 @@ __device__ void ms_push_expand(const MsArgs<OffT> &a, const MsState &st, MsWarpS
     const uint64_t T = st.T;
     const uint64_t ntiles = (T + MS_WTILE - 1) / MS_WTILE;
     const uint64_t nwarps = (uint64_t)gridDim.x * MS_WARPS;
-    const uint64_t gw = (uint64_t)blockIdx.x * MS_WARPS + (threadIdx.x >> 5);
+    const uint64_t gw = grx_warp();
     const uint64_t per = (ntiles + nwarps - 1) / nwarps;
     const uint64_t tb0 = gw * per;
     const uint64_t tb1 = min(ntiles, tb0 + per);
@@ -411,7 +411,7 @@ __device__ void ms_push_finalize(const MsArgs<OffT> &a, const MsState &st, uint1
         const unsigned int lane = threadIdx.x & 31;
         const int64_t nsc = (a.words + 31) / 32;
         const int64_t nwarps = (int64_t)gridDim.x * MS_WARPS;
-        for (int64_t sc = (int64_t)blockIdx.x * MS_WARPS + (threadIdx.x >> 5); sc < nsc; sc += nwarps) {
+        for (int64_t sc = grx_warp(); sc < nsc; sc += nwarps) {
             const int64_t wd = sc * 32 + lane;
             const uint32_t bits = wd < a.words ? __ldcg(a.tbits + wd) : 0u;
             if (bits) a.tbits[wd] = 0u;
@@ -514,7 +514,7 @@ __device__ void ms_pull(const MsArgs<OffT> &a, const MsState &st, MsPullSmem &w,
     const bool small = R < MS_ROWS;              // few rows a warp: it finishes its longer ones itself
     const int64_t nch = (a.n_active + R - 1) / R;
     const int64_t nwarps = (int64_t)gridDim.x * MS_WARPS;
-    for (int64_t ch = (int64_t)blockIdx.x * MS_WARPS + (threadIdx.x >> 5); ch < nch;) {
+    for (int64_t ch = grx_warp(); ch < nch;) {
         unsigned int nn = 0;
         if (lane == 0) nn = atomicAdd(wq, 1u);
         if (!__ldcg(a.sat + ch)) {
@@ -646,7 +646,7 @@ __device__ void ms_pull_rest(const MsArgs<OffT> &a, const MsState &st, MsCounts 
     const unsigned long long *cin = pk3(a.cur[0], a.cur[1], a.cur[2], st.L % 3);
     const int64_t n = ld_relaxed_u32(&a.ctl->ucount[(st.L + 1) & 3]);
     const int64_t nwarps = (int64_t)gridDim.x * MS_WARPS;
-    for (int64_t t = (int64_t)blockIdx.x * MS_WARPS + (threadIdx.x >> 5); t < n; t += nwarps) {
+    for (int64_t t = grx_warp(); t < n; t += nwarps) {
         const int2 r = __ldcg(a.rest + t);
         const int32_t v = __ldg(a.active + r.x);
         const int64_t e0 = (int64_t)__ldg(a.aoff + r.x) + 2 + MS_HEAD + (int64_t)r.y * MS_PIECE;

@@ -145,7 +145,7 @@ __device__ void relax_round(const SsspArgs<OffT> &a, const SsState &st, SsWarpSm
     const uint64_t T = st.T;
     const uint64_t ntiles = (T + SS_WTILE - 1) / SS_WTILE;
     const uint64_t nwarps = (uint64_t)gridDim.x * SS_WARPS;
-    const uint64_t gw = (uint64_t)blockIdx.x * SS_WARPS + (threadIdx.x >> 5);
+    const uint64_t gw = grx_warp();
     // Batches of up to SS_BATCH tiles: the first by the warp's number, the others
     // from the round's counter.  What a tile costs varies along the queue (R-MAT 22,
     // mean of three sources: one equal share a warp 1,824 us, batches of 16 / 8 / 4 / 2
@@ -271,7 +271,7 @@ __device__ void changed_to_queue(const SsspArgs<OffT> &a, const SsState &st, uin
     const unsigned int lane = threadIdx.x & 31;
     const int64_t nsc = (a.words + 31) / 32;
     const int64_t nwarps = (int64_t)gridDim.x * SS_WARPS;
-    for (int64_t sc = (int64_t)blockIdx.x * SS_WARPS + (threadIdx.x >> 5); sc < nsc; sc += nwarps) {
+    for (int64_t sc = grx_warp(); sc < nsc; sc += nwarps) {
         const int64_t wd = sc * 32 + lane;
         const uint32_t bits = wd < a.words ? __ldcg(a.cbits + wd) : 0u;
         if (bits) a.cbits[wd] = 0u;
