@@ -198,11 +198,12 @@ __device__ __forceinline__ void warp_batches(TravCtl *ctl, int phase, uint64_t T
     if (batch == 0) return;
     const uint64_t nbatch = (ntiles + batch - 1) / batch;
     unsigned int *wq = &ctl->wq[phase & 3];
+    const bool more = nbatch > nwarps;      // else a thousand atomics on one word, for nothing
     for (uint64_t bt = grx_warp(); bt < nbatch;) {
         unsigned int nn = 0;
-        if ((threadIdx.x & 31) == 0) nn = atomicAdd(wq, 1u);
+        if ((threadIdx.x & 31) == 0 && more) nn = atomicAdd(wq, 1u);
         body(bt * batch, min(ntiles, (bt + 1) * batch));
-        bt = nwarps + __shfl_sync(GRX_FULL_MASK, nn, 0);
+        bt = more ? nwarps + __shfl_sync(GRX_FULL_MASK, nn, 0) : nbatch;
     }
 }
 

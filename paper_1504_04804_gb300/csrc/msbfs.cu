@@ -514,9 +514,10 @@ __device__ void ms_pull(const MsArgs<OffT> &a, const MsState &st, MsPullSmem &w,
     const bool small = R < MS_ROWS;              // few rows a warp: it finishes its longer ones itself
     const int64_t nch = (a.n_active + R - 1) / R;
     const int64_t nwarps = (int64_t)gridDim.x * MS_WARPS;
+    const bool more = nch > nwarps;              // else a thousand atomics on one word, for nothing
     for (int64_t ch = grx_warp(); ch < nch;) {
         unsigned int nn = 0;
-        if (lane == 0) nn = atomicAdd(wq, 1u);
+        if (lane == 0 && more) nn = atomicAdd(wq, 1u);
         if (!__ldcg(a.sat + ch)) {
             int32_t v[PER];
             uint32_t s[PER], deg[PER];
@@ -634,7 +635,7 @@ __device__ void ms_pull(const MsArgs<OffT> &a, const MsState &st, MsPullSmem &w,
             open = __any_sync(GRX_FULL_MASK, open);
             if (lane == 0 && !open) a.sat[ch] = 1;
         }
-        ch = nwarps + __shfl_sync(GRX_FULL_MASK, nn, 0);
+        ch = more ? nwarps + __shfl_sync(GRX_FULL_MASK, nn, 0) : nch;
     }
 }
 
