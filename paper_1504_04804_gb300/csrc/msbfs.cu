@@ -105,6 +105,7 @@ struct MsState {
     uint8_t flush;      // this pull level starts with a flush (slots full)
     uint8_t bmp;        // push level that marks touched vertices in a bitmap
     uint8_t keep;       // push level whose new lanes go to a history slot
+    uint8_t flushed;    // a flush came before
     int32_t slot_depth[MS_HSLOTS];
     uint32_t q, T;      // |Q_L| and its edge count
     unsigned long long seen_pairs;    // (vertex, lane) pairs labelled so far
@@ -182,6 +183,7 @@ __device__ MsState ms_next_state(const MsArgs<OffT> &a, const MsState &st, bool 
     ns.q = (uint32_t)(pk >> 32);
     ns.T = (uint32_t)pk;
     ns.qin = st.dir == DIR_PUSH;
+    ns.flushed |= st.flush;
     if (st.dir == DIR_PULL || st.keep) {
         const int h = st.flush ? 0 : st.hslots;
         ns.slot_depth[h] = st.L + 1;
@@ -743,10 +745,15 @@ __device__ __forceinline__ void ms_flush_slots(const MsArgs<OffT> &a, int nslots
     }
 }
 
+// Four vertices a thread where nearly every word of four is written whole (the only
+// flush of a traversal) and every thread has some; words written in part cost four
+// times the stores.
 template <typename OffT>
-__device__ void ms_flush(const MsArgs<OffT> &a, int nslots, const int32_t *slot_depth, bool final) {
-    const bool wide = (a.nv & 3) == 0 && ((uintptr_t)a.depth & 15) == 0;
-    if (!wide) ms_flush_slots<OffT, MS_HSLOTS, 1>(a, nslots, slot_depth, final);
+__device__ void ms_flush(const MsArgs<OffT> &a, int nslots, const int32_t *slot_depth, bool final, bool flushed) {
+    const bool wide = final && !flushed && (a.nv & 3) == 0 && ((uintptr_t)a.depth & 15) == 0 &&
+                      a.nv / 4 >= (int32_t)(gridDim.x * blockDim.x);
+    if (!wide && nslots <= 3) ms_flush_slots<OffT, 3, 1>(a, nslots, slot_depth, final);
+    else if (!wide) ms_flush_slots<OffT, MS_HSLOTS, 1>(a, nslots, slot_depth, final);
     else if (nslots <= 3) ms_flush_slots<OffT, 3, 4>(a, nslots, slot_depth, final);
     else if (nslots <= 4) ms_flush_slots<OffT, 4, 4>(a, nslots, slot_depth, final);
     else ms_flush_slots<OffT, MS_HSLOTS, 4>(a, nslots, slot_depth, final);
@@ -815,7 +822,7 @@ __global__ void __launch_bounds__(MS_BLOCK, MS_MIN_BLOCKS) k_msbfs_persistent(Ms
         } else if (op == MOP_FINAL) {
             ms_push_finalize<OffT>(a, st, sm.w[threadIdx.x >> 5].list);
         } else if (op == MOP_FLUSH) {
-            ms_flush<OffT>(a, MS_HSLOTS, st.slot_depth, false);
+            ms_flush<OffT>(a, MS_HSLOTS, st.slot_depth, false, st.flushed);
         } else {
             MsCounts c = {0ull, 0ull, 0ull, 0ull, 0ull};
             if (op == MOP_PULL) ms_pull<OffT, STATS>(a, st, sm.p[threadIdx.x >> 5], c);
@@ -842,7 +849,7 @@ __global__ void __launch_bounds__(MS_BLOCK, MS_MIN_BLOCKS) k_msbfs_persistent(Ms
         __syncthreads();
     }
     // depths of the pull levels still in the history slots, -1 for the rest
-    ms_flush<OffT>(a, s_st.hslots, s_st.slot_depth, true);
+    ms_flush<OffT>(a, s_st.hslots, s_st.slot_depth, true, s_st.flushed);
     __syncthreads();
     if (threadIdx.x == 0) {
         __threadfence();
