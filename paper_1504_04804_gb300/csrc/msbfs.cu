@@ -517,6 +517,9 @@ __device__ void ms_pull(const MsArgs<OffT> &a, const MsState &st, MsPullSmem &w,
     const int64_t nch = (a.n_active + R - 1) / R;
     const int64_t nwarps = (int64_t)gridDim.x * MS_WARPS;
     const bool more = nch > nwarps;              // else a thousand atomics on one word, for nothing
+    // the active row j of chunk ch: neighbours, or on small graphs spread over the whole
+    // range (R-MAT's longest rows are neighbours, and a warp would have them all)
+    auto row_of = [&](int64_t ch, int64_t j) { return small ? j * nch + ch : ch * R + j; };
     for (int64_t ch = grx_warp(); ch < nch;) {
         unsigned int nn = 0;
         if (lane == 0 && more) nn = atomicAdd(wq, 1u);
@@ -527,7 +530,7 @@ __device__ void ms_pull(const MsArgs<OffT> &a, const MsState &st, MsPullSmem &w,
             int2 f2[PER];
 #pragma unroll
             for (int k = 0; k < PER; ++k) {
-                const int64_t i = ch * R + k * 32 + lane;
+                const int64_t i = row_of(ch, k * 32 + lane);
                 v[k] = -1;
                 s[k] = deg[k] = 0u;
                 if (k * 32 + (int)lane < R && i < a.n_active) {
@@ -547,7 +550,10 @@ __device__ void ms_pull(const MsArgs<OffT> &a, const MsState &st, MsPullSmem &w,
                 acc[k] |= f2[k].y >= 0 ? __ldca(cin + f2[k].y) : 0ull;
                 if (STATS) c.gathered += (f2[k].x >= 0 ? 1 : 0) + (f2[k].y >= 0 ? 1 : 0);
             }
-            if (STATS && lane == 0) c.rows += (unsigned long long)min((int64_t)R, a.n_active - ch * R);
+            if (STATS) {
+#pragma unroll
+                for (int k = 0; k < PER; ++k) c.rows += v[k] >= 0 ? 1ull : 0ull;
+            }
             bool open = false;
             int nh = 0;
 #pragma unroll
@@ -559,7 +565,7 @@ __device__ void ms_pull(const MsArgs<OffT> &a, const MsState &st, MsPullSmem &w,
                     const int h = nh + __popc(m & lanemask_lt());
                     w.s[h] = s[k];
                     w.deg[h] = deg[k];
-                    w.i[h] = (int32_t)(ch * R + k * 32 + lane);
+                    w.i[h] = (int32_t)row_of(ch, k * 32 + lane);
                     w.v[h] = v[k];
                     w.miss[h] = miss[k];
                     w.acc[h] = acc[k];
