@@ -18,7 +18,8 @@
 //  * Pull level (dense frontier): warps take the non-isolated vertices 128 at a
 //    time and gather cur[u] over a row only until every lane the row misses is
 //    found (edge skipping, for all lanes at once): its first two neighbours
-//    (first2), a lane per row; then eight lanes per row, 32 edges a step.  Rows
+//    (first2), a lane per row, and its first ten on graphs of few edges a
+//    vertex; then eight lanes per row, 32 edges a step.  Rows
 //    still open after MS_HEAD edges leave the rest to a second phase, in pieces
 //    of 1,024 edges over the grid, and are finished by a third.
 //  * Depths found by pull levels and large push levels are not written per level:
@@ -51,6 +52,11 @@ constexpr int MS_ROWS = 128;                        // pull: rows a warp takes a
 // 24 / 22 / 20: 30 7.58 / 2.27 / 0.82 ms, 126 7.02 / 2.16 / 0.89, 254 7.12 / 2.30 /
 // 0.98, 510 7.37 / 2.57 / 1.16).
 constexpr uint32_t MS_HEAD = 126;
+// Pull, fewer than eight edges a vertex: edges of a row that a lane takes, its rows'
+// loads in flight together.  Eight lanes a row have little to do there (uniform random,
+// 2M vertices of degree 4, 64 sources: a level that reads every edge 154 us, by edge
+// tiles 101, so 63; the traversal 2,044 -> 1,529 us).
+constexpr uint32_t MS_LANE_HEAD = 10;
 constexpr uint32_t MS_WARP_ROW = 2048;              // pull, small graphs: rows up to this stay in the first phase
 constexpr uint32_t MS_PIECE = 1024;                 // pull: edges of a piece of the second phase
 constexpr int MS_HSLOTS = 6;                        // history slots of pull levels
@@ -79,6 +85,7 @@ struct MsArgs {
     unsigned long long *hist[MS_HSLOTS];
     int2 *rest;                       // pieces of open rows: (active row, piece)
     int rows;                         // pull: rows a warp takes at a time
+    int few;                          // pull: few edges a vertex
     uint8_t *sat;                     // per `rows` rows: every one has all lanes seen
     int32_t *Q[3];
     uint32_t *E[3];
@@ -517,6 +524,7 @@ __device__ void ms_pull(const MsArgs<OffT> &a, const MsState &st, MsPullSmem &w,
     const int64_t nch = (a.n_active + R - 1) / R;
     const int64_t nwarps = (int64_t)gridDim.x * MS_WARPS;
     const bool more = nch > nwarps;              // else a thousand atomics on one word, for nothing
+    const uint32_t lane_head = a.few ? MS_LANE_HEAD : 2;
     // the active row j of chunk ch: neighbours, or on small graphs spread over the whole
     // range (R-MAT's longest rows are neighbours, and a warp would have them all)
     auto row_of = [&](int64_t ch, int64_t j) { return small ? j * nch + ch : ch * R + j; };
@@ -554,12 +562,33 @@ __device__ void ms_pull(const MsArgs<OffT> &a, const MsState &st, MsPullSmem &w,
 #pragma unroll
                 for (int k = 0; k < PER; ++k) c.rows += v[k] >= 0 ? 1ull : 0ull;
             }
+            if (a.few) {                             // short rows: a lane takes a row's first ten edges
+#pragma unroll 1
+                for (uint32_t at = 2; at < MS_LANE_HEAD; at += 4) {
+#pragma unroll
+                    for (int k0 = 0; k0 < PER; k0 += 2) {
+                        int32_t u[2][4];
+#pragma unroll
+                        for (int k = k0; k < k0 + 2; ++k)
+#pragma unroll
+                            for (int j = 0; j < 4; ++j)
+                                u[k - k0][j] = at + j < deg[k] && (miss[k] & ~acc[k]) ? __ldg(a.col + (int64_t)s[k] + at + j) : -1;
+#pragma unroll
+                        for (int k = k0; k < k0 + 2; ++k)
+#pragma unroll
+                            for (int j = 0; j < 4; ++j) {
+                                if (u[k - k0][j] >= 0) acc[k] |= __ldca(cin + u[k - k0][j]);
+                                if (STATS) c.gathered += u[k - k0][j] >= 0 ? 1ull : 0ull;
+                            }
+                    }
+                }
+            }
             bool open = false;
             int nh = 0;
 #pragma unroll
             for (int k = 0; k < PER; ++k) {
                 acc[k] &= miss[k];
-                const bool more = (miss[k] & ~acc[k]) != 0ull && deg[k] > 2;
+                const bool more = (miss[k] & ~acc[k]) != 0ull && deg[k] > lane_head;
                 const unsigned int m = __ballot_sync(GRX_FULL_MASK, more);
                 if (more) {
                     const int h = nh + __popc(m & lanemask_lt());
@@ -586,7 +615,7 @@ __device__ void ms_pull(const MsArgs<OffT> &a, const MsState &st, MsPullSmem &w,
                 const int64_t e0 = w.s[h];
                 const unsigned long long ms = w.miss[h];
                 unsigned long long ac = w.acc[h];
-                for (uint32_t at = 2; at < end && (ms & ~ac); at += 32) {
+                for (uint32_t at = lane_head; at < end && (ms & ~ac); at += 32) {
                     int32_t u[4];
                     unsigned long long g[4];
 #pragma unroll
@@ -945,6 +974,7 @@ grx_status ms_launch_typed(grx_graph *g, const int32_t *srcs, int n, int32_t *de
     if (max_grid > GRX_MAX_GRID) max_grid = GRX_MAX_GRID;
     const int blocks = grx_grid(o, MS_BLOCK, max_grid);
     a.rows = ms_rows(g, blocks);
+    a.few = g->ne < 8 * g->n_active;
     GRX_CUDA(cudaMemsetAsync(g->bar_flags, 0, sizeof(unsigned int) * (size_t)blocks, s));
     GRX_CUDA(cudaMemsetAsync(&g->ctl->bar_release, 0, sizeof(unsigned int), s));
     if (o->collect_stats) GRX_CUDA(cudaMemsetAsync(g->stats, 0, sizeof(DevStats), s));
