@@ -134,7 +134,7 @@ struct grx_graph {
     unsigned long long *ms_hist[6];  // multi-source BFS: pull levels' new lanes, [nv] each
     int2 *ms_rest;                   // multi-source BFS: pieces of rows a pull level leaves open
     uint32_t *ms_tbits;              // multi-source BFS: touched bitmap of bitmap push levels
-    uint8_t *ms_sat;                 // multi-source BFS: per 128 rows, all lanes seen
+    uint8_t *ms_sat;                 // multi-source BFS: per ms_rows() rows, all lanes seen
     uint32_t *ms_dist;               // batched SSSP, vertex-major [nv][64]
     int ms_ready;
     // betweenness centrality (allocated on first use)
@@ -145,13 +145,14 @@ struct grx_graph {
     unsigned long long *bcm_hist;    // [GRX_BCM_MAX_LEVELS][nv] lanes at each depth
     double *bcm_sig, *bcm_acc;       // [nv][64]
     int32_t *bcm_srcs;               // [64] device copy of the sources
-    // CUDA-graph level loop of bfs (GRX_LOOP_GRAPH), per parent flag
+    // optional buffers (grx_alloc_optional), like the sorted PageRank rows
     void *ss_lines;                  // list rounds of sssp: lines, pieces, vertices (first use)
     uint32_t ss_list_T;              // ... edges of a round per block
     int ss_list_blocks;              // ... blocks they are laid out for
     struct NarrowBuffers *narrow;    // narrow levels of bfs (narrow.cuh), first use
     int fixed_scratch;               // bfs_noalloc's view: nothing may be allocated
     int keep_optional;               // optional buffers are part of a captured graph
+    // CUDA-graph level loop of bfs (GRX_LOOP_GRAPH), per parent flag
     cudaGraphExec_t bfs_gexec[2];
     void *bfs_gargs;                 // device copy of the call's arguments
     // 64-bit vertex ids (graph_load_csr64): columns, frontier queues and
