@@ -254,8 +254,6 @@ grx_status grx_cc_launch(grx_graph *g, int32_t *label, const grx_opts *o, cudaSt
     a.stats = g->stats;
     a.bar_flags = g->bar_flags;
     a.timeout_ns = grx_timeout_ns(o);
-    // paths, meshes, uniform random graphs: no vertex joined to a good part of the graph
-    if (g->nv > 1 << 17 && (g->max_deg <= 64 || g->max_deg <= (uint32_t)g->nv >> 10))
-        return cc_launch<1, 256>(g, a, o, s);
+    if (g->nv > 1 << 17 && !grx_has_hubs(g)) return cc_launch<1, 256>(g, a, o, s);
     return g->ne >= 8ll * g->nv ? cc_launch<2, 1024>(g, a, o, s) : cc_launch<1, 1024>(g, a, o, s);
 }

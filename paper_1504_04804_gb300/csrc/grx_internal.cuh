@@ -168,6 +168,12 @@ struct grx_graph {
     int nallocs;
 };
 
+// Whether some vertex is joined to a good part of the graph, as on R-MAT and social
+// graphs, unlike paths, meshes and uniform random graphs.
+inline bool grx_has_hubs(const grx_graph *g) {
+    return g->max_deg > 64 && g->max_deg > (uint32_t)g->nv >> 10;
+}
+
 // Whether s is being captured (or may not be asked): no time to allocate what a
 // call can do without.
 bool grx_capturing(cudaStream_t s);

@@ -70,6 +70,7 @@ struct SsspArgs {
     uint32_t bmp_min_T;
     unsigned long long timeout_ns;
     int32_t src;
+    int even;                                // no hubs: a round's tiles in equal shares
     // list rounds (lines NULL: none), per block: pieces by round parity, vertices
     NarrowWord *lines, *pieces;
     int32_t *verts;
@@ -149,8 +150,11 @@ __device__ void relax_round(const SsspArgs<OffT> &a, const SsState &st, SsWarpSm
     // Batches of up to SS_BATCH tiles: the first by the warp's number, the others
     // from the round's counter.  What a tile costs varies along the queue (R-MAT 22,
     // mean of three sources: one equal share a warp 1,824 us, batches of 16 / 8 / 4 / 2
-    // tiles 1,618 / 1,577 / 1,569 / 1,744; a batch costs a search).
-    const uint64_t batch = min((uint64_t)SS_BATCH, (ntiles + nwarps - 1) / nwarps);
+    // tiles 1,618 / 1,577 / 1,569 / 1,744; a batch costs a search).  Without hubs it
+    // does not, and equal shares are the better form (uniform random, 2M vertices of
+    // degree 16: 1,536 us, batches 1,597; in bands of 100 1,430 and 1,518).
+    const uint64_t share = (ntiles + nwarps - 1) / nwarps;
+    const uint64_t batch = a.even ? share : min((uint64_t)SS_BATCH, share);
     if (batch == 0) return;
     const uint64_t nbatch = (ntiles + batch - 1) / batch;
     unsigned int *wq = &a.ctl->wq[L & 3];
@@ -854,6 +858,7 @@ grx_status launch_typed(grx_graph *g, int32_t src, uint32_t *dist, const grx_opt
     a.stats = g->stats;
     a.timeout_ns = grx_timeout_ns(o);
     a.src = src;
+    a.even = !grx_has_hubs(g);
     a.lines = a.pieces = nullptr;
     a.verts = nullptr;
     a.list_T = a.group = a.list_rounds = 0;

@@ -149,6 +149,20 @@ def test_large_rounds_run_on_the_whole_grid(grx, nv, ne, full):
         dg.free()
 
 
+@pytest.mark.parametrize("off64", [False, True])
+def test_rounds_in_equal_shares(grx, off64):
+    """No hubs and many edges: rounds of a million edges and more, several tiles a warp, the last share cut short."""
+    g = _weighted(*_uniform(90_000, 2_900_000, 9), wmax=40, seed=3)
+    assert np.diff(g.row_offsets).max() <= 87 and g.ne >= 8 * g.nv
+    dg = grx.load(g, offsets64=off64)
+    want = oracle.sssp(g.row_offsets, g.col_indices, g.weights, 5)
+    for delta in (0, 10):
+        for kw in ({}, {"grid_blocks": 3}, {"push_bitmap": -1.0}):
+            d = grx.sssp(dg, 5, opts=grx.opts(sssp_delta=delta, **kw))
+            grx.graph_status(dg)
+            assert np.array_equal(grx.as_uint32(d), want), (delta, kw)
+
+
 def test_narrow_levels_run_where_bfs_has_many_small_ones(grx):
     """The counterpart for BFS (its results are tested with its limits elsewhere): the group's lines are used."""
     g = inputs.grid_graph(301, 97, p_del=0.1, seed=5)
