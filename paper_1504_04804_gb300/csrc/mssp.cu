@@ -217,10 +217,9 @@ __device__ void mp_expand(const MpArgs<OffT> &a, int L, uint32_t q, uint64_t T, 
     if (batch == 0) return;
     const uint64_t nbatch = (ntiles + batch - 1) / batch;
     unsigned int *wq = &a.ctl->wq[L & 3];
-    const bool more = nbatch > nwarps;           // else a thousand atomics on one word, for nothing
     for (uint64_t bt = gw; bt < nbatch;) {
         unsigned int nn = 0;
-        if (lane == 0 && more) nn = atomicAdd(wq, 1u);
+        if (lane == 0) nn = atomicAdd(wq, 1u);
         const uint64_t tb0 = bt * batch, tb1 = min(ntiles, tb0 + batch);
         int64_t i0 = warp_upper_index_cg(Qe, (int64_t)q, (uint32_t)(tb0 * MP_WTILE));
         for (uint64_t tile = tb0; tile < tb1; ++tile) {
@@ -278,7 +277,7 @@ __device__ void mp_expand(const MpArgs<OffT> &a, int L, uint32_t q, uint64_t T, 
             i0 = (next_start == e1) ? i0 + n : i0 + n - 1;
             __syncwarp();
         }
-        bt = more ? nwarps + __shfl_sync(GRX_FULL_MASK, nn, 0) : nbatch;
+        bt = nwarps + __shfl_sync(GRX_FULL_MASK, nn, 0);
     }
 }
 

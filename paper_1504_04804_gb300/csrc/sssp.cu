@@ -146,7 +146,6 @@ __device__ void relax_round(const SsspArgs<OffT> &a, const SsState &st, SsWarpSm
     const uint64_t T = st.T;
     const uint64_t ntiles = (T + SS_WTILE - 1) / SS_WTILE;
     const uint64_t nwarps = (uint64_t)gridDim.x * SS_WARPS;
-    const uint64_t gw = grx_warp();
     // Batches of up to SS_BATCH tiles: the first by the warp's number, the others
     // from the round's counter.  What a tile costs varies along the queue (R-MAT 22,
     // mean of three sources: one equal share a warp 1,824 us, batches of 16 / 8 / 4 / 2
@@ -158,10 +157,10 @@ __device__ void relax_round(const SsspArgs<OffT> &a, const SsState &st, SsWarpSm
     if (batch == 0) return;
     const uint64_t nbatch = (ntiles + batch - 1) / batch;
     unsigned int *wq = &a.ctl->wq[L & 3];
-    const bool more = nbatch > nwarps;           // else a thousand atomics on one word, for nothing
+    const uint64_t gw = grx_warp();
     for (uint64_t bt = gw; bt < nbatch;) {
         unsigned int nn = 0;
-        if (lane == 0 && more) nn = atomicAdd(wq, 1u);
+        if (lane == 0) nn = atomicAdd(wq, 1u);
         const uint64_t tb0 = bt * batch, tb1 = min(ntiles, tb0 + batch);
         int64_t i0 = warp_upper_index_cg(Qe, q, (uint32_t)(tb0 * SS_WTILE));
         for (uint64_t tile = tb0; tile < tb1; ++tile) {
@@ -260,7 +259,7 @@ __device__ void relax_round(const SsspArgs<OffT> &a, const SsState &st, SsWarpSm
             i0 = (next_start == e1) ? i0 + n : i0 + n - 1;
             __syncwarp();
         }
-        bt = more ? nwarps + __shfl_sync(GRX_FULL_MASK, nn, 0) : nbatch;
+        bt = nwarps + __shfl_sync(GRX_FULL_MASK, nn, 0);
     }
 }
 
