@@ -27,6 +27,7 @@ __global__ void k_block_popcounts(const uint32_t *bits, int64_t words, uint32_t 
         uint32_t t = 0;
         for (int i = 0; i < ACT_BLOCK / 32; ++i) t += ws[i];
         bsum[blockIdx.x] = t;
+        if (blockIdx.x == 0) bsum[gridDim.x] = bits[words];   // the largest degree, behind the bitmap
     }
 }
 
@@ -109,17 +110,18 @@ grx_status grx_edge_tiles(grx_graph *g, int tile, cudaStream_t s, const int2 **o
 
 grx_status grx_build_active(grx_graph *g, cudaStream_t s) {
     const int64_t nblocks = (g->words + ACT_WORDS_PER_BLOCK - 1) / ACT_WORDS_PER_BLOCK;
-    uint32_t *bsum = (uint32_t *)grx_ctx_alloc(g->ctx, (size_t)nblocks * 4, s);
+    const size_t bsum_bytes = (size_t)(nblocks + 1) * 4;
+    uint32_t *bsum = (uint32_t *)grx_ctx_alloc(g->ctx, bsum_bytes, s);
     if (!bsum) return grx_fail(GRX_ENOMEM, "active list: allocation failed");
     k_block_popcounts<<<(unsigned)nblocks, ACT_BLOCK, 0, s>>>(g->nz_bits, g->words, bsum);
-    std::vector<uint32_t> h((size_t)nblocks);
-    cudaError_t e = cudaMemcpyAsync(h.data(), bsum, (size_t)nblocks * 4, cudaMemcpyDeviceToHost, s);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(&g->max_deg, g->nz_bits + g->words, 4, cudaMemcpyDeviceToHost, s);
+    std::vector<uint32_t> h((size_t)nblocks + 1);
+    cudaError_t e = cudaMemcpyAsync(h.data(), bsum, bsum_bytes, cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     if (e != cudaSuccess) {
-        grx_ctx_free(g->ctx, bsum, (size_t)nblocks * 4, s);
+        grx_ctx_free(g->ctx, bsum, bsum_bytes, s);
         return grx_cuda_fail(e, "active list: block counts");
     }
+    g->max_deg = h[(size_t)nblocks];
     uint64_t total = 0;
     for (int64_t i = 0; i < nblocks; ++i) {
         uint32_t c = h[(size_t)i];
@@ -130,12 +132,12 @@ grx_status grx_build_active(grx_graph *g, cudaStream_t s) {
     g->active = (int32_t *)grx_alloc(g, (size_t)total * 4 + 16, s);
     g->aoff = (uint32_t *)grx_alloc(g, (size_t)(total + 1) * 4 + 16, s);
     if (!g->active || !g->aoff) {
-        grx_ctx_free(g->ctx, bsum, (size_t)nblocks * 4, s);
+        grx_ctx_free(g->ctx, bsum, bsum_bytes, s);
         return grx_fail(GRX_ENOMEM, "active list: allocation failed");
     }
     e = cudaMemcpyAsync(bsum, h.data(), (size_t)nblocks * 4, cudaMemcpyHostToDevice, s);
     if (e != cudaSuccess) {
-        grx_ctx_free(g->ctx, bsum, (size_t)nblocks * 4, s);
+        grx_ctx_free(g->ctx, bsum, bsum_bytes, s);
         return grx_cuda_fail(e, "active list: prefix upload");
     }
     if (g->off64)
@@ -147,7 +149,7 @@ grx_status grx_build_active(grx_graph *g, cudaStream_t s) {
     uint32_t ne32 = (uint32_t)g->ne;
     e = cudaMemcpyAsync(g->aoff + total, &ne32, 4, cudaMemcpyHostToDevice, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);   // ne32 and h are stack/heap locals
-    grx_ctx_free(g->ctx, bsum, (size_t)nblocks * 4, s);
+    grx_ctx_free(g->ctx, bsum, bsum_bytes, s);
     if (e != cudaSuccess) return grx_cuda_fail(e, "active list: fill");
     return GRX_OK;
 }
